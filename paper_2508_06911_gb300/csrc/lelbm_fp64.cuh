@@ -1,0 +1,530 @@
+// The FP64 EPR (Eq. IID7-IID11) and moment streaming (Eq. IIE3) in lattice form, for 1D and 2D
+// cells with a row table.  GB300 issues one FP64 warp instruction per SM every 16 cycles, in which
+// its four schedulers issue up to 64 FP32 or integer ones: the number of FP64 operations per cell
+// is the time of the FP64 path, and everything else here is arranged around that count.
+//   - The velocity set is swept from the lattice point nearest to u outwards, row by row, and
+//     along a row outwards from its centre.  On the lattice the exponent is a polynomial in
+//     integer offsets (k, j), so populations follow from multiplicative forward differences in
+//     both directions: a row costs about a dozen products where seven exponentials stood, and the
+//     error growth (~n^3/6 ulp over n steps) starts at the centre.
+//   - The children of split points are a lattice of spacing 1/2 of their own, swept the same way.
+//   - A Newton pass sums only the residual's moments (degree <= 3 and <= 2) in FP64, as power sums
+//     of the integer offsets (exact weights, made by integer operations) moved to thermal units
+//     once per pass.  The Jacobian and the solve of an update are FP32, from the same populations:
+//     an update only steers the iteration, whose FP64 residual is judged against the tolerance as
+//     before, and an update with a Jacobian to 2^-24 leaves about 1e-5 of the residual, far below
+//     what the quadratic step itself leaves until the residual is at rounding.
+//   - The membership decisions come from the row table, taken once per cell.
+// A solve that breaks down here is redone by the all-FP64 Newton (solve_fg), so what converges and
+// what falls back is decided there.
+#pragma once
+
+#include <cstdint>
+
+#include "lelbm_df.cuh"
+
+namespace lbm {
+
+// FP64 -> FP32 by truncation with integer operations (the conversion instruction runs on the
+// FP64 pipe).  Positive normal values; below 2^-126 zero, from 2^128 on (and NaN) infinity.
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const float f = __uint_as_float(__funnelshift_l(lo, hi - 0x38000000u, 3));
+    return hi < 0x38100000u ? 0.f : (hi >= 0x47f00000u ? __int_as_float(0x7f800000) : f);
+}
+
+// Coefficients d[ix(a, b)] of k^a j^b in the exponent 1 + sum_j lam_j T_j at the thermal points
+// (x0 + k h, y0 + j h).
+template <int D, bool FLUON>
+__device__ __forceinline__ void lattice_poly(const double* lam, double x0, double y0, double h, double* d) {
+    using Q = DFPop<D, FLUON>;
+    constexpr int P = Q::P;
+#pragma unroll
+    for (int j = 0; j < Q::N; j++) d[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))] = lam[j];
+    d[0] += 1.0;
+#pragma unroll
+    for (int b = 0; b <= (D == 2 ? P : 0); b++) {
+        const int n = P - b;
+#pragma unroll
+        for (int k = 0; k < P; k++)
+#pragma unroll
+            for (int i = P - 1; i >= 0; i--)
+                if (k < n && i >= k && i < n) d[Q::ix(i, b)] = fma(x0, d[Q::ix(i + 1, b)], d[Q::ix(i, b)]);
+    }
+    if constexpr (D == 2) {
+#pragma unroll
+        for (int a = 0; a <= P; a++) {
+            const int n = P - a;
+#pragma unroll
+            for (int k = 0; k < P; k++)
+#pragma unroll
+                for (int i = P - 1; i >= 0; i--)
+                    if (k < n && i >= k && i < n) d[Q::ix(a, i)] = fma(y0, d[Q::ix(a, i + 1)], d[Q::ix(a, i)]);
+        }
+    }
+    double hp[P + 1];
+    hp[0] = 1.0;
+#pragma unroll
+    for (int k = 1; k <= P; k++) hp[k] = hp[k - 1] * h;
+#pragma unroll
+    for (int b = 0; b <= (D == 2 ? P : 0); b++)
+#pragma unroll
+        for (int a = 0; a + b <= P; a++)
+            if (a + b > 0) d[Q::ix(a, b)] *= hp[a + b];
+}
+
+// Ratios of neighbouring populations at an anchor, from the exponent polynomial p (lattice_poly).
+// Second and third ratios compound over a sweep, so they are exponentials of their own where a long
+// row needs it (along x) and products of at most two factors elsewhere.
+template <int D, bool FLUON>
+struct SweepFactors {
+    double e0, r, l, r2, r3, l3;            // population, ratios to k = +1 and -1, second and third ratios
+    double u, ud, u2, u2d, u3, u3d;         // ratios of e0 to the rows j = +1 and -1, second, third
+    double m11, i11, m12, i12, m21, i21;    // exp(-+p_11), exp(-+p_12), exp(-+p_21)
+
+    __device__ __forceinline__ void init(const double* p, double wgt) {
+        using Q = DFPop<D, FLUON>;
+        const double p10 = p[Q::ix(1, 0)], p20 = p[Q::ix(2, 0)];
+        const double p30 = FLUON ? p[FLUON ? Q::ix(3, 0) : 0] : 0.0;
+        e0 = wgt * exp(-p[0]);
+        r = exp(-(p10 + p20 + p30));
+        l = exp(p10 - p20 + p30);
+        r2 = exp(-(2.0 * p20 + 6.0 * p30));
+        if constexpr (FLUON) {
+            r3 = exp(-6.0 * p30);
+            l3 = 1.0 / r3;
+        }
+        if constexpr (D == 2) {
+            const double p01 = p[Q::ix(0, 1)], p02 = p[Q::ix(0, 2)];
+            const double p03 = FLUON ? p[FLUON ? Q::ix(0, 3) : 0] : 0.0;
+            u = exp(-(p01 + p02 + p03));
+            ud = exp(p01 - p02 + p03);
+            u2 = exp(-(2.0 * p02 + 6.0 * p03));
+            m11 = exp(-p[Q::ix(1, 1)]);
+            i11 = 1.0 / m11;
+            if constexpr (FLUON) {
+                u3 = exp(-6.0 * p03);
+                u3d = 1.0 / u3;
+                u2d = u2 * (u3d * u3d);
+                m12 = exp(-p[Q::ix(1, 2)]);
+                i12 = 1.0 / m12;
+                m21 = exp(-p[Q::ix(2, 1)]);
+                i21 = 1.0 / m21;
+            }
+        }
+    }
+};
+
+// The row state of one population and its advance to the next row (up or down).
+template <int D, bool FLUON>
+struct SweepRows {
+    double E, R, L, R2;            // at k = 0 of the row: population, ratios to the right and left, second ratio
+    double U, U2, U3, V, VL, W, V2, V2L;
+
+    __device__ __forceinline__ void start(const SweepFactors<D, FLUON>& f, bool down) {
+        E = f.e0;
+        R = f.r;
+        L = f.l;
+        R2 = f.r2;
+        if constexpr (D == 2) {
+            U = down ? f.ud : f.u;
+            U2 = FLUON && down ? f.u2d : f.u2;
+            V = down ? f.i11 : f.m11;
+            VL = down ? f.m11 : f.i11;
+            if constexpr (FLUON) {
+                const double a21 = down ? f.i21 : f.m21;
+                U3 = down ? f.u3d : f.u3;
+                V *= f.m12 * a21;
+                VL *= f.i12 * a21;
+                V2 = f.m12 * f.m12;
+                V2L = f.i12 * f.i12;
+                W = a21 * a21;
+            }
+        }
+    }
+    __device__ __forceinline__ void advance() {
+        if constexpr (D == 2) {
+            E *= U;
+            U *= U2;
+            R *= V;
+            L *= VL;
+            if constexpr (FLUON) {
+                U2 *= U3;
+                V *= V2;
+                VL *= V2L;
+                R2 *= W;
+            }
+        }
+    }
+};
+
+// Rows that one anchor serves on each side: a new anchor every 2 kAnchorRows + 1 rows bounds the
+// compounded rounding of tall sets; up to R_ac = 7 (RT = 3.5 at n = 4) one anchor serves all.
+constexpr int kAnchorRows = 8;
+
+// Visits the lattice points (x0 + k h, y0 + j h) of rows jlo..jhi: ext(j, i0, i1, h0, h1) gives a
+// row's points i0..i1 without the hole h0..h1 (empty: h0 = 1, h1 = 0); point(k, j, f, g) gets every
+// point with its populations (weights wf, wg included), row_end(j) follows a row that is not empty.
+template <int D, class Ext, class Pt, class RowEnd>
+__device__ __forceinline__ void lattice_sweep(const double* lf, const double* lg, bool doF, bool doG, double x0,
+                                              double y0, double h, double wf, double wg, int jlo, int jhi,
+                                              const Ext& ext, Pt& point, RowEnd& row_end) {
+    int ja = 0;
+    while (ja - kAnchorRows > jlo) ja -= 2 * kAnchorRows + 1;
+#pragma unroll 1
+    for (; ja - kAnchorRows <= jhi; ja += 2 * kAnchorRows + 1) {
+        SweepFactors<D, true> ff;
+        SweepFactors<D, false> fg;
+        if (doF) {
+            double p[DFPop<D, true>::NB];
+            lattice_poly<D, true>(lf, x0, fma(widen((float)ja), h, y0), h, p);
+            ff.init(p, wf);
+        }
+        if (doG) {
+            double p[DFPop<D, false>::NB];
+            lattice_poly<D, false>(lg, x0, fma(widen((float)ja), h, y0), h, p);
+            fg.init(p, wg);
+        }
+        const double l3sq = doF ? ff.l3 * ff.l3 : 0.0;
+#pragma unroll 1
+        for (int down = 0; down < (D == 2 ? 2 : 1); down++) {
+            SweepRows<D, true> sf;
+            SweepRows<D, false> sg;
+            if (doF) sf.start(ff, down);
+            if (doG) sg.start(fg, down);
+            const int step = down ? -1 : 1;
+            const int j_end = down ? max(jlo, ja - kAnchorRows) : min(jhi, ja + kAnchorRows);
+#pragma unroll 1
+            for (int j = ja; step * (j_end - j) >= 0; j += step) {
+                int i0 = 0, i1 = -1, h0, h1;
+                if (j >= jlo && j <= jhi && !(down && j == ja)) ext(j, i0, i1, h0, h1);
+                if (i0 <= i1) {
+#pragma unroll 1
+                    for (int left = 0; left < 2; left++) {
+                        double e = 0.0, r = 0.0, r2 = 0.0, r3 = 0.0, eg = 0.0, rg = 0.0;
+                        if (doF) {
+                            e = sf.E;
+                            r = left ? sf.L : sf.R;
+                            r2 = left ? sf.R2 * l3sq : sf.R2;
+                            r3 = left ? ff.l3 : ff.r3;
+                        }
+                        if (doG) {
+                            eg = sg.E;
+                            rg = left ? sg.L : sg.R;
+                        }
+                        const int n = left ? -i0 : i1;
+#pragma unroll 1
+                        for (int i = 0; i <= n; i++) {
+                            const int k = left ? -i : i;
+                            if (!(left && i == 0) && k >= i0 && k <= i1 && (k < h0 || k > h1)) point(k, j, e, eg);
+                            if (doF) {
+                                e *= r;
+                                r *= r2;
+                                r2 *= r3;
+                            }
+                            if (doG) {
+                                eg *= rg;
+                                rg *= fg.r2;
+                            }
+                        }
+                    }
+                    row_end(j);
+                }
+                if (doF) sf.advance();
+                if (doG) sg.advance();
+            }
+        }
+    }
+}
+
+// The one or two lattices of a cell's velocity set: lattice 0 holds the level-0 points (spacing 1,
+// anchored at the integer velocity nearest to u), lattice 1 the children of split points (spacing
+// 1/2, anchored a quarter cell below it).
+template <int D>
+struct CellLattice {
+    int xn, yn;      // anchor of lattice 0
+    int n;           // lattices in use
+    double fx, fy;   // u - (xn, yn)
+
+    __device__ __forceinline__ void init(const CellState<D>& c, const RowTable<D>& tab) {
+        fx = c.u[0] - (double)tab.xc;
+        xn = tab.xc + (fx > 0.5 ? 1 : 0);
+        fx = c.u[0] - (double)xn;
+        fy = 0.0;
+        yn = 0;
+        if constexpr (D == 2) {
+            fy = c.u[1] - (double)tab.yc;
+            yn = tab.yc + (fy > 0.5 ? 1 : 0);
+            fy = c.u[1] - (double)yn;
+        }
+        n = (D == 2 ? tab.band_n > 0 : tab.a <= tab.b) ? 2 : 1;
+    }
+    // rows of lattice `child`
+    __device__ __forceinline__ void rows(const RowTable<D>& tab, bool child, int& jlo, int& jhi) const {
+        jlo = jhi = 0;
+        if constexpr (D == 2) {
+            jlo = tab.y_first - yn;
+            jhi = jlo + tab.nrows - 1;
+            if (child) {
+                jlo = 2 * (jlo + tab.band_first);
+                jhi = jlo + 2 * tab.band_n - 1;
+            }
+        }
+    }
+    __device__ __forceinline__ void ext(const RowTable<D>& tab, bool child, int j, int& i0, int& i1, int& h0,
+                                        int& h1) const {
+        int x0, x1, a, b;
+        if constexpr (D == 2) {
+            tab.row_ext(yn + (child ? j >> 1 : j) - tab.y_first, x0, x1, a, b);
+        } else {
+            x0 = tab.x0;
+            x1 = tab.x1;
+            a = tab.a;
+            b = tab.b;
+        }
+        if (child) {
+            i0 = 2 * (a - xn);
+            i1 = 2 * (b - xn) + 1;
+            h0 = 1;
+            h1 = 0;
+            if (a > b) i1 = i0 - 1;
+        } else {
+            i0 = x0 - xn;
+            i1 = x1 - xn;
+            h0 = a - xn;
+            h1 = b - xn;
+            if (a > b) {
+                h0 = 1;
+                h1 = 0;
+            }
+        }
+    }
+};
+
+// Power sums L[ix(a, b)] = sum k^a j^b f of a lattice (spacing hs in thermal units, u at (fx, fy) in
+// its units) -> the moments sum x^a y^b f in thermal units about u, added to T.
+template <int D, bool FLUON>
+__device__ __forceinline__ void add_thermal(const double* Ls, double fx, double fy, double hs, double* T) {
+    using Q = DFPop<D, FLUON>;
+    constexpr int P = Q::P;
+    double sp[P + 1];
+    sp[0] = 1.0;
+#pragma unroll
+    for (int k = 1; k <= P; k++) sp[k] = sp[k - 1] * hs;
+    double K[Q::NB];
+#pragma unroll
+    for (int b = 0; b <= (D == 2 ? P : 0); b++) {
+        double col[P + 1], out[P + 1];
+#pragma unroll
+        for (int a = 0; a <= P; a++) col[a] = a + b <= P ? Ls[Q::ix(a, a + b <= P ? b : 0)] : 0.0;
+        origin_shift<P>(col, fx, out);
+#pragma unroll
+        for (int a = 0; a + b <= P; a++) K[Q::ix(a, b)] = out[a];
+    }
+    if constexpr (D == 1) {
+#pragma unroll
+        for (int a = 0; a <= P; a++) T[a] = fma(K[a], sp[a], T[a]);
+    } else {
+#pragma unroll
+        for (int a = 0; a <= P; a++) {
+            double col[P + 1], out[P + 1];
+#pragma unroll
+            for (int b = 0; b <= P; b++) col[b] = a + b <= P ? K[Q::ix(a + b <= P ? a : 0, b)] : 0.0;
+            origin_shift<P>(col, fy, out);
+#pragma unroll
+            for (int b = 0; a + b <= P; b++) T[Q::ix(a, b)] = fma(out[b], sp[a + b], T[Q::ix(a, b)]);
+        }
+    }
+}
+
+// One pass over the velocity set: the thermal moments of degree <= 3 of f (if doF) and <= 2 of g
+// (if doG) in FP64 (TF, TG) and the Jacobian's moments in FP32 (MF, MG).  Returns the point count.
+template <int D>
+__device__ __forceinline__ unsigned int moment_pass64(const CellState<D>& c, const RowTable<D>& tab,
+                                                      const CellLattice<D>& lat, const double* lf, const double* lg,
+                                                      bool doF, bool doG, double* TF, double* TG, float* MF,
+                                                      float* MG) {
+    using MS = MomentSet<D>;
+    using QF = DFPop<D, true>;
+    using QG = DFPop<D, false>;
+#pragma unroll
+    for (int i = 0; i < QF::NB; i++) TF[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < QG::NB; i++) TG[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < MS::NF; i++) MF[i] = 0.f;
+#pragma unroll
+    for (int i = 0; i < MS::NG; i++) MG[i] = 0.f;
+    unsigned int q = 0;
+#pragma unroll 1
+    for (int l = 0; l < lat.n; l++) {
+        const bool child = l == 1;
+        const double hs = child ? 0.5 * c.inv_sig : c.inv_sig;
+        const double ox = child ? 2.0 * lat.fx + 0.5 : lat.fx;  // u from the anchor, in spacings
+        const double oy = child ? 2.0 * lat.fy + 0.5 : lat.fy;
+        const float h32 = (float)hs, x32 = (float)(-ox * hs), y32 = (float)(-oy * hs);
+        const double w = child ? (D == 2 ? 0.25 : 0.5) : 1.0;
+        double LF[QF::NB], LG[QG::NB], S[4], G[3];
+        float SF[MS::PF + 1], SG[MS::PG + 1];
+#pragma unroll
+        for (int i = 0; i < QF::NB; i++) LF[i] = 0.0;
+#pragma unroll
+        for (int i = 0; i < QG::NB; i++) LG[i] = 0.0;
+        auto clear = [&]() {
+#pragma unroll
+            for (int a = 0; a < 4; a++) S[a] = 0.0;
+#pragma unroll
+            for (int a = 0; a < 3; a++) G[a] = 0.0;
+#pragma unroll
+            for (int a = 0; a <= MS::PF; a++) SF[a] = 0.f;
+#pragma unroll
+            for (int a = 0; a <= MS::PG; a++) SG[a] = 0.f;
+        };
+        clear();
+        auto point = [&](int k, int, double f, double g) {
+            q++;
+            const float kf = (float)k;  // k^2 and k^3 exact in FP32 up to |k| = 256
+            const double k1 = widen(kf), k2 = widen(kf * kf);
+            const float x = fmaf(kf, h32, x32);
+            const float x2 = x * x, x3 = x2 * x, x4 = x2 * x2;
+            const float pw[7] = {1.f, x, x2, x3, x4, x4 * x, x3 * x3};
+            if (doF) {
+                const double k3 = widen(kf * kf * kf);
+                S[0] += f;
+                S[1] = fma(k1, f, S[1]);
+                S[2] = fma(k2, f, S[2]);
+                S[3] = fma(k3, f, S[3]);
+                const float ff = narrow(f);
+#pragma unroll
+                for (int a = 0; a <= MS::PF; a++) SF[a] = fmaf(pw[a], ff, SF[a]);
+            }
+            if (doG) {
+                G[0] += g;
+                G[1] = fma(k1, g, G[1]);
+                G[2] = fma(k2, g, G[2]);
+                const float gf = narrow(g);
+#pragma unroll
+                for (int a = 0; a <= MS::PG; a++) SG[a] = fmaf(pw[a], gf, SG[a]);
+            }
+        };
+        auto row_end = [&](int j) {
+            if constexpr (D == 1) {
+#pragma unroll
+                for (int a = 0; a < 4; a++) LF[a] = S[a];
+#pragma unroll
+                for (int a = 0; a < 3; a++) LG[a] = G[a];
+#pragma unroll
+                for (int a = 0; a <= MS::PF; a++) MF[a] += SF[a];
+#pragma unroll
+                for (int a = 0; a <= MS::PG; a++) MG[a] += SG[a];
+            } else {
+                const float jf = (float)j, y = fmaf(jf, h32, y32);
+                const double jp[4] = {1.0, widen(jf), widen(jf * jf), widen(jf * jf * jf)};
+                float yp[MS::PF + 1];
+                yp[0] = 1.f;
+#pragma unroll
+                for (int k = 1; k <= MS::PF; k++) yp[k] = yp[k - 1] * y;
+                if (doF) {
+#pragma unroll
+                    for (int b = 0; b <= 3; b++)
+#pragma unroll
+                        for (int a = 0; a + b <= 3; a++)
+                            LF[QF::ix(a, b)] = b ? fma(jp[b], S[a], LF[QF::ix(a, b)]) : LF[QF::ix(a, b)] + S[a];
+#pragma unroll
+                    for (int b = 0; b <= MS::PF; b++)
+#pragma unroll
+                        for (int a = 0; a + b <= MS::PF; a++)
+                            MF[tix(a, b, MS::PF)] = fmaf(SF[a], yp[b], MF[tix(a, b, MS::PF)]);
+                }
+                if (doG) {
+#pragma unroll
+                    for (int b = 0; b <= 2; b++)
+#pragma unroll
+                        for (int a = 0; a + b <= 2; a++)
+                            LG[QG::ix(a, b)] = b ? fma(jp[b], G[a], LG[QG::ix(a, b)]) : LG[QG::ix(a, b)] + G[a];
+#pragma unroll
+                    for (int b = 0; b <= MS::PG; b++)
+#pragma unroll
+                        for (int a = 0; a + b <= MS::PG; a++)
+                            MG[tix(a, b, MS::PG)] = fmaf(SG[a], yp[b], MG[tix(a, b, MS::PG)]);
+                }
+                clear();
+            }
+        };
+        int jlo, jhi;
+        lat.rows(tab, child, jlo, jhi);
+        auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
+        lattice_sweep<D>(lf, lg, doF, doG, -ox * hs, -oy * hs, hs, w, w, jlo, jhi, ext, point, row_end);
+        if (doF) add_thermal<D, true>(LF, ox, oy, hs, TF);
+        if (doG) add_thermal<D, false>(LG, ox, oy, hs, TG);
+    }
+    return q;
+}
+
+// Newton update from the FP64 residual and the FP32 Jacobian of one pass (Eq. IID8-IID11).
+// Returns as newton_step_tol.
+template <int D, bool FLUON>
+__device__ __forceinline__ int newton_step64(const double* T, const float* Mom, const double* con, double* lam,
+                                             double tol, int max_iter, int it) {
+    using Q = DFPop<D, FLUON>;
+    constexpr int N = Q::N, PJ = Q::PJ;
+    float x[N];
+    long long worst = 0;  // |r| as integers: ordered as the doubles are, with NaN above infinity
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        const double r = T[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))] - con[j];
+        const long long b = __double_as_longlong(r) & 0x7fffffffffffffffLL;
+        worst = b > worst ? b : worst;
+        const float a = narrow(__longlong_as_double(b));
+        x[j] = __double2hiint(r) < 0 ? -a : a;
+    }
+    if (worst >= 0x7ff0000000000000LL) return -1;
+    const bool conv = worst <= __double_as_longlong(tol);
+    if (!conv && it >= max_iter) return -2;
+    float A[N * (N + 1) / 2];
+#pragma unroll
+    for (int i = 0; i < N; i++)
+#pragma unroll
+        for (int j = 0; j <= i; j++)
+            A[tri(i, j)] = Mom[D == 1 ? bx<D, FLUON>(i) + bx<D, FLUON>(j)
+                                      : tix(bx<D, FLUON>(i) + bx<D, FLUON>(j), by<D, FLUON>(i) + by<D, FLUON>(j), PJ)];
+    if (!ldlt_solve<float, N>(A, x)) return -1;
+    bool fin = true;
+#pragma unroll
+    for (int j = 0; j < N; j++) {
+        fin = fin && isfinite(x[j]);
+        lam[j] += widen(x[j]);
+    }
+    if (!fin) return -1;
+    return conv ? 1 : 0;
+}
+
+// Joint Newton iterations of both populations as solve_fg, with lattice-form passes.
+template <int D>
+__device__ __forceinline__ void solve_fg64(const CellState<D>& c, const RowTable<D>& tab, const CellLattice<D>& lat,
+                                           const double* conF, const double* conG, bool has_g, double* lf, double* lg,
+                                           const Model& m, int& sf, int& sg, unsigned int& npf, unsigned int& npg) {
+    bool fa = true, ga = has_g;
+    sf = 0;
+    sg = 0;
+#pragma unroll 1
+    for (int it = 0; fa || ga; it++) {
+        double TF[DFPop<D, true>::NB], TG[DFPop<D, false>::NB];
+        float MF[MomentSet<D>::NF], MG[MomentSet<D>::NG];
+        const unsigned int q = moment_pass64<D>(c, tab, lat, lf, lg, fa, ga, TF, TG, MF, MG);
+        if (ga) {
+            npg += q;
+            const int r = newton_step64<D, false>(TG, MG, conG, lg, m.tol, m.max_iter, it);
+            sg = r < 0 ? r : sg + 1;
+            ga = r == 0;
+        }
+        if (fa) {
+            npf += q;
+            const int r = newton_step64<D, true>(TF, MF, conF, lf, m.tol, m.max_iter, it);
+            sf = r < 0 ? r : sf + 1;
+            fa = r == 0;
+        }
+    }
+}
+
+}  // namespace lbm

@@ -25,7 +25,7 @@
 #include <mutex>
 
 #include "../../include/lelbm.h"
-#include "lelbm_device.cuh"
+#include "lelbm_step.cuh"
 
 namespace lbm {
 namespace {
@@ -118,14 +118,27 @@ __global__ void __launch_bounds__(128) noalloc_cell_kernel(Model m, Topo t, cons
     const long long* blk = scratch_blk();
     const int* len = scratch_len();
     const int* pads = scratch_pad();
-    __shared__ unsigned long long s_hist[64];
-    __shared__ unsigned long long s_cells, s_feq, s_fmx, s_q, s_dmax, s_pf, s_pg, s_pm;
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) s_hist[i] = 0;
-    if (threadIdx.x == 0) s_cells = s_feq = s_fmx = s_q = s_dmax = s_pf = s_pg = s_pm = 0;
+    __shared__ BlockCounters bc;
+    __shared__ ThreadCounters s_tc[128];
+    __shared__ double s_con[128][NF + NG];                                  // constraints of each thread's cell
+    __shared__ char2 s_rows[D == 2 ? 128 : 1][D == 2 ? kRowsMax : 1];       // and its row table
+    double* conF = s_con[threadIdx.x];
+    double* conG = conF + NF;
+    counters_init(bc);
+    s_tc[threadIdx.x] = ThreadCounters{0, 0, 0, 0, 0, 0, {0, 0.0, 0, 0}, 0, 0, 0};
+    ThreadCounters& tc = s_tc[threadIdx.x];
     __syncthreads();
+    Geometry g{};  // what the landing rules read (no walls; the 1D instance comes with the cell)
+    g.D = D;
+    g.NX = t.NX;
+    g.NY = t.NY;
+    g.ncell = t.ncell;
+    g.nx = t.nx;
+    g.ny = t.ny;
+    g.pad = t.pad;
+    g.periodic[0] = t.periodic[0];
+    g.periodic[1] = t.periodic[1];
 
-    unsigned long long my_cells = 0, my_pf = 0, my_pg = 0, my_q = 0, my_pts = 0;
-    double my_dmax = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long cell = (long long)blockIdx.x * blockDim.x + threadIdx.x; cell < t.ncell; cell += stride) {
         // where this cell's moments come from (Sec. III.A fill, done on the fly); the same
@@ -170,192 +183,25 @@ __global__ void __launch_bounds__(128) noalloc_cell_kernel(Model m, Topo t, cons
         CellState<D> c;
         collide<D>(M, m, c);  // as prepare_cell (lelbm_step.cuh) on the FP64 path
         if (!c.ok) {
-            atomicAdd(&s_fmx, 1ull);
+            atomicAdd(&bc.fmx, 1ull);
             atomicMin(&stats->first_fail, (unsigned long long)cell);
             continue;
         }
-        my_cells++;
+        tc.cells++;
         Stencil<D> st;
         st.init(c, m);
-        const bool has_g = m.K > 0.0;
         double lf[NF], lg[NG];
-        maxwell_start<D, NF>(c.RT, lf);
-        int sf = epr_newton<D, true>(c, st, c.cf, lf, m, my_pf);
-        int sg = 0;
-        if (has_g) {
-            maxwell_start<D, NG>(c.RT, lg);
-            sg = epr_newton<D, false>(c, st, c.cg, lg, m, my_pg);
-        } else {
+        maxwell_start_fg<D, NF, NG>(c.RT, lf, lg);
 #pragma unroll
-            for (int j = 0; j < NG; j++) lg[j] = 0.0;
-        }
-        if (sf >= 0 && sg >= 0) {
-            atomicAdd(&s_hist[sf < 63 ? sf : 63], 1ull);
-            if (has_g) atomicAdd(&s_hist[sg < 63 ? sg : 63], 1ull);
-        } else {
-            // the fallback chain of fp64_tail (lelbm_step.cuh): equilibrium constraints, then
-            // normalised Maxwellian weights; a change there must be made here too
-            double ef[NF], eg[NG];
+        for (int j = 0; j < NF; j++) conF[j] = c.cf[j];
 #pragma unroll
-            for (int j = 0; j < NF; j++) ef[j] = 0.0;
-#pragma unroll
-            for (int j = 0; j < NG; j++) eg[j] = 0.0;
-            ef[0] = eg[0] = 1.0;
-            int jj = 1 + D;
-#pragma unroll
-            for (int a = 0; a < D; a++)
-#pragma unroll
-                for (int b = a; b < D; b++) {
-                    ef[jj] = eg[jj] = (a == b) ? 1.0 : 0.0;
-                    jj++;
-                }
-            maxwell_start<D, NF>(c.RT, lf);
-            sf = epr_newton<D, true>(c, st, ef, lf, m, my_pf);
-            sg = 0;
-            if (has_g) {
-                maxwell_start<D, NG>(c.RT, lg);
-                sg = epr_newton<D, false>(c, st, eg, lg, m, my_pg);
-            }
-            if (sf >= 0 && sg >= 0) {
-                atomicAdd(&s_feq, 1ull);
-            } else {
-                double S = 0.0;
-                auto sum = [&](const double* cp, double dC) {
-                    double t2 = 0.0;
-#pragma unroll
-                    for (int a = 0; a < D; a++) {
-                        const double tt = (cp[a] - c.u[a]) * c.inv_sig;
-                        t2 += tt * tt;
-                    }
-                    S += dC * exp(-0.5 * t2);
-                };
-                st.for_each(sum);
-#pragma unroll
-                for (int j = 0; j < NF; j++) lf[j] = 0.0;
-                lf[0] = log(S) - 1.0;
-                jj = 1 + D;
-#pragma unroll
-                for (int a = 0; a < D; a++)
-#pragma unroll
-                    for (int b = a; b < D; b++) {
-                        lf[jj] = (a == b) ? 0.5 : 0.0;
-                        jj++;
-                    }
-#pragma unroll
-                for (int j = 0; j < NG; j++) lg[j] = lf[j];
-                atomicAdd(&s_fmx, 1ull);
-                atomicMin(&stats->first_fail, (unsigned long long)cell);
-            }
-        }
-        // moment streaming (Eq. IIE3) with the landing rules of the padded layout: those of
-        // land() (lelbm_land.cuh) and the cloud-in-cell sharing of scatter_cell (lelbm_step.cuh)
-        const double mfs = c.rho, mgs = c.rho * m.K * c.RT;
-        unsigned long long q = 0;
-        double dmax2 = 0.0;
-        auto emit = [&](const double* cp, double dC) {
-            q++;
-            double tt[D];
-#pragma unroll
-            for (int a = 0; a < D; a++) tt[a] = (cp[a] - c.u[a]) * c.inv_sig;
-            double T[NF];
-            Basis<D, true>::eval(tt, T);
-            double e = 1.0;
-#pragma unroll
-            for (int j = 0; j < NF; j++) e += lf[j] * T[j];
-            const double mf = mfs * dC * exp(-e);
-            double mg = 0.0;
-            if (has_g) {
-                double eg = 1.0;
-#pragma unroll
-                for (int j = 0; j < NG; j++) eg += lg[j] * T[j];
-                mg = mgs * dC * exp(-eg);
-            }
-            double csq = 0.0;
-#pragma unroll
-            for (int a = 0; a < D; a++) csq += cp[a] * cp[a];
-            dmax2 = fmax(dmax2, csq);
-            double dM[NM];
-            dM[0] = mf;
-#pragma unroll
-            for (int a = 0; a < D; a++) dM[1 + a] = cp[a] * mf;
-#pragma unroll
-            for (int a = 0; a < D; a++)
-#pragma unroll
-                for (int b = a; b < D; b++) dM[iM2<D>(a, b)] = cp[a] * cp[b] * mf;
-#pragma unroll
-            for (int gg = 0; gg < D; gg++) dM[iMD<D>(gg)] = csq * cp[gg] * mf;
-            dM[iG0<D>()] = mg;
-#pragma unroll
-            for (int gg = 0; gg < D; gg++) dM[iG1<D>(gg)] = cp[gg] * mg;
-            int base[D];
-            double w1[D];
-#pragma unroll
-            for (int a = 0; a < D; a++) {
-                const double fl = floor(cp[a]);
-                base[a] = (int)fl;
-                w1[a] = cp[a] - fl;
-            }
-            const int ncx = w1[0] > 0.0 ? 2 : 1;
-            const int ncy = (D == 2 && w1[D - 1] > 0.0) ? 2 : 1;
-            for (int sy = 0; sy < ncy; sy++)
-                for (int sx = 0; sx < ncx; sx++) {
-                    double w = sx ? w1[0] : 1.0 - w1[0];
-                    long long tgt;
-                    if constexpr (D == 1) {
-                        long long x = cell + base[0] + sx;
-                        if (t.periodic[0]) {
-                            long long r = (x - lo) % n;
-                            if (r < 0) r += n;
-                            x = lo + r;
-                        } else if (x < lo || x >= lo + n) {
-                            continue;
-                        }
-                        tgt = x;
-                    } else {
-                        w *= sy ? w1[D - 1] : 1.0 - w1[D - 1];
-                        int tx = ix + base[0] + sx, ty = iy + base[D - 1] + sy;
-                        if (t.periodic[0]) {
-                            tx %= t.nx;
-                            if (tx < 0) tx += t.nx;
-                        } else if (tx < t.pad || tx >= t.pad + t.nx) {
-                            continue;
-                        }
-                        if (t.periodic[1]) {
-                            ty %= t.ny;
-                            if (ty < 0) ty += t.ny;
-                        } else if (ty < t.pad || ty >= t.pad + t.ny) {
-                            continue;
-                        }
-                        tgt = (long long)ty * t.NX + tx;
-                    }
-#pragma unroll
-                    for (int mm = 0; mm < NM; mm++) atomicAdd(Mout + mm * t.ncell + tgt, w * dM[mm]);
-                }
-        };
-        st.for_each(emit);
-        my_q = q > my_q ? q : my_q;
-        my_pts += q;
-        my_dmax = fmax(my_dmax, sqrt(dmax2));
+        for (int j = 0; j < NG; j++) conG[j] = c.cg[j];
+        RowTable<D> tab;
+        tab.build(c, st, s_rows[D == 2 ? threadIdx.x : 0]);
+        fp64_cell<D>(m, g, nullptr, Mout, stats, CellPlace{cell, lo, n, ix, iy}, bc, tc, conF, conG, c, st, tab, lf, lg,
+                     false);
     }
-    atomicAdd(&s_cells, my_cells);
-    atomicAdd(&s_pf, my_pf);
-    atomicAdd(&s_pg, my_pg);
-    atomicAdd(&s_pm, my_pts);
-    atomicMax(&s_q, my_q);
-    atomicMax(&s_dmax, (unsigned long long)__double_as_longlong(my_dmax));
-    __syncthreads();
-    for (int i = threadIdx.x; i < 64; i += blockDim.x)
-        if (s_hist[i]) atomicAdd(&stats->newton_hist[i], s_hist[i]);
-    if (threadIdx.x == 0) {
-        atomicAdd(&stats->cells, s_cells);
-        atomicAdd(&stats->points_f, s_pf);
-        atomicAdd(&stats->points_g, s_pg);
-        atomicAdd(&stats->points_ms, s_pm);
-        if (s_feq) atomicAdd(&stats->fallback_eq, s_feq);
-        if (s_fmx) atomicAdd(&stats->fallback_mx, s_fmx);
-        atomicMax(&stats->q_max, s_q);
-        atomicMax(&stats->disp_max_bits, s_dmax);
-    }
+    counters_flush(bc, tc, stats);
 }
 
 // Device address of g_noalloc_scratch, looked up once per device.

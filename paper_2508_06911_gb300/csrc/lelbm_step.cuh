@@ -24,6 +24,7 @@
 
 #include "lelbm_device.cuh"
 #include "lelbm_df.cuh"
+#include "lelbm_fp64.cuh"
 #include "lelbm_internal.h"
 #include "lelbm_land.cuh"
 #include "lelbm_mlp.cuh"
@@ -442,11 +443,6 @@ __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g
 // Moment streaming, Eq. (IIE3): T_N(c_i) rho f'_i and T_N(c_i) rho K RT g'_i added at
 // x + c_i.  Level-0 points land on one cell; refined points are shared between the
 // cells they overlap (cloud-in-cell).
-//
-// With CHECK, the same pass also accumulates the moments of degree <= 3 (fluons)
-// and <= 2 (phonons) of the deposited populations and returns whether their
-// residual against conF / conG is within the tolerance (the FP64 judge of the
-// mixed path).  sign = -1 removes a previous deposit of the same populations.
 // Image populations of the no-slip walls (Sec. III.B, Eq. IIIB10-IIIB15) for a cell whose
 // streaming gave no-slip boundary n (1 at rest, 2 moving at u_w) the mass absorbed[2(n-1)]
 // (f) and the phonon energy absorbed[2(n-1)+1] (g).  The images of boundary n are the EPR
@@ -537,33 +533,39 @@ static __device__ __noinline__ void noslip_images(const Model& m, const Geometry
     }
 }
 
-template <int D, bool CHECK>
-__device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
-                                             long long cell, const CellState<D>& c, const Stencil<D>& st,
-                                             const double* lf, const double* lg, LocalStats& ls, double sign = 1.0,
-                                             const double* conF = nullptr, const double* conG = nullptr) {
-    constexpr int NM = Dim<D>::NM;
-    constexpr int RF = D == 1 ? 4 : 10, RG = D == 1 ? 3 : 6;  // monomials of degree <= 3 / <= 2
-    const bool has_g = m.K > 0.0;
-    const double mfs = sign * c.rho;               // rho dV f'
-    const double mgs = sign * c.rho * m.K * c.RT;  // rho K RT dV g'
-    double RFm[RF], RGm[RG];
-    if constexpr (CHECK) {
-#pragma unroll
-        for (int i = 0; i < RF; i++) RFm[i] = 0.0;
-#pragma unroll
-        for (int i = 0; i < RG; i++) RGm[i] = 0.0;
-    }
-    long long lo = 0;
-    int n = 0, ix = 0, iy = 0;
+// Where a cell's populations land: its place in the grid.
+struct CellPlace {
+    long long cell;
+    long long lo;  // 1D: first interior cell of the instance
+    int n;         // 1D: interior length of the instance
+    int ix, iy;    // 2D: padded coordinates
+};
+
+template <int D>
+__device__ __forceinline__ CellPlace cell_place(const Geometry& g, long long cell) {
+    CellPlace p{cell, 0, 0, 0, 0};
     if constexpr (D == 1) {
         const int b = g.inst_of_cell[cell];
-        lo = g.inst_lo[b];
-        n = g.inst_n[b];
+        p.lo = g.inst_lo[b];
+        p.n = g.inst_n[b];
     } else {
-        iy = (int)(cell / g.NX);
-        ix = (int)(cell - (long long)iy * g.NX);
+        p.iy = (int)(cell / g.NX);
+        p.ix = (int)(cell - (long long)p.iy * g.NX);
     }
+    return p;
+}
+
+template <int D>
+__device__ __forceinline__ void scatter_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                             const CellPlace& at, const CellState<D>& c, const Stencil<D>& st,
+                                             const double* lf, const double* lg, LocalStats& ls, const double* conF,
+                                             const double* conG) {
+    constexpr int NM = Dim<D>::NM;
+    const bool has_g = m.K > 0.0;
+    const double mfs = c.rho;               // rho dV f'
+    const double mgs = c.rho * m.K * c.RT;  // rho K RT dV g'
+    const long long cell = at.cell, lo = at.lo;
+    const int n = at.n, ix = at.ix, iy = at.iy;
     unsigned long long q = 0;
     long long walls = 0;
     double dmax2 = 0.0;
@@ -601,7 +603,7 @@ __device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, 
     auto deposit_traced = [&](const double* cp, double mf, double mg) {
         if constexpr (D == 2)
             walls += stream_traced(g, type, Mout, ix, iy, cp, mf, mg, kStreamReal, g.noslip ? absorbed : nullptr)
-                         ? (sign > 0.0 ? 1 : -1)
+                         ? 1
                          : 0;
     };
     auto row = [&](int cy, int xa, int xb) {
@@ -609,19 +611,8 @@ __device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, 
         if constexpr (D == 2) y = ((double)cy - c.u[1]) * c.inv_sig;
         double cf[4], cg[3];
         row_coeffs<D>(lf, lg, y, cf, cg);
-        double SF[4] = {0.0, 0.0, 0.0, 0.0}, SG[3] = {0.0, 0.0, 0.0};
         auto point = [&](int k, double x, double f, double gp) {
             const int cx = xa + k;
-            if constexpr (CHECK) {
-                const double x2 = x * x;
-                SF[0] += f;
-                SF[1] += x * f;
-                SF[2] += x2 * f;
-                SF[3] += x2 * x * f;
-                SG[0] += gp;
-                SG[1] += x * gp;
-                SG[2] += x2 * gp;
-            }
             double cp[D];
             cp[0] = (double)cx;
             if constexpr (D == 2) cp[1] = (double)cy;
@@ -631,18 +622,6 @@ __device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, 
                 deposit(land<D>(g, cell, lo, n, ix, iy, cx, cy), cp, mfs * f, mgs * gp);
         };
         row_eval(cf, cg, true, has_g, ((double)xa - c.u[0]) * c.inv_sig, c.inv_sig, xb - xa + 1, point);
-        if constexpr (CHECK) {
-            // fold y^b into the moments x^a y^b (a + b <= 3 / <= 2)
-            double yp[4] = {1.0, y, y * y, y * y * y};
-#pragma unroll
-            for (int b = 0; b <= (D == 2 ? 3 : 0); b++)
-#pragma unroll
-                for (int a = 0; a + b <= 3; a++) RFm[tix(a, b, 3)] += SF[a] * yp[b];
-#pragma unroll
-            for (int b = 0; b <= (D == 2 ? 2 : 0); b++)
-#pragma unroll
-                for (int a = 0; a + b <= 2; a++) RGm[tix(a, b, 2)] += SG[a] * yp[b];
-        }
         q += (unsigned long long)(xb - xa + 1);
         const double ex = (double)(abs(xa) > abs(xb) ? xa : xb);
         dmax2 = fmax(dmax2, ex * ex + (double)cy * (double)cy);
@@ -656,17 +635,6 @@ __device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, 
         const double f = dC * exp(-(((cf[3] * x + cf[2]) * x + cf[1]) * x + cf[0]));
         const double gp = has_g ? dC * exp(-((cg[2] * x + cg[1]) * x + cg[0])) : 0.0;
         const double mf = mfs * f, mg = mgs * gp;
-        if constexpr (CHECK) {
-            double px[4] = {1.0, x, x * x, x * x * x}, py[4] = {1.0, y, y * y, y * y * y};
-#pragma unroll
-            for (int b = 0; b <= (D == 2 ? 3 : 0); b++)
-#pragma unroll
-                for (int a = 0; a + b <= 3; a++) RFm[tix(a, b, 3)] += px[a] * py[b] * f;
-#pragma unroll
-            for (int b = 0; b <= (D == 2 ? 2 : 0); b++)
-#pragma unroll
-                for (int a = 0; a + b <= 2; a++) RGm[tix(a, b, 2)] += px[a] * py[b] * gp;
-        }
         q++;
         double csq = 0.0;
         int base[D];
@@ -702,26 +670,106 @@ __device__ __forceinline__ bool scatter_cell(const Model& m, const Geometry& g, 
     ls.points += q;
     ls.walls += walls;
     ls.disp_max2 = fmax(ls.disp_max2, dmax2);
-    if constexpr (CHECK) {
-        double rmax = 0.0;
-        bool finite = true;
-#pragma unroll
-        for (int j = 0; j < RF; j++) {
-            const double r = RFm[tix(bx<D, true>(j), by<D, true>(j), 3)] - conF[j];
-            finite = finite && isfinite(r);
-            rmax = fmax(rmax, fabs(r));
-        }
-        if (has_g) {
-#pragma unroll
-            for (int j = 0; j < RG; j++) {
-                const double r = RGm[tix(bx<D, false>(j), by<D, false>(j), 2)] - conG[j];
-                finite = finite && isfinite(r);
-                rmax = fmax(rmax, fabs(r));
-            }
-        }
-        return finite && rmax <= m.tol;
+}
+
+// scatter_cell in lattice form (lelbm_fp64.cuh), for a cell with a row table.
+template <int D>
+__device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                          const CellPlace& at, const CellState<D>& c, const Stencil<D>& st,
+                                          const RowTable<D>& tab, const CellLattice<D>& lat, const double* lf,
+                                          const double* lg, LocalStats& ls, const double* conF, const double* conG) {
+    constexpr int NM = Dim<D>::NM;
+    const bool has_g = m.K > 0.0;
+    const double mfs = c.rho, mgs = c.rho * m.K * c.RT;  // rho dV f', rho K RT dV g'
+    bool near_wall = false;  // as in scatter_cell
+    if constexpr (D == 2) {
+        if (g.wall_dist)
+            near_wall = (double)g.wall_dist[at.cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5;
     }
-    return true;
+    double absorbed[4] = {0.0, 0.0, 0.0, 0.0};
+    long long walls = 0;
+    unsigned int q = 0;
+    int far4 = 0;  // largest |c|^2 in (1/4 cell)^2
+#pragma unroll 1
+    for (int l = 0; l < lat.n; l++) {
+        const bool child = l == 1;
+        const double hs = child ? 0.5 * c.inv_sig : c.inv_sig;
+        const double ox = child ? 2.0 * lat.fx + 0.5 : lat.fx, oy = child ? 2.0 * lat.fy + 0.5 : lat.fy;
+        const double w = child ? (D == 2 ? 0.25 : 0.5) : 1.0;
+        auto point = [&](int k, int j, double mf, double mg) {
+            q++;
+            // velocity in quarter cells, exact; on the lattice or a quarter off it on either side
+            const int qx = child ? 4 * lat.xn - 1 + 2 * k : 4 * (lat.xn + k);
+            const int qy = D == 2 ? (child ? 4 * lat.yn - 1 + 2 * j : 4 * (lat.yn + j)) : 0;
+            far4 = max(far4, qx * qx + qy * qy);
+            const double cx = widen(0.25f * (float)qx), cy = D == 2 ? widen(0.25f * (float)qy) : 0.0;
+            if constexpr (D == 2) {
+                if (near_wall) {
+                    const double cp[2] = {cx, cy};
+                    walls += stream_traced(g, type, Mout, at.ix, at.iy, cp, mf, mg, kStreamReal,
+                                           g.noslip ? absorbed : nullptr)
+                                 ? 1
+                                 : 0;
+                    return;
+                }
+            }
+            double v[NM];
+            v[0] = mf;
+            v[1] = cx * mf;
+            if constexpr (D == 2) {
+                v[2] = cy * mf;
+                v[3] = cx * v[1];
+                v[4] = cx * v[2];
+                v[5] = cy * v[2];
+                const double e = v[3] + v[5];
+                v[6] = cx * e;
+                v[7] = cy * e;
+                v[8] = mg;
+                v[9] = cx * mg;
+                v[10] = cy * mg;
+            } else {
+                v[2] = cx * v[1];
+                v[3] = cx * v[2];
+                v[4] = mg;
+                v[5] = cx * mg;
+            }
+            const int bx0 = qx >> 2, by0 = qy >> 2;
+            if (!child) {
+                const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, bx0, by0);
+                if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) return;
+#pragma unroll
+                for (int mm = 0; mm < NM; mm++) atomicAdd(Mout + mm * g.ncell + tgt, v[mm]);
+                return;
+            }
+            // cloud-in-cell: along each axis 3/4 on the nearer cell, 1/4 on the other
+            const double wx1 = (qx & 3) == 3 ? 0.75 : 0.25, wy1 = (qy & 3) == 3 ? 0.75 : 0.25;
+#pragma unroll 1
+            for (int sy = 0; sy < (D == 2 ? 2 : 1); sy++)
+#pragma unroll 1
+                for (int sx = 0; sx < 2; sx++) {
+                    double ws = sx ? wx1 : 1.0 - wx1;
+                    if constexpr (D == 2) ws *= sy ? wy1 : 1.0 - wy1;
+                    const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, bx0 + sx, by0 + sy);
+                    if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) continue;
+#pragma unroll
+                    for (int mm = 0; mm < NM; mm++) atomicAdd(Mout + mm * g.ncell + tgt, ws * v[mm]);
+                }
+        };
+        auto row_end = [](int) {};
+        int jlo, jhi;
+        lat.rows(tab, child, jlo, jhi);
+        auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
+        lattice_sweep<D>(lf, lg, true, has_g, -ox * hs, -oy * hs, hs, w * mfs, w * mgs, jlo, jhi, ext, point,
+                         row_end);
+    }
+    if constexpr (D == 2) {
+        if (absorbed[0] != 0.0 || absorbed[1] != 0.0 || absorbed[2] != 0.0 || absorbed[3] != 0.0)
+            noslip_images(m, g, type, Mout, at.cell, at.ix, at.iy, c, st, lf, lg, conF, conG, mfs, mgs, absorbed);
+    }
+    if (q > ls.q_max) ls.q_max = q;
+    ls.points += q;
+    ls.walls += walls;
+    ls.disp_max2 = fmax(ls.disp_max2, 0.0625 * (double)far4);
 }
 
 // Per-block counters in shared memory, flushed to DevStats once per block.
@@ -801,17 +849,68 @@ __device__ __forceinline__ float start_base(int j, float l0) {
     return j == 0 ? l0 : (diag2 ? 0.5f : 0.f);
 }
 
+// Deterministic streaming: the multipliers that the gather kernel deposits from.
+template <int D>
+__device__ __forceinline__ void keep_for_gather(const Model& m, const Geometry& g, long long cell,
+                                                const CellState<D>& c, const Stencil<D>& st, const double* lf,
+                                                const double* lg) {
+    constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
+    const bool has_g = m.K > 0.0;
+#pragma unroll
+    for (int j = 0; j < NF; j++) m.det_lam[(long long)j * g.ncell + cell] = lf[j];
+#pragma unroll
+    for (int j = 0; j < NG; j++) m.det_lam[(long long)(NF + j) * g.ncell + cell] = has_g ? lg[j] : 0.0;
+    double umax = 0.0;
+#pragma unroll
+    for (int a = 0; a < D; a++) umax = fmax(umax, fabs(c.u[a]));
+    atomicMax(m.det_halo, (int)ceil(umax + (double)st.R + 0.5) + 1);
+}
+
+// What a converged solve leaves behind: the Newton counts, the stored start of the next step and the
+// training pair.
+template <int D>
+__device__ __forceinline__ void keep_solution(const Model& m, const Geometry& g, long long cell, BlockCounters& bc,
+                                              const CellState<D>& c, const Stencil<D>& st, const double* lf,
+                                              const double* lg, int sf, int sg) {
+    constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
+    const bool has_g = m.K > 0.0;
+    atomicAdd(&bc.hist[sf < 63 ? sf : 63], 1ull);
+    if (has_g) atomicAdd(&bc.hist[sg < 63 ? sg : 63], 1ull);
+    if (m.lam_store) {  // the converged multipliers minus Eq. (IID13), as FP32 corrections
+        const float l0 = (float)maxwell_l0<D>(c.RT);
+#pragma unroll
+        for (int j = 0; j < NF; j++)
+            m.lam_store[(long long)j * g.ncell + cell] = (float)lf[j] - start_base<D>(j, l0);
+#pragma unroll
+        for (int j = 0; j < NG; j++)
+            m.lam_store[(long long)(NF + j) * g.ncell + cell] = has_g ? (float)lg[j] - start_base<D>(j, l0) : 0.f;
+    }
+    if (m.rec_x) {  // training pairs: features and converged multipliers minus Eq. (IID13)
+        float xin[MlpDims<D>::NIN];
+        mlp_features<D>(c, st, xin);
+        double mf[NF], mg[NG];
+        maxwell_start_fg<D, NF, NG>(c.RT, mf, mg);
+#pragma unroll
+        for (int k = 0; k < MlpDims<D>::NIN; k++) m.rec_x[cell * MlpDims<D>::NIN + k] = xin[k];
+#pragma unroll
+        for (int j = 0; j < NF; j++) m.rec_y[cell * MlpDims<D>::NOUT + j] = (float)(lf[j] - mf[j]);
+#pragma unroll
+        for (int j = 0; j < NG; j++) m.rec_y[cell * MlpDims<D>::NOUT + NF + j] = has_g ? (float)(lg[j] - mg[j]) : 0.f;
+    }
+}
+
 // The FP64 EPR of one cell from the multipliers lf, lg, with the fallbacks of a failed
 // solve (equilibrium constraints, then normalised Maxwellian weights), and its FP64
 // streaming pass.
 template <int D>
 __device__ __forceinline__ void fp64_tail(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
-                                          DevStats* stats, long long cell, BlockCounters& bc,
+                                          DevStats* stats, const CellPlace& at, BlockCounters& bc,
                                           unsigned int& pf, unsigned int& pg, unsigned int& retry,
                                           LocalStats& ls, double* conF, double* conG, const CellState<D>& c,
                                           const Stencil<D>& st, double* lf, double* lg, bool learned) {
     constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
     const bool has_g = m.K > 0.0;
+    const long long cell = at.cell;
     int sf, sg;
     solve_fg<D>(c, st, conF, conG, has_g, lf, lg, m, sf, sg, pf, pg);
     if ((sf < 0 || sg < 0) && learned) {  // the plain EPR is the fallback of the learned start
@@ -820,29 +919,7 @@ __device__ __forceinline__ void fp64_tail(const Model& m, const Geometry& g, con
         solve_fg<D>(c, st, conF, conG, has_g, lf, lg, m, sf, sg, pf, pg);
     }
     if (sf >= 0 && sg >= 0) {
-        atomicAdd(&bc.hist[sf < 63 ? sf : 63], 1ull);
-        if (has_g) atomicAdd(&bc.hist[sg < 63 ? sg : 63], 1ull);
-        if (m.lam_store) {  // the converged multipliers minus Eq. (IID13), as FP32 corrections
-            const float l0 = (float)maxwell_l0<D>(c.RT);
-#pragma unroll
-            for (int j = 0; j < NF; j++)
-                m.lam_store[(long long)j * g.ncell + cell] = (float)lf[j] - start_base<D>(j, l0);
-#pragma unroll
-            for (int j = 0; j < NG; j++)
-                m.lam_store[(long long)(NF + j) * g.ncell + cell] = has_g ? (float)lg[j] - start_base<D>(j, l0) : 0.f;
-        }
-        if (m.rec_x) {  // training pairs: features and converged multipliers minus Eq. (IID13)
-            float xin[MlpDims<D>::NIN];
-            mlp_features<D>(c, st, xin);
-            double mf[NF], mg[NG];
-            maxwell_start_fg<D, NF, NG>(c.RT, mf, mg);
-#pragma unroll
-            for (int k = 0; k < MlpDims<D>::NIN; k++) m.rec_x[cell * MlpDims<D>::NIN + k] = xin[k];
-#pragma unroll
-            for (int j = 0; j < NF; j++) m.rec_y[cell * MlpDims<D>::NOUT + j] = (float)(lf[j] - mf[j]);
-#pragma unroll
-            for (int j = 0; j < NG; j++) m.rec_y[cell * MlpDims<D>::NOUT + NF + j] = has_g ? (float)(lg[j] - mg[j]) : 0.f;
-        }
+        keep_solution<D>(m, g, cell, bc, c, st, lf, lg, sf, sg);
     } else {
         // equilibrium constraints (omega = 1) for both populations
 #pragma unroll
@@ -889,14 +966,7 @@ __device__ __forceinline__ void fp64_tail(const Model& m, const Geometry& g, con
         }
     }
     if (m.det_lam) {  // deterministic streaming: the gather kernel deposits from these
-#pragma unroll
-        for (int j = 0; j < NF; j++) m.det_lam[(long long)j * g.ncell + cell] = lf[j];
-#pragma unroll
-        for (int j = 0; j < NG; j++) m.det_lam[(long long)(NF + j) * g.ncell + cell] = has_g ? lg[j] : 0.0;
-        double umax = 0.0;
-#pragma unroll
-        for (int a = 0; a < D; a++) umax = fmax(umax, fabs(c.u[a]));
-        atomicMax(m.det_halo, (int)ceil(umax + (double)st.R + 0.5) + 1);
+        keep_for_gather<D>(m, g, cell, c, st, lf, lg);
         unsigned long long q = 0;  // the velocity set's size and reach, for the counters
         auto count = [&](const double* cp, double) {
             q++;
@@ -909,13 +979,91 @@ __device__ __forceinline__ void fp64_tail(const Model& m, const Geometry& g, con
         if (q > ls.q_max) ls.q_max = q;
         return;
     }
-    scatter_cell<D, false>(m, g, type, Mout, cell, c, st, lf, lg, ls, 1.0, conF, conG);
+    scatter_cell<D>(m, g, type, Mout, at, c, st, lf, lg, ls, conF, conG);
 }
 
 struct TailCounts {
     unsigned int pf, pg, retry;
     LocalStats ls;
 };
+
+// fp64_tail from the multipliers lf, lg, out of line: the FP64 path's cells without a row table, and
+// those whose lattice-form solve broke down (then from Eq. IID13).
+template <int D>
+static __device__ __noinline__ TailCounts fp64_general_cold(const Model& m, const Geometry& g, const uint8_t* type,
+                                                            double* Mout, DevStats* stats, const CellPlace at,
+                                                            BlockCounters* bc, double* conF, double* conG,
+                                                            const CellState<D> c, const Stencil<D> st, double* lf,
+                                                            double* lg, bool learned) {
+    TailCounts t{0, 0, 0, {0, 0.0, 0, 0}};
+    fp64_tail<D>(m, g, type, Mout, stats, at, *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf, lg, learned);
+    return t;
+}
+
+__device__ __forceinline__ void add_tail(ThreadCounters& tc, const TailCounts& t) {
+    tc.pf += t.pf;
+    tc.pg += t.pg;
+    tc.retry += t.retry;
+    if (t.ls.q_max > tc.ls.q_max) tc.ls.q_max = t.ls.q_max;
+    tc.ls.points += t.ls.points;
+    tc.ls.walls += t.ls.walls;
+    tc.ls.disp_max2 = fmax(tc.ls.disp_max2, t.ls.disp_max2);
+}
+
+// Size and reach of a cell's velocity set, for the counters of a cell that does not stream here.
+template <int D>
+__device__ __forceinline__ void count_set(const RowTable<D>& tab, const CellLattice<D>& lat, LocalStats& ls) {
+    unsigned int q = 0;
+    int far4 = 0;
+    for (int l = 0; l < lat.n; l++) {
+        int jlo, jhi;
+        lat.rows(tab, l == 1, jlo, jhi);
+        for (int j = jlo; j <= jhi; j++) {
+            int i0, i1, h0, h1;
+            lat.ext(tab, l == 1, j, i0, i1, h0, h1);
+            if (i0 > i1) continue;
+            q += (unsigned int)(i1 - i0 + 1) - (h0 <= h1 ? (unsigned int)(h1 - h0 + 1) : 0u);
+            // the row's ends (a hole at an end leaves a nearer point, which the child row passes)
+            const int a = l ? 4 * lat.xn - 1 + 2 * i0 : 4 * (lat.xn + i0), b = l ? 4 * lat.xn - 1 + 2 * i1 : 4 * (lat.xn + i1);
+            const int y = D == 2 ? (l ? 4 * lat.yn - 1 + 2 * j : 4 * (lat.yn + j)) : 0;
+            if (l || h0 > h1 || h0 > i0) far4 = max(far4, a * a + y * y);
+            if (l || h0 > h1 || h1 < i1) far4 = max(far4, b * b + y * y);
+        }
+    }
+    if (q > ls.q_max) ls.q_max = q;
+    ls.disp_max2 = fmax(ls.disp_max2, 0.0625 * (double)far4);
+}
+
+// The FP64 path's cell after the collision: EPR from the multipliers lf, lg, and moment streaming, in
+// lattice form where the cell has a row table whose offsets are exact in FP32 (|k|^3 < 2^24).
+template <int D>
+__device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                          DevStats* stats, const CellPlace& at, BlockCounters& bc,
+                                          ThreadCounters& tc, double* conF, double* conG, const CellState<D>& c,
+                                          const Stencil<D>& st, const RowTable<D>& tab, double* lf, double* lg,
+                                          bool learned) {
+    const bool has_g = m.K > 0.0;
+    if (tab.ok && st.R <= 250) {
+        CellLattice<D> lat;
+        lat.init(c, tab);
+        int sf, sg;
+        solve_fg64<D>(c, tab, lat, conF, conG, has_g, lf, lg, m, sf, sg, tc.pf, tc.pg);
+        if (sf >= 0 && sg >= 0) {
+            keep_solution<D>(m, g, at.cell, bc, c, st, lf, lg, sf, sg);
+            if (m.det_lam) {
+                keep_for_gather<D>(m, g, at.cell, c, st, lf, lg);
+                count_set<D>(tab, lat, tc.ls);
+            } else {
+                scatter64<D>(m, g, type, Mout, at, c, st, tab, lat, lf, lg, tc.ls, conF, conG);
+            }
+            return;
+        }
+        if (learned) tc.retry++;
+        learned = false;
+        maxwell_start_fg<D, Dim<D>::NF, Dim<D>::NG>(c.RT, lf, lg);
+    }
+    add_tail(tc, fp64_general_cold<D>(m, g, type, Mout, stats, at, &bc, conF, conG, c, st, lf, lg, learned));
+}
 
 // fp64_tail from Eq. (IID13), out of line, for the FP32 path's rare failed solves; the
 // FP32 constraints cf32, cg32 are widened to FP64.
@@ -932,7 +1080,8 @@ static __device__ __noinline__ TailCounts fp64_tail_cold(const Model& m, const G
     for (int j = 0; j < Dim<D>::NG; j++) c.cg[j] = conG[j] = (double)cg32[j];
     double lf[Dim<D>::NF], lg[Dim<D>::NG];
     maxwell_start_fg<D, Dim<D>::NF, Dim<D>::NG>(c.RT, lf, lg);
-    fp64_tail<D>(m, g, type, Mout, stats, cell, *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf, lg, false);
+    fp64_tail<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf,
+                 lg, false);
     return t;
 }
 
@@ -1085,7 +1234,8 @@ static __device__ __noinline__ TailCounts fp64_cell_cold(const Model& m, const G
     for (int j = 0; j < Dim<D>::NG; j++) conG[j] = c.cg[j];
     double lf[Dim<D>::NF], lg[Dim<D>::NG];
     maxwell_start_fg<D, Dim<D>::NF, Dim<D>::NG>(c.RT, lf, lg);
-    fp64_tail<D>(m, g, type, Mout, stats, cell, *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf, lg, false);
+    fp64_tail<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf,
+                 lg, false);
     return t;
 }
 
@@ -1213,7 +1363,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
     RowTable<D> tab;
     if constexpr (PREC == PREC_FP32)
         tab.build32(c, st, rowbuf);
-    else if constexpr (PREC == PREC_MIXED)
+    else
         tab.build(c, st, rowbuf);
     if constexpr (PREC == PREC_FP32) {
         // FP32 Newton and FP32 streaming; the plain FP64 EPR is the fallback
@@ -1243,13 +1393,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
         // register allocation of the whole FP32 path
         tc.redo++;
         const TailCounts t = fp64_tail_cold<D>(m, g, type, Mout, stats, cell, &bc, conF, conG, c, st);
-        tc.pf += t.pf;
-        tc.pg += t.pg;
-        tc.retry += t.retry;
-        if (t.ls.q_max > tc.ls.q_max) tc.ls.q_max = t.ls.q_max;
-        tc.ls.points += t.ls.points;
-        tc.ls.walls += t.ls.walls;
-        tc.ls.disp_max2 = fmax(tc.ls.disp_max2, t.ls.disp_max2);
+        add_tail(tc, t);
     } else {
         if constexpr (PREC == PREC_MIXED) {
             // FP32 Newton, double-float correction and streaming judged at the FP64
@@ -1259,17 +1403,10 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
                 return;
             tc.redo++;
             const TailCounts t = fp64_cell_cold<D>(m, g, type, Min, Mout, stats, cell, &bc, conF, conG);
-            tc.pf += t.pf;
-            tc.pg += t.pg;
-            tc.retry += t.retry;
-            if (t.ls.q_max > tc.ls.q_max) tc.ls.q_max = t.ls.q_max;
-            tc.ls.points += t.ls.points;
-            tc.ls.walls += t.ls.walls;
-            tc.ls.disp_max2 = fmax(tc.ls.disp_max2, t.ls.disp_max2);
+            add_tail(tc, t);
             return;
         }
-        fp64_tail<D>(m, g, type, Mout, stats, cell, bc, tc.pf, tc.pg, tc.retry, tc.ls, conF, conG, c, st, lf, lg,
-                     learned);
+        fp64_cell<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), bc, tc, conF, conG, c, st, tab, lf, lg, learned);
     }
 }
 
@@ -1484,13 +1621,7 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
         // levels or rows than it holds), a failed FP32 phase or a missed check
         tc.redo++;
         const TailCounts t = fp64_cell_cold<D>(m, g, type, Min, Mout, stats, cell, &bc, conF, conG);
-        tc.pf += t.pf;
-        tc.pg += t.pg;
-        tc.retry += t.retry;
-        if (t.ls.q_max > tc.ls.q_max) tc.ls.q_max = t.ls.q_max;
-        tc.ls.points += t.ls.points;
-        tc.ls.walls += t.ls.walls;
-        tc.ls.disp_max2 = fmax(tc.ls.disp_max2, t.ls.disp_max2);
+        add_tail(tc, t);
     }
 }
 
@@ -1520,11 +1651,11 @@ __global__ void __launch_bounds__(cell_threads<PREC>(), min_blocks<D, PREC>()) c
     __shared__ BlockCounters bc;
     constexpr int NT = cell_threads<PREC>();
     __shared__ Con<PREC> s_con[NT][NF + NG];  // constraints of each thread's cell (out of registers)
-    // 2D row tables of the FP32 passes (one per thread)
-    __shared__ char2 s_rows[(D == 2 && PREC != PREC_FP64) ? NT : 1][(D == 2 && PREC != PREC_FP64) ? kRowsMax : 1];
+    // 2D row tables (one per thread)
+    __shared__ char2 s_rows[D == 2 ? NT : 1][D == 2 ? kRowsMax : 1];
     Con<PREC>* conF = s_con[threadIdx.x];
     Con<PREC>* conG = conF + NF;
-    char2* rowbuf = (D == 2 && PREC != PREC_FP64) ? s_rows[threadIdx.x] : nullptr;
+    char2* rowbuf = D == 2 ? s_rows[threadIdx.x] : nullptr;
     // double-float table of 2^(j/512) (mixed path)
     __shared__ float2 s_exp[PREC == PREC_MIXED ? kExpTab : 1];
     __shared__ long long s_beta[PREC == PREC_MIXED ? NT : 1][DFPop<D, true>::NB];  // exponent coefficients

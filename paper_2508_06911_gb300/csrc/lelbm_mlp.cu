@@ -18,7 +18,7 @@
 namespace lbm {
 namespace {
 
-constexpr int TB = 64;  // samples per block of the gradient kernel
+constexpr int TB = 64;  // samples per tile of the gradient kernel
 
 // Sum and sum of squares of every column of a row-major [n x cols] array.
 __global__ void column_stats_kernel(const float* A, long long n, int cols, double* sums) {
@@ -36,107 +36,299 @@ __global__ void to_bf16_kernel(const float* src, __nv_bfloat16* dst, int n) {
         dst[i] = __float2bfloat16(src[i]);
 }
 
-// Loss and gradient of one block of TB samples.  Every thread runs the forward and
-// backward pass of one sample and leaves its per-sample vectors in shared memory;
-// the weight gradients are then block-level products (dW2 = dZ2^T H1 and so on)
-// computed by slices of the flat parameter index and added to grad.
+// Loss and gradient over a range of samples, TB at a time.  FP32 throughout, at the BF16-rounded
+// weights.  The six products of a tile (three layers forward, two back, and the three weight
+// gradients) are register-tiled: a thread holds 8 samples x 4 features of a layer's tile, so a step
+// of the inner loop is 32 FMAs for three shared-memory loads, where one thread per sample had to load
+// an operand for every FMA.  Activations lie transposed in shared memory ([feature][sample]); the
+// derivatives of SiLU wait in registers.  Blocks are persistent: each keeps the whole gradient in
+// registers (a tile's sums are formed on their own, then added) and adds it to grad once, instead of
+// one atomic addition per parameter and 64 samples.  Two blocks share an SM, so one computes while the
+// other waits at a barrier.  2^20 pairs in 2D: see the launch bounds' note for times.
+constexpr int kGradThreads = 128;
+constexpr int kLD = TB + 4;  // row stride of the transposed tiles: float4 rows that start 4 banks apart
+
 template <int D>
-__global__ void __launch_bounds__(TB) mlp_grad_kernel(const __nv_bfloat16* Wb, const float* nrm, const float* X,
-                                                      const float* Y, const long long* idx, long long b0, int bsize,
-                                                      float scale, float* grad, double* loss) {
+struct GradTile {
     using Md = MlpDims<D>;
     using Ly = MlpLayout<D>;
-    constexpr int NIN = Md::NIN, NOUT = Md::NOUT, H = Md::H;
-    extern __shared__ float smem[];
-    float* Wf = smem;                           // NW weights as float
-    float* S_XS = Wf + ((Ly::NW + 3) & ~3);     // [TB][NIN] standardised inputs
-    float* S_H1 = S_XS + TB * NIN;              // [TB][H]
-    float* S_Z1 = S_H1 + TB * H;                // [TB][H] z1, then dz1
-    float* S_Z2 = S_Z1 + TB * H;                // [TB][H] z2, then dz2
-    float* S_H2 = S_Z2 + TB * H;                // [TB][H]
-    float* S_DY = S_H2 + TB * H;                // [TB][NOUT]
-    for (int i = threadIdx.x; i < Ly::NW; i += blockDim.x) Wf[i] = __bfloat162float(Wb[i]);
-    __syncthreads();
+    static constexpr int H = Md::H;
+    static constexpr int NI = (Md::NIN + 7) & ~7, NO = (Md::NOUT + 7) & ~7;  // padded with zeros
+    float W1t[NI][H], W2t[H][H], W2[H][H], W3t[H][NO], W3[NO][H];  // t: [input][output]
+    float b1[H], b2[H], b3[NO];
+    float xs[NI][kLD], h1[H][kLD], h2[H][kLD], dz2[H][kLD], dy[NO][kLD];  // h2's place takes dz1
+};
 
-    const int t = threadIdx.x;
-    const int r = blockIdx.x * TB + t;
-    const bool valid = r < bsize;
-    float* xs = S_XS + t * NIN;
-    float* h1 = S_H1 + t * H;
-    float* z1 = S_Z1 + t * H;
-    float* z2 = S_Z2 + t * H;
-    float* h2 = S_H2 + t * H;
-    float* dy = S_DY + t * NOUT;
-    float myloss = 0.f;
-    if (valid) {
-        const long long row = idx ? idx[b0 + r] : b0 + r;
+// acc[r][c] += sum_k A[k][s0 + r] B[k][f0 + c]
+template <int K, int LB>
+__device__ __forceinline__ void tile_product(const float* A, const float* B, float (&acc)[8][4]) {
+#pragma unroll 8
+    for (int k = 0; k < K; k++) {
+        const float4 a0 = *reinterpret_cast<const float4*>(A + k * kLD);
+        const float4 a1 = *reinterpret_cast<const float4*>(A + k * kLD + 4);
+        const float4 b = *reinterpret_cast<const float4*>(B + k * LB);
+        const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+        const float bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int m = 0; m < NIN; m++) xs[m] = (X[row * NIN + m] - nrm[m]) / nrm[NIN + m];
-        for (int j = 0; j < H; j++) {
-            float z = Wf[Ly::B1 + j];
+        for (int r = 0; r < 8; r++)
 #pragma unroll
-            for (int m = 0; m < NIN; m++) z = fmaf(Wf[Ly::W1 + j * NIN + m], xs[m], z);
-            z1[j] = z;
-            h1[j] = silu(z);
-        }
-        for (int i = 0; i < H; i++) {
-            float z = Wf[Ly::B2 + i];
-            for (int j = 0; j < H; j++) z = fmaf(Wf[Ly::W2 + i * H + j], h1[j], z);
-            z2[i] = z;
-            h2[i] = silu(z);
-        }
-        for (int k = 0; k < NOUT; k++) {
-            float y = Wf[Ly::B3 + k];
-            for (int i = 0; i < H; i++) y = fmaf(Wf[Ly::W3 + k * H + i], h2[i], y);
-            const float tgt = (Y[row * NOUT + k] - nrm[2 * NIN + k]) / nrm[2 * NIN + NOUT + k];
-            const float e = y - tgt;
-            myloss += e * e;
-            dy[k] = scale * e;
-        }
-        // dz2 = (W3^T dy) * silu'(z2), stored over z2
-        for (int i = 0; i < H; i++) {
-            float s = 0.f;
-#pragma unroll
-            for (int k = 0; k < NOUT; k++) s = fmaf(Wf[Ly::W3 + k * H + i], dy[k], s);
-            z2[i] = s * silu_grad(z2[i]);
-        }
-        // dz1 = (W2^T dz2) * silu'(z1), stored over z1
-        for (int j = 0; j < H; j++) {
-            float s = 0.f;
-            for (int i = 0; i < H; i++) s = fmaf(Wf[Ly::W2 + i * H + j], z2[i], s);
-            z1[j] = s * silu_grad(z1[j]);
-        }
-    } else {
-        for (int m = 0; m < NIN; m++) xs[m] = 0.f;
-        for (int j = 0; j < H; j++) h1[j] = z1[j] = z2[j] = h2[j] = 0.f;
-        for (int k = 0; k < NOUT; k++) dy[k] = 0.f;
+            for (int c = 0; c < 4; c++) acc[r][c] = fmaf(av[r], bv[c], acc[r][c]);
     }
-    __syncthreads();
-    for (int e = threadIdx.x; e < Ly::NW; e += blockDim.x) {
-        float s = 0.f;
-        if (e < Ly::B1) {
-            const int j = (e - Ly::W1) / NIN, m = (e - Ly::W1) % NIN;
-            for (int q = 0; q < TB; q++) s = fmaf(S_Z1[q * H + j], S_XS[q * NIN + m], s);
-        } else if (e < Ly::W2) {
-            const int j = e - Ly::B1;
-            for (int q = 0; q < TB; q++) s += S_Z1[q * H + j];
-        } else if (e < Ly::B2) {
-            const int i = (e - Ly::W2) / H, j = (e - Ly::W2) % H;
-            for (int q = 0; q < TB; q++) s = fmaf(S_Z2[q * H + i], S_H1[q * H + j], s);
-        } else if (e < Ly::W3) {
-            const int i = e - Ly::B2;
-            for (int q = 0; q < TB; q++) s += S_Z2[q * H + i];
-        } else if (e < Ly::B3) {
-            const int k = (e - Ly::W3) / H, i = (e - Ly::W3) % H;
-            for (int q = 0; q < TB; q++) s = fmaf(S_DY[q * NOUT + k], S_H2[q * H + i], s);
-        } else {
-            const int k = e - Ly::B3;
-            for (int q = 0; q < TB; q++) s += S_DY[q * NOUT + k];
+}
+
+// column c of a thread's tile to row f0 + c of a transposed array
+__device__ __forceinline__ void store_column(float* row, const float (&v)[8][4], int c) {
+    *reinterpret_cast<float4*>(row) = make_float4(v[0][c], v[1][c], v[2][c], v[3][c]);
+    *reinterpret_cast<float4*>(row + 4) = make_float4(v[4][c], v[5][c], v[6][c], v[7][c]);
+}
+
+// Sums over the tile's samples of A[ia][s] B[ib + 16... ][s]: out[r] += sum_s a[s] B_r[s], R rows of B
+// LDB floats apart.
+template <int R>
+__device__ __forceinline__ void sample_sums(const float* a, const float* B, int ldb, float (&out)[R]) {
+    float t[R];
+#pragma unroll
+    for (int r = 0; r < R; r++) t[r] = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < TB; s += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(a + s);
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            const float4 y = *reinterpret_cast<const float4*>(B + r * ldb + s);
+            t[r] = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, t[r]))));
         }
-        atomicAdd(&grad[e], s);
     }
-    for (int o = 16; o > 0; o >>= 1) myloss += __shfl_xor_sync(0xffffffffu, myloss, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, (double)myloss);
+#pragma unroll
+    for (int r = 0; r < R; r++) out[r] += t[r];
+}
+
+template <int D>
+__global__ void __launch_bounds__(kGradThreads, 2) mlp_grad_kernel(const __nv_bfloat16* Wb, const float* nrm,
+                                                                   const float* X, const float* Y,
+                                                                   const long long* idx, long long b0, int bsize,
+                                                                   float scale, float* grad, double* loss) {
+    using G = GradTile<D>;
+    using Md = MlpDims<D>;
+    using Ly = MlpLayout<D>;
+    constexpr int NIN = Md::NIN, NOUT = Md::NOUT, H = Md::H, NI = G::NI, NO = G::NO;
+    static_assert(H == 64 && TB == 64 && kGradThreads == 128, "thread tiles");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    G& S = *reinterpret_cast<G*>(smem_raw);
+    const int tid = threadIdx.x;
+    for (int i = tid; i < NI * H; i += kGradThreads) {
+        const int m = i / H, j = i % H;
+        S.W1t[m][j] = m < NIN ? __bfloat162float(Wb[Ly::W1 + j * NIN + m]) : 0.f;
+    }
+    for (int i = tid; i < H * H; i += kGradThreads) {
+        const float w = __bfloat162float(Wb[Ly::W2 + i]);
+        S.W2[i / H][i % H] = w;
+        S.W2t[i % H][i / H] = w;
+    }
+    for (int i = tid; i < NO * H; i += kGradThreads) {
+        const int k = i / H, j = i % H;
+        const float w = k < NOUT ? __bfloat162float(Wb[Ly::W3 + k * H + j]) : 0.f;
+        S.W3[k][j] = w;
+        S.W3t[j][k] = w;
+    }
+    for (int i = tid; i < H; i += kGradThreads) {
+        S.b1[i] = __bfloat162float(Wb[Ly::B1 + i]);
+        S.b2[i] = __bfloat162float(Wb[Ly::B2 + i]);
+        if (i < NO) S.b3[i] = i < NOUT ? __bfloat162float(Wb[Ly::B3 + i]) : 0.f;
+    }
+    const int s0 = (tid >> 4) * 8, f0 = (tid & 15) * 4;  // layer tiles: 8 samples x 4 features
+    const int row = tid & 63, half = tid >> 6;           // one row (sample, feature) and half of the other side
+    const int gi = tid >> 4, gj = tid & 15;              // gW2: rows gi + 8 r, columns gj + 16 c
+    float g2[8][4], g1[NI / 2], g3[NO / 2], gb1 = 0.f, gb2 = 0.f, gb3 = 0.f, myloss = 0.f;
+    double loss_sum = 0.0;
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) g2[r][c] = 0.f;
+#pragma unroll
+    for (int k = 0; k < NI / 2; k++) g1[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < NO / 2; k++) g3[k] = 0.f;
+
+    const int ntile = (bsize + TB - 1) / TB;
+    for (int tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+        const int r = tile * TB + row;
+        const bool valid = r < bsize;
+        const long long src = valid ? (idx ? idx[b0 + r] : b0 + r) : 0;
+        float tgt[NO / 2];
+#pragma unroll
+        for (int k = 0; k < NI / 2; k++) {
+            const int m = half * (NI / 2) + k;
+            S.xs[m][row] = valid && m < NIN ? (X[src * NIN + m] - nrm[m]) / nrm[NIN + m] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < NO / 2; k++) {
+            const int o = half * (NO / 2) + k;
+            tgt[k] = valid && o < NOUT ? (Y[src * NOUT + o] - nrm[2 * NIN + o]) / nrm[2 * NIN + NOUT + o] : 0.f;
+        }
+        __syncthreads();  // xs written (and, from the second tile on, the last one's sums read)
+        float d1[8][4], d2[8][4];  // SiLU'(z1), SiLU'(z2)
+        {
+            float z[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] = S.b1[f0 + c];
+            tile_product<NI, H>(&S.xs[0][s0], &S.W1t[0][f0], z);
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const float e = 1.f / (1.f + __expf(-z[q][c]));
+                    d1[q][c] = e * (1.f + z[q][c] * (1.f - e));
+                    z[q][c] *= e;
+                }
+#pragma unroll
+            for (int c = 0; c < 4; c++) store_column(&S.h1[f0 + c][s0], z, c);
+        }
+        __syncthreads();
+        {
+            float z[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] = S.b2[f0 + c];
+            tile_product<H, H>(&S.h1[0][s0], &S.W2t[0][f0], z);
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const float e = 1.f / (1.f + __expf(-z[q][c]));
+                    d2[q][c] = e * (1.f + z[q][c] * (1.f - e));
+                    z[q][c] *= e;
+                }
+#pragma unroll
+            for (int c = 0; c < 4; c++) store_column(&S.h2[f0 + c][s0], z, c);
+        }
+        __syncthreads();
+        {
+            // outputs, loss and dy: sample `row`, half of the outputs
+            float y[NO / 2];
+#pragma unroll
+            for (int k = 0; k < NO / 2; k++) y[k] = S.b3[half * (NO / 2) + k];
+#pragma unroll 8
+            for (int i = 0; i < H; i++) {
+                const float h = S.h2[i][row];
+#pragma unroll
+                for (int k = 0; k < NO / 2; k++) y[k] = fmaf(S.W3t[i][half * (NO / 2) + k], h, y[k]);
+            }
+#pragma unroll
+            for (int k = 0; k < NO / 2; k++) {
+                const int o = half * (NO / 2) + k;
+                const float e = valid && o < NOUT ? y[k] - tgt[k] : 0.f;
+                myloss += e * e;
+                S.dy[o][row] = scale * e;
+            }
+        }
+        __syncthreads();
+        {
+            // dz2 = (W3^T dy) SiLU'(z2)
+            float z[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] = 0.f;
+            tile_product<NO, H>(&S.dy[0][s0], &S.W3[0][f0], z);
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] *= d2[q][c];
+#pragma unroll
+            for (int c = 0; c < 4; c++) store_column(&S.dz2[f0 + c][s0], z, c);
+        }
+        __syncthreads();
+        {
+            // dz1 = (W2^T dz2) SiLU'(z1)
+            float z[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] = 0.f;
+            tile_product<H, H>(&S.dz2[0][s0], &S.W2[0][f0], z);
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) z[q][c] *= d1[q][c];
+            sample_sums<NO / 2>(&S.h2[row][0], &S.dy[half * (NO / 2)][0], kLD, g3);
+            __syncthreads();  // h2 read
+#pragma unroll
+            for (int c = 0; c < 4; c++) store_column(&S.h2[f0 + c][s0], z, c);
+        }
+        {
+            // gW2 += dz2^T h1
+            float t[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) t[q][c] = 0.f;
+#pragma unroll 2
+            for (int s = 0; s < TB; s += 4) {
+                float4 b[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) b[c] = *reinterpret_cast<const float4*>(&S.h1[gj + 16 * c][s]);
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const float4 a = *reinterpret_cast<const float4*>(&S.dz2[gi + 8 * q][s]);
+#pragma unroll
+                    for (int c = 0; c < 4; c++)
+                        t[q][c] = fmaf(a.x, b[c].x, fmaf(a.y, b[c].y, fmaf(a.z, b[c].z, fmaf(a.w, b[c].w, t[q][c]))));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+#pragma unroll
+                for (int c = 0; c < 4; c++) g2[q][c] += t[q][c];
+        }
+        __syncthreads();  // dz1 written
+        sample_sums<NI / 2>(&S.h2[row][0], &S.xs[half * (NI / 2)][0], kLD, g1);
+        {
+            const float* a = half ? &S.dz2[row][0] : &S.h2[row][0];
+            float t = 0.f;
+#pragma unroll 4
+            for (int s = 0; s < TB; s += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(a + s);
+                t += (v.x + v.y) + (v.z + v.w);
+            }
+            if (half)
+                gb2 += t;
+            else
+                gb1 += t;
+            if (tid < NO) {
+                float u = 0.f;
+#pragma unroll 4
+                for (int s = 0; s < TB; s += 4) {
+                    const float4 v = *reinterpret_cast<const float4*>(&S.dy[tid][s]);
+                    u += (v.x + v.y) + (v.z + v.w);
+                }
+                gb3 += u;
+            }
+        }
+        loss_sum += (double)myloss;
+        myloss = 0.f;
+        __syncthreads();  // the tile's arrays are free
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q++)
+#pragma unroll
+        for (int c = 0; c < 4; c++) atomicAdd(&grad[Ly::W2 + (gi + 8 * q) * H + gj + 16 * c], g2[q][c]);
+#pragma unroll
+    for (int k = 0; k < NI / 2; k++) {
+        const int m = half * (NI / 2) + k;
+        if (m < NIN) atomicAdd(&grad[Ly::W1 + row * NIN + m], g1[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < NO / 2; k++) {
+        const int o = half * (NO / 2) + k;
+        if (o < NOUT) atomicAdd(&grad[Ly::W3 + o * H + row], g3[k]);
+    }
+    atomicAdd(&grad[half ? Ly::B2 + row : Ly::B1 + row], half ? gb2 : gb1);
+    if (tid < NOUT) atomicAdd(&grad[Ly::B3 + tid], gb3);
+    for (int o = 16; o > 0; o >>= 1) loss_sum += __shfl_xor_sync(0xffffffffu, loss_sum, o);
+    if ((tid & 31) == 0) atomicAdd(loss, loss_sum);
 }
 
 // Adam on the FP32 master weights; refreshes the BF16 copy and clears the gradient.
@@ -156,20 +348,16 @@ __global__ void adam_kernel(float* master, __nv_bfloat16* Wb, float* grad, float
 }
 
 template <int D>
-size_t grad_smem_bytes() {
-    using Md = MlpDims<D>;
-    using Ly = MlpLayout<D>;
-    return sizeof(float) * (((Ly::NW + 3) & ~3) + TB * (Md::NIN + 4 * Md::H + Md::NOUT));
-}
-
-template <int D>
 int launch_grad(const __nv_bfloat16* Wb, const float* nrm, const float* X, const float* Y, const long long* idx,
                 long long b0, int bsize, float scale, float* grad, double* loss, cudaStream_t s) {
-    const size_t sm = grad_smem_bytes<D>();
-    if (cudaFuncSetAttribute(mlp_grad_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    const size_t sm = sizeof(GradTile<D>);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaFuncSetAttribute(mlp_grad_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
         return LELBM_E_CUDA;
-    const int blocks = (bsize + TB - 1) / TB;
-    mlp_grad_kernel<D><<<blocks, TB, sm, s>>>(Wb, nrm, X, Y, idx, b0, bsize, scale, grad, loss);
+    const int blocks = std::min((bsize + TB - 1) / TB, 2 * sms);  // two to an SM
+    mlp_grad_kernel<D><<<blocks, kGradThreads, sm, s>>>(Wb, nrm, X, Y, idx, b0, bsize, scale, grad, loss);
     return cudaGetLastError() == cudaSuccess ? LELBM_OK : LELBM_E_CUDA;
 }
 

@@ -53,11 +53,6 @@ struct MlpLayout {
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
 
-__device__ __forceinline__ float silu_grad(float z) {
-    const float s = 1.f / (1.f + __expf(-z));
-    return s * (1.f + z * (1.f - s));
-}
-
 template <int D, bool F32 = false>
 __device__ __forceinline__ void mlp_features(const CellState<D>& c, const Stencil<D>& st, float* x) {
     // the constraints in FP32: the FP32 path's own (exact), else rounded from FP64

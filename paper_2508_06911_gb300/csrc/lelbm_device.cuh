@@ -862,56 +862,6 @@ struct Basis {
 
 __device__ __forceinline__ constexpr int tri(int i, int j) { return i * (i + 1) / 2 + j; }
 
-// Cholesky factorisation of the packed lower triangle and solve A x = b.
-template <int N>
-__device__ __forceinline__ bool chol_solve(double* A, double* b) {
-#pragma unroll
-    for (int j = 0; j < N; j++) {
-        double s = A[tri(j, j)];
-#pragma unroll
-        for (int k = 0; k < j; k++) s -= A[tri(j, k)] * A[tri(j, k)];
-        if (!(s > 0.0)) return false;
-        const double d = sqrt(s);
-        const double id = 1.0 / d;
-        A[tri(j, j)] = d;
-#pragma unroll
-        for (int i = j + 1; i < N; i++) {
-            double t = A[tri(i, j)];
-#pragma unroll
-            for (int k = 0; k < j; k++) t -= A[tri(i, k)] * A[tri(j, k)];
-            A[tri(i, j)] = t * id;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < N; i++) {
-        double t = b[i];
-#pragma unroll
-        for (int k = 0; k < i; k++) t -= A[tri(i, k)] * b[k];
-        b[i] = t / A[tri(i, i)];
-    }
-#pragma unroll
-    for (int i = N - 1; i >= 0; i--) {
-        double t = b[i];
-#pragma unroll
-        for (int k = i + 1; k < N; k++) t -= A[tri(k, i)] * b[k];
-        b[i] = t / A[tri(i, i)];
-    }
-    return true;
-}
-
-// Eq. (IID13) in thermal units: lambda_0 = -1 + D/2 ln(2 pi RT), lambda_aa = 1/2.
-template <int D, int N>
-__device__ __forceinline__ void maxwell_start(double RT, double* lam) {
-#pragma unroll
-    for (int j = 0; j < N; j++) lam[j] = 0.0;
-    lam[0] = -1.0 + 0.5 * D * log(2.0 * 3.14159265358979323846 * RT);
-    int j = 1 + D;
-#pragma unroll
-    for (int a = 0; a < D; a++)
-#pragma unroll
-        for (int b = a; b < D; b++) lam[j++] = (a == b) ? 0.5 : 0.0;
-}
-
 // lambda_0 of Eq. (IID13).
 template <int D>
 __device__ __forceinline__ double maxwell_l0(double RT) {
@@ -954,67 +904,6 @@ __device__ __forceinline__ void maxwell_start32(float RT, float* lf, float* lg) 
             lf[j] = lg[j] = (a == b) ? 0.5f : 0.f;
             j++;
         }
-}
-
-// Newton-Raphson on the multipliers (Eq. IID8-IID11): returns the number of
-// updates (converged, one polishing update included), -1 on a breakdown
-// (non-finite residual, non-positive pivot), -2 at the iteration cap.
-template <int D, bool FLUON>
-__device__ int epr_newton(const CellState<D>& c, const Stencil<D>& st, const double* con, double* lam,
-                          const Model& m, unsigned long long& npts) {
-    using B = Basis<D, FLUON>;
-    constexpr int N = B::N;
-    constexpr int NA = N * (N + 1) / 2;
-    int updates = 0;
-    bool polished = false;
-    for (int it = 0;; it++) {
-        double A[NA];
-#pragma unroll
-        for (int i = 0; i < NA; i++) A[i] = 0.0;
-        const bool needA = !polished;
-        auto acc = [&](const double* cp, double dC) {
-            npts++;
-            double t[D];
-#pragma unroll
-            for (int a = 0; a < D; a++) t[a] = (cp[a] - c.u[a]) * c.inv_sig;
-            double T[N];
-            B::eval(t, T);
-            double e = 1.0;
-#pragma unroll
-            for (int j = 0; j < N; j++) e += lam[j] * T[j];
-            const double f = dC * exp(-e);
-            if (needA) {
-#pragma unroll
-                for (int i = 0; i < N; i++) {
-                    const double tf = T[i] * f;
-#pragma unroll
-                    for (int j = 0; j <= i; j++) A[tri(i, j)] += tf * T[j];
-                }
-            } else {
-#pragma unroll
-                for (int i = 0; i < N; i++) A[tri(i, 0)] += T[i] * f;
-            }
-        };
-        st.for_each(acc);
-        double r[N];
-        double rmax = 0.0;
-        bool finite = true;
-#pragma unroll
-        for (int j = 0; j < N; j++) {
-            r[j] = A[tri(j, 0)] - con[j];
-            finite = finite && isfinite(r[j]);
-            rmax = fmax(rmax, fabs(r[j]));
-        }
-        if (!finite) return -1;
-        if (polished) return updates;
-        const bool conv = rmax <= m.tol;
-        if (!conv && it >= m.max_iter) return -2;
-        if (!chol_solve<N>(A, r)) return -1;
-#pragma unroll
-        for (int j = 0; j < N; j++) lam[j] += r[j];
-        updates++;
-        if (conv) polished = true;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1512,10 +1401,10 @@ __device__ __forceinline__ unsigned long long moment_pass32(const CellState<D>& 
                 for (int a = 0; a + b <= MS::PG; a++) MG[tix(a, b, MS::PG)] = fmaf(SG[a], yp[b], MG[tix(a, b, MS::PG)]);
         }
     };
-    auto row = [&](int cy, int xa, int xb) { sweep(D == 2 ? tab.ty(cy) : 0.f, tab.tx(xa), s32, xb - xa + 1, 1.f); };
     if (TAB || tab.ok) {
         // level-0 runs as rows; the children of the split points a..b of a row as child rows
-        // (cy -/+ 1/4) of 2 (b - a + 1) points at p -/+ 1/4, spacing 1/2, weight 2^-D each
+        // (cy -/+ 1/4) of 2 (b - a + 1) points at p -/+ 1/4, spacing 1/2, weight 2^-D each.  One
+        // code site for every kind of row: several inlined copies do not fit the instruction caches.
         constexpr float wch = D == 1 ? 0.5f : 0.25f;
 #pragma unroll 1
         for (int r = 0; r < (D == 2 ? tab.nrows : 1); r++) {
@@ -1529,18 +1418,22 @@ __device__ __forceinline__ unsigned long long moment_pass32(const CellState<D>& 
                 ra = tab.a;
                 rb = tab.b;
             }
-            if (ra <= rb) {
-                if (rx0 <= ra - 1) row(cy, rx0, ra - 1);
-                if (rb + 1 <= rx1) row(cy, rb + 1, rx1);
+            const bool split = ra <= rb;
 #pragma unroll 1
-                for (int sy = (D == 2 ? -1 : 0); sy <= (D == 2 ? 1 : 0); sy += 2)
-                    sweep(D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f, tab.tx(ra, -0.25f), 0.5f * s32,
-                          2 * (rb - ra + 1), wch);
-            } else if (rx0 <= rx1) {
-                row(cy, rx0, rx1);
+            for (int seg = 0; seg < (split ? (D == 2 ? 4 : 3) : 1); seg++) {
+                const bool child = seg >= 2;
+                const int xa = child ? ra : (seg == 0 ? rx0 : rb + 1);
+                const int xb = child ? rb : (seg == 0 && split ? ra - 1 : rx1);
+                if (xa > xb) continue;
+                const float sy = D == 2 && child ? (seg == 2 ? -0.25f : 0.25f) : 0.f;
+                sweep(D == 2 ? tab.ty(cy, sy) : 0.f, tab.tx(xa, child ? -0.25f : 0.f), child ? 0.5f * s32 : s32,
+                      child ? 2 * (xb - xa + 1) : xb - xa + 1, child ? wch : 1.f);
             }
         }
     } else if constexpr (!TAB) {
+        auto row = [&](int cy, int xa, int xb) {
+            sweep(D == 2 ? tab.ty(cy) : 0.f, tab.tx(xa), s32, xb - xa + 1, 1.f);
+        };
         auto leaf = [&](const double* cp, double dC) {
             add_point((float)((cp[0] - c.u[0]) * c.inv_sig), D == 2 ? (float)((cp[D - 1] - c.u[D - 1]) * c.inv_sig) : 0.f,
                       (float)dC);
@@ -1548,62 +1441,6 @@ __device__ __forceinline__ unsigned long long moment_pass32(const CellState<D>& 
         st.for_each_row(row, leaf);
     }
     return q;
-}
-
-// FP32 Newton phase followed by one FP64 Newton pass.  Returns false when a
-// solve broke down (the caller then runs the plain FP64 solve).  sf, sg count
-// the FP64 updates; np32 counts the points of the FP32 passes.
-template <int D>
-__device__ __forceinline__ bool solve_fg_mixed(const CellState<D>& c, const Stencil<D>& st, const RowTable<D>& tab,
-                                               const double* conF, const double* conG, bool has_g, double* lf,
-                                               double* lg, const Model& m, int& sf, int& sg, unsigned int& npf,
-                                               unsigned int& npg, unsigned int& np32) {
-    using MS = MomentSet<D>;
-    constexpr int NF = Basis<D, true>::N, NG = Basis<D, false>::N;
-    constexpr float tol32 = 2e-5f;  // thermal units; the FP64 pass takes it to round-off
-    constexpr int max32 = 12;
-    float lf32[NF], lg32[NG], cf32[NF], cg32[NG];
-#pragma unroll
-    for (int j = 0; j < NF; j++) {
-        lf32[j] = (float)lf[j];
-        cf32[j] = (float)conF[j];
-    }
-#pragma unroll
-    for (int j = 0; j < NG; j++) {
-        lg32[j] = (float)lg[j];
-        cg32[j] = (float)conG[j];
-    }
-    bool fa = true, ga = has_g;
-    for (int it = 0; (fa || ga) && it < max32; it++) {
-        float MF32[MS::NF], MG32[MS::NG];
-        np32 += moment_pass32<D>(c, st, tab, lf32, lg32, fa, ga, MF32, MG32);
-        if (ga) {
-            const int r = newton_step32<D, false>(MG32, cg32, lg32, tol32, max32, it);
-            if (r < 0) return false;
-            if (r == 1) ga = false;
-        }
-        if (fa) {
-            const int r = newton_step32<D, true>(MF32, cf32, lf32, tol32, max32, it);
-            if (r < 0) return false;
-            if (r == 1) fa = false;
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < NF; j++) lf[j] = (double)lf32[j];
-#pragma unroll
-    for (int j = 0; j < NG; j++) lg[j] = (double)lg32[j];
-    double MF[MS::NF], MG[MS::NG];
-    const unsigned long long q = moment_pass<D>(c, st, lf, lg, true, has_g, MF, MG);
-    sg = 0;
-    if (has_g) {
-        npg += q;
-        if (newton_step_tol<D, false>(MG, conG, lg, m.tol, 1, 0) < 0) return false;
-        sg = 1;
-    }
-    npf += q;
-    if (newton_step_tol<D, true>(MF, conF, lf, m.tol, 1, 0) < 0) return false;
-    sf = 1;
-    return true;
 }
 
 // FP32 Newton alone (the FP32 path): FP32 passes and FP32 solves until the FP32

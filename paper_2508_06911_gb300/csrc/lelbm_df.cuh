@@ -29,23 +29,6 @@
 namespace lbm {
 
 // ---------------------------------------------------------------------------
-// FP32 <-> FP64 bit helpers (integer operations only; GB300's FP64 pipe also runs
-// the FP32 <-> FP64 conversion instructions).
-// ---------------------------------------------------------------------------
-// Subnormals become zero.
-__device__ __forceinline__ float flush_sub(float v) { return (__float_as_uint(v) & 0x7f800000u) ? v : 0.f; }
-
-// FP32 -> FP64: the exponent is rebiased from 127 to 1023 by one addition and the
-// mantissa shifted into place.  Normal numbers widen exactly; zeros and subnormals give
-// zero.  Infinities and NaNs, which a converged solve does not produce, come out finite.
-__device__ __forceinline__ double widen(float v) {
-    const unsigned int b = __float_as_uint(v);
-    const bool tiny = (b & 0x7f800000u) == 0u;
-    const unsigned int hi = (((b >> 3) & 0x0fffffffu) + 0x38000000u) | (b & 0x80000000u);
-    return __hiloint2double(tiny ? 0 : (int)hi, tiny ? 0 : (int)(b << 29));
-}
-
-// ---------------------------------------------------------------------------
 // Error-free transformations (explicitly rounded, so they cannot be contracted).
 // ---------------------------------------------------------------------------
 // Knuth's TwoSum: s + e = a + b exactly, for any a, b.
@@ -314,10 +297,7 @@ struct DFStream {
     const Geometry* g;
     const uint8_t* type;
     double* Mout;
-    long long cell;
-    long long lo;   // 1D: first interior cell of the instance
-    int n;          // 1D: interior length of the instance
-    int ix, iy;     // 2D: padded coordinates of the cell
+    CellPlace at;
     bool near_wall;
     float mh, ml;   // rho dV (fluons) or rho K RT dV (phonons), signed, as a double-float
     long long* beta;  // the thread's slot for the exponent coefficients (shared memory)
@@ -353,71 +333,61 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
     unsigned long long q = 0;
     long long walls = 0;
     int dmax = 0;
-    // deposit of T_N(c) m (m = ds.m f) at cell tgt: the population's stored moments, each
-    // as two FP64 atomic additions (the high and the low word, both widened exactly)
-    auto put = [&](long long tgt, int mm, float T, float vh, float vl) {
-        if (T == 0.f) return;
-        float p, e;
-        two_prod(T, vh, p, e);
-        e = __fmaf_rn(T, vl, e);
-        double* a = ds.Mout + (long long)mm * ds.g->ncell + tgt;
-        atomicAdd(a, widen(p));
-        atomicAdd(a, widen(e));
-    };
-    auto deposit = [&](long long tgt, float cx, float cy, float vh, float vl) {
-        if (tgt < 0 || !lands_on_fluid<D>(*ds.g, ds.type, tgt)) return;
-        if constexpr (FLUON) {
-            put(tgt, 0, 1.f, vh, vl);
-            put(tgt, 1, cx, vh, vl);
-            if constexpr (D == 2) put(tgt, 2, cy, vh, vl);
-            put(tgt, iM2<D>(0, 0), cx * cx, vh, vl);
-            const float csq = D == 2 ? fmaf(cx, cx, cy * cy) : cx * cx;
-            if constexpr (D == 2) {
-                put(tgt, iM2<D>(0, 1), cx * cy, vh, vl);
-                put(tgt, iM2<D>(1, 1), cy * cy, vh, vl);
-                put(tgt, iMD<D>(1), csq * cy, vh, vl);
-            }
-            put(tgt, iMD<D>(0), csq * cx, vh, vl);
-        } else {
-            put(tgt, iG0<D>(), 1.f, vh, vl);
-            put(tgt, iG1<D>(0), cx, vh, vl);
-            if constexpr (D == 2) put(tgt, iG1<D>(1), cy, vh, vl);
-        }
-    };
-    // a streamed point at lattice velocity (cx, cy) of population weight f; refined points
-    // (frac != 0) are shared by cloud-in-cell weights
-    auto stream_point = [&](float cx, float cy, float fh, float fl, bool refined) {
+    // a population at the lattice velocity (cx, cy): its mass in FP64, then FP64 moments and one
+    // atomic addition each (FP64 products cost fewer issue slots than double-float ones)
+    auto mass = [&](float fh, float fl) {
         float vh, vl;
         df_mul(ds.mh, ds.ml, fh, fl, vh, vl);
-        if constexpr (D == 2) {
-            if (ds.near_wall) {
-                const double cpd[2] = {(double)cx, (double)cy};
-                const double v = widen(vh) + widen(vl);
-                const bool hit =
-                    stream_traced(*ds.g, ds.type, ds.Mout, ds.ix, ds.iy, cpd, FLUON ? v : 0.0, FLUON ? 0.0 : v);
-                if (FLUON && hit) walls += ds.mh > 0.f ? 1 : -1;  // a path is counted once, with its fluons
-                return;
-            }
+        return widen(vh) + widen(vl);
+    };
+    // 1D: a child has only two landing cells, so its shares go one by one, as double-float products
+    // (FP32 instructions) with two atomic additions each, of the high and the low word (both widened
+    // exactly): 16 FP64 operations a child for merged columns cost the batch's cold tubes 2 %
+    auto put_df = [&](int dx, float cx, float vh, float vl) {
+        const long long tgt = land<D>(*ds.g, ds.at.cell, ds.at.lo, ds.at.n, 0, 0, dx, 0);
+        if (tgt < 0) return;
+        auto put = [&](int mm, float T) {
+            if (T == 0.f) return;
+            float p, e;
+            two_prod(T, vh, p, e);
+            e = __fmaf_rn(T, vl, e);
+            double* a = ds.Mout + (long long)mm * ds.g->ncell + tgt;
+            atomicAdd(a, widen(p));
+            atomicAdd(a, widen(e));
+        };
+        if constexpr (FLUON) {
+            put(0, 1.f);
+            put(1, cx);
+            put(2, cx * cx);
+            put(3, cx * cx * cx);
+        } else {
+            put(4, 1.f);
+            put(5, cx);
         }
-        if (!refined) {
-            deposit(land<D>(*ds.g, ds.cell, ds.lo, ds.n, ds.ix, ds.iy, (int)cx, (int)cy), cx, cy, vh, vl);
+    };
+    auto stream_1d = [&](float cx, float fh, float fl, bool child) {
+        float vh, vl;
+        df_mul(ds.mh, ds.ml, fh, fl, vh, vl);
+        if (!child) {
+            put_df((int)cx, cx, vh, vl);
             return;
         }
-        // children sit at +-1/4: along each axis 3/4 on the nearer cell, 1/4 on the other
-        const float flx = floorf(cx), fly = floorf(cy);
-        const float w1x = cx - flx, w1y = cy - fly;
+        const float flx = floorf(cx), w1 = cx - flx;
 #pragma unroll 1
-        for (int sy = 0; sy < (D == 2 ? 2 : 1); sy++)
-#pragma unroll 1
-            for (int sx = 0; sx < 2; sx++) {
-                float w = sx ? w1x : 1.f - w1x;
-                if constexpr (D == 2) w *= sy ? w1y : 1.f - w1y;
-                float sh, sl;
-                two_prod(w, vh, sh, sl);
-                sl = __fmaf_rn(w, vl, sl);
-                deposit(land<D>(*ds.g, ds.cell, ds.lo, ds.n, ds.ix, ds.iy, (int)flx + sx, D == 2 ? (int)fly + sy : 0),
-                        cx, cy, sh, sl);
-            }
+        for (int sx = 0; sx < 2; sx++) {
+            const float w = sx ? w1 : 1.f - w1;
+            float sh, sl;
+            two_prod(w, vh, sh, sl);
+            put_df((int)flx + sx, cx, sh, __fmaf_rn(w, vl, sl));
+        }
+    };
+    auto trace = [&](double cx, double cy, double v) {
+        if constexpr (D == 2) {
+            const double cp[2] = {cx, cy};
+            const bool hit = stream_traced(*ds.g, ds.type, ds.Mout, ds.at.ix, ds.at.iy, cp, FLUON ? v : 0.0,
+                                           FLUON ? 0.0 : v);
+            if (FLUON && hit) walls += ds.mh > 0.f ? 1 : -1;  // a path is counted once, with its fluons
+        }
     };
     // folds the row sums S (residual) and SJ (Jacobian) of a row at lattice offset Yf
     // (thermal y32) into the cell moments
@@ -466,10 +436,15 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
     // Every segment of a row -- its level-0 runs (lattice step 1) and, for split points, its
     // child rows (children at p -/+ 1/4, step 1/2, weight 2^-D) -- is one arithmetic
     // progression of points along x, swept by the same loop: the exponent advances by exact
-    // forward differences D0..D3 (int64, kFixBits fractional bits) from its first point.
-    const int nrows = D == 2 ? tab.nrows : 1;
+    // forward differences D0..D3 (int64, kFixBits fractional bits) from its first point.  The
+    // level-0 runs of all rows go first (lattice 0), then all child rows (lattice 1): the code of
+    // one kind then stays in the instruction caches.
 #pragma unroll 1
-    for (int rr = 0; rr < nrows; rr++) {
+    for (int lat = 0; lat < 2; lat++) {
+    const int r_first = D == 2 && lat ? tab.band_first : 0;
+    const int r_end = D == 2 ? (lat ? r_first + tab.band_n : tab.nrows) : 1;
+#pragma unroll 1
+    for (int rr = r_first; rr < r_end; rr++) {
         int rx0, rx1, ra, rb, cy = 0;
         if constexpr (D == 2) {
             tab.row_ext(rr, rx0, rx1, ra, rb);
@@ -483,11 +458,11 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
         const int Y = cy - tab.yc;
         const bool split = ra <= rb;
         long long gm[P + 1];
-        if (rx0 <= rx1) fix_row<D, FLUON>(beta, Y, gm);
+        if (lat == 0 && rx0 <= rx1) fix_row<D, FLUON>(beta, Y, gm);
         // segments 0, 1: level-0 runs rx0..ra-1 and rb+1..rx1 (the whole row when no point
         // splits); 2 (and 3 in 2D): the child rows at cy - 1/4 and cy + 1/4
 #pragma unroll 1
-        for (int seg = 0; seg < (D == 2 ? 4 : 3); seg++) {
+        for (int seg = 2 * lat; seg < (lat ? (D == 2 ? 4 : 3) : 2); seg++) {
             long long D0, D1, D2 = 0, D3 = 0;
             float Xf, h, Yf, y32;
             int np, dn;
@@ -543,12 +518,36 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
 #pragma unroll
             for (int a = 0; a <= PJ; a++) SJ[a] = 0.f;
             const float cyf = (float)tab.yc + Yf;  // c_y of the segment's points
+            const bool child = dn != 0;
+            const int sy = D == 2 && child ? (seg == 2 ? -1 : 1) : 0;
+            const bool traced = D == 2 && MODE == DF_STREAM && ds.near_wall;
+            ChildRow<D, FLUON, !FLUON> kids;
+            if constexpr (MODE == DF_STREAM) kids.start();
+            const int nk = D == 2 && MODE == DF_STREAM && child && !traced ? np + 3 : np;
 #pragma unroll 1
-            for (int k = 0; k < np; k++) {
-                float fh, fl;
-                exp2_fix(D0, etab, dn, fh, fl);
-                accumulate(S, SJ, Xf, fh, fl);
-                if constexpr (MODE == DF_STREAM) stream_point((float)tab.xc + Xf, cyf, fh, fl, dn != 0);
+            for (int k = 0; k < nk; k++) {
+                float fh = 0.f, fl = 0.f;
+                if (k < np) {
+                    exp2_fix(D0, etab, dn, fh, fl);
+                    accumulate(S, SJ, Xf, fh, fl);
+                }
+                if constexpr (MODE == DF_STREAM) {
+                    const float cx = (float)tab.xc + Xf;
+                    if constexpr (D == 1) {
+                        stream_1d(cx, fh, fl, child);
+                    } else {
+                    const double v = mass(fh, fl);
+                    if (traced) {
+                        trace(widen(cx), D == 2 ? widen(cyf) : 0.0, v);
+                    } else if (child) {
+                        kids.add(*ds.g, ds.type, ds.Mout, ds.at, ra, k, cy, sy, v, v);
+                    } else {
+                        double vm[Stored<D, FLUON, !FLUON>::N];
+                        stored_moments<D, FLUON, !FLUON>(widen(cx), widen(cyf), v, v, vm);
+                        deposit_at<D, FLUON, !FLUON>(*ds.g, ds.type, ds.Mout, ds.at, tab.xc + (int)Xf, cy, vm);
+                    }
+                    }
+                }
                 D0 += D1;
                 D1 += D2;
                 if constexpr (P == 3) D2 += D3;
@@ -557,6 +556,7 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
             q += (unsigned long long)np;
             fold(S, SJ, Yf, y32);
         }
+    }
     }
     npts += (unsigned int)q;
     if constexpr (MODE == DF_STREAM) {

@@ -11,6 +11,23 @@
 
 namespace lbm {
 
+// ---------------------------------------------------------------------------
+// FP32 <-> FP64 bit helpers (integer operations only; GB300's FP64 pipe also runs
+// the FP32 <-> FP64 conversion instructions).
+// ---------------------------------------------------------------------------
+// Subnormals become zero.
+__device__ __forceinline__ float flush_sub(float v) { return (__float_as_uint(v) & 0x7f800000u) ? v : 0.f; }
+
+// FP32 -> FP64: the exponent is rebiased from 127 to 1023 by one addition and the
+// mantissa shifted into place.  Normal numbers widen exactly; zeros and subnormals give
+// zero.  Infinities and NaNs, which a converged solve does not produce, come out finite.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned int b = __float_as_uint(v);
+    const bool tiny = (b & 0x7f800000u) == 0u;
+    const unsigned int hi = (((b >> 3) & 0x0fffffffu) + 0x38000000u) | (b & 0x80000000u);
+    return __hiloint2double(tiny ? 0 : (int)hi, tiny ? 0 : (int)(b << 29));
+}
+
 struct LocalStats {
     unsigned long long q_max;
     double disp_max2;
@@ -56,6 +73,166 @@ __device__ __forceinline__ bool lands_on_fluid(const Geometry& g, const uint8_t*
     if constexpr (D == 1) return true;
     return g.wall_dist == nullptr || type[tgt] == CELL_FLUID;
 }
+
+// Where a cell's populations land: its place in the grid.
+struct CellPlace {
+    long long cell;
+    long long lo;  // 1D: first interior cell of the instance
+    int n;         // 1D: interior length of the instance
+    int ix, iy;    // 2D: padded coordinates
+};
+
+template <int D>
+__device__ __forceinline__ CellPlace cell_place(const Geometry& g, long long cell) {
+    CellPlace p{cell, 0, 0, 0, 0};
+    if constexpr (D == 1) {
+        const int b = g.inst_of_cell[cell];
+        p.lo = g.inst_lo[b];
+        p.n = g.inst_n[b];
+    } else {
+        p.iy = (int)(cell / g.NX);
+        p.ix = (int)(cell - (long long)p.iy * g.NX);
+    }
+    return p;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 deposits of fluons (F), phonons (G) or both.  Their stored moments of one velocity are
+// products of the coordinates with the population (ten FP64 products in 2D); one atomic addition
+// per moment.
+// ---------------------------------------------------------------------------
+template <int D, bool F, bool G>
+struct Stored {
+    static constexpr int NFM = F ? (D == 1 ? 4 : 8) : 0, NGM = G ? 1 + D : 0, N = NFM + NGM;
+    __device__ __forceinline__ static constexpr int moment(int k) { return k < NFM ? k : k - NFM + iG0<D>(); }
+};
+
+// T_N(c) f and T_N(c) g of the velocity (cx, cy).
+template <int D, bool F, bool G>
+__device__ __forceinline__ void stored_moments(double cx, double cy, double f, double gp, double* v) {
+    constexpr int NFM = Stored<D, F, G>::NFM;
+    if constexpr (F) {
+        v[0] = f;
+        v[1] = cx * f;
+        if constexpr (D == 1) {
+            v[2] = cx * v[1];
+            v[3] = cx * v[2];
+        } else {
+            v[2] = cy * f;
+            v[3] = cx * v[1];
+            v[4] = cx * v[2];
+            v[5] = cy * v[2];
+            const double e = v[3] + v[5];
+            v[6] = cx * e;
+            v[7] = cy * e;
+        }
+    }
+    if constexpr (G) {
+        v[NFM] = gp;
+        v[NFM + 1] = cx * gp;
+        if constexpr (D == 2) v[NFM + 2] = cy * gp;
+    }
+}
+
+// Adds v to the cell at the lattice displacement (dx, dy), unless the population leaves the grid or
+// lands on a wall.
+template <int D, bool F, bool G>
+__device__ __forceinline__ void deposit_at(const Geometry& g, const uint8_t* type, double* Mout, const CellPlace& at,
+                                           int dx, int dy, const double* v) {
+    const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, dx, dy);
+    if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) return;
+#pragma unroll
+    for (int k = 0; k < Stored<D, F, G>::N; k++) atomicAdd(Mout + Stored<D, F, G>::moment(k) * g.ncell + tgt, v[k]);
+}
+
+// v / 4 (exact) by an integer subtraction on the exponent.
+__device__ __forceinline__ double quarter(double v) {
+    const int hi = __double2hiint(v), e = hi & 0x7ff00000;
+    return (e > 0x00200000 && e < 0x7ff00000) ? __hiloint2double(hi - 0x00200000, __double2loint(v)) : 0.25 * v;
+}
+
+// The children of one child row (split points first, first + 1, ...; children h = 0, 1, ... at
+// p -/+ 1/4, p = first + h / 2), merged per landing column before they are deposited: a child lands
+// 3/4 on its parent's column p and 1/4 on p -/+ 1, and in 2D 3/4 on the parent's row cy and 1/4 on
+// cy + sy.  On a row the eight stored fluon moments are combinations of the four sums x^a f (a <= 3)
+// and the phonons' of two, so a child costs 16 FP64 operations and a column 18, where depositing
+// every share alone took 11 for each of its four landing cells and four times the atomic additions.
+// A column is complete after the left child of the next point, so a row of n children ends with
+// three empty ones; every column leaves through one code site (refined cells are bound by
+// instruction fetch: with a site for each of the last columns and for both rows the 1024^2 mixed
+// step at RT 0.35 took 11.8 ms, with one 8.0 ms).
+template <int D, bool F, bool G>
+struct ChildRow {
+    static constexpr int NS = (F ? 4 : 0) + (G ? 2 : 0);
+    double a[NS], b[NS];  // sums of the columns p - 1 | p (before a left | right child) and the next
+
+    __device__ __forceinline__ void start() {
+#pragma unroll
+        for (int k = 0; k < NS; k++) a[k] = b[k] = 0.0;
+    }
+    // the next child, of mass f and energy gp (zero past the last)
+    __device__ __forceinline__ void add(const Geometry& g, const uint8_t* type, double* Mout, const CellPlace& at,
+                                        int first, int h, int cy, int sy, double f, double gp) {
+        using S = Stored<D, F, G>;
+        const int p = first + (h >> 1);
+        const bool left = (h & 1) == 0;
+        const double x = widen((float)p + (left ? -0.25f : 0.25f));  // exact: |p| < 2^21
+        const double wa = left ? 0.25 : 0.75, wb = left ? 0.75 : 0.25;
+        double s[NS];
+        if constexpr (F) {
+            s[0] = f;
+#pragma unroll
+            for (int k = 1; k < 4; k++) s[k] = x * s[k - 1];
+        }
+        if constexpr (G) {
+            s[NS - 2] = gp;
+            s[NS - 1] = x * gp;
+        }
+#pragma unroll
+        for (int k = 0; k < NS; k++) {
+            a[k] = fma(wa, s[k], a[k]);
+            b[k] = fma(wb, s[k], b[k]);
+        }
+        if (!left) return;
+        double v[S::N];
+        if constexpr (D == 1) {
+#pragma unroll
+            for (int k = 0; k < NS; k++) v[k] = a[k];
+        } else {
+            const double y = widen((float)cy + 0.25f * (float)sy);
+            if constexpr (F) {
+                v[0] = a[0];
+                v[1] = a[1];
+                v[2] = y * a[0];
+                v[3] = a[2];
+                v[4] = y * a[1];
+                v[5] = y * v[2];
+                v[6] = fma(y, v[4], a[3]);
+                v[7] = y * (a[2] + v[5]);
+            }
+            if constexpr (G) {
+                v[S::NFM] = a[NS - 2];
+                v[S::NFM + 1] = a[NS - 1];
+                v[S::NFM + 2] = y * a[NS - 2];
+            }
+        }
+#pragma unroll 1
+        for (int k = D == 2 ? 0 : 1; k < 2; k++) {  // in 2D a quarter on the row cy + sy, then the rest on cy
+            double o[S::N];
+#pragma unroll
+            for (int i = 0; i < S::N; i++) {
+                o[i] = k == 0 ? quarter(v[i]) : v[i];
+                if (k == 0) v[i] -= o[i];
+            }
+            deposit_at<D, F, G>(g, type, Mout, at, p - 1, k == 0 ? cy + sy : cy, o);
+        }
+#pragma unroll
+        for (int k = 0; k < NS; k++) {
+            a[k] = b[k];
+            b[k] = 0.0;
+        }
+    }
+};
 
 // ---------------------------------------------------------------------------
 // Solid boundary, Sec. III.B (stationary adiabatic slip wall, 2D).

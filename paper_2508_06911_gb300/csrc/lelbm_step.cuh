@@ -143,6 +143,184 @@ static __device__ __noinline__ bool stream_traced32(const Geometry& g, const uin
     return L.touched;
 }
 
+// What the emitted fractions miss of the conserved moments stays in the cell.
+template <int D>
+__device__ __forceinline__ void keep_shortfall32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                                 long long cell, const CellState<D>& c, const Acc32& em,
+                                                 const Acc32* ep, const Acc32& ee) {
+    if (type[cell] != CELL_FLUID) return;
+    double usq = 0.0;
+#pragma unroll
+    for (int a = 0; a < D; a++) usq += c.u[a] * c.u[a];
+    const double dm = c.rho - em.value();
+    const double dE = c.rho * (usq + ((double)D + m.K) * c.RT) - ee.value();
+    atomicAdd(Mout + cell, dm);
+#pragma unroll
+    for (int a = 0; a < D; a++) {
+        atomicAdd(Mout + (1 + a) * g.ncell + cell, c.rho * c.u[a] - ep[a].value());
+        atomicAdd(Mout + iM2<D>(a, a) * g.ncell + cell, dE / (double)D);
+    }
+}
+
+// Moment streaming of the FP32 path for a cell with a row table and no wall in reach.  The level-0
+// points of all rows go first, then the child rows, whose children are merged per landing column
+// (as in ChildRow, in FP32): four sums x^a f and two x^a g a column, expanded to the stored moments
+// once and shared 3/4 : 1/4 between the rows cy and cy + sy; the larger share is rounded and the
+// smaller is the exact difference, so the accounting takes a column once.
+template <int D>
+__device__ __forceinline__ void scatter_table32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                                long long cell, const CellState<D>& c, const RowTable<D>& tab,
+                                                const float* lf, const float* lg, LocalStats& ls) {
+    constexpr int NM = Dim<D>::NM;
+    const bool has_g = m.K > 0.0;
+    const float mfs = (float)c.rho;                              // rho dV f'
+    const float mgs = has_g ? (float)(c.rho * m.K * c.RT) : 0.f;  // rho K RT dV g'
+    const CellPlace at = cell_place<D>(g, cell);
+    Acc32 em{0.f, 0.f}, ee{0.f, 0.f}, ep[D];
+#pragma unroll
+    for (int a = 0; a < D; a++) ep[a] = Acc32{0.f, 0.f};
+    auto account = [&](const float* v) {
+        em.add(v[0]);
+#pragma unroll
+        for (int a = 0; a < D; a++) ep[a].add(v[1 + a]);
+#pragma unroll
+        for (int a = 0; a < D; a++) ee.add(v[iM2<D>(a, a)]);
+        ee.add(v[iG0<D>()]);
+    };
+    auto put = [&](int dx, int dy, const float* v) {
+        const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, dx, dy);
+        if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) return;
+        double* p = Mout + tgt;
+#pragma unroll
+        for (int mm = 0; mm < NM; mm++) atomicAdd(p + mm * g.ncell, widen(v[mm]));
+    };
+    unsigned int q = 0;
+    int dmax = 0;
+    const float s32 = tab.s32;
+#pragma unroll 1
+    for (int lat = 0; lat < 2; lat++) {
+        const int r_first = D == 2 && lat ? tab.band_first : 0;
+        const int r_end = D == 2 ? (lat ? r_first + tab.band_n : tab.nrows) : 1;
+#pragma unroll 1
+        for (int r = r_first; r < r_end; r++) {
+            int rx0, rx1, ra, rb, cy = 0;
+            if constexpr (D == 2) {
+                tab.row_ext(r, rx0, rx1, ra, rb);
+                cy = tab.y_first + r;
+            } else {
+                rx0 = tab.x0;
+                rx1 = tab.x1;
+                ra = tab.a;
+                rb = tab.b;
+            }
+            const bool split = ra <= rb;
+            if (lat == 0) {
+                float cf[4], cg[3];
+                row_coeffs32<D>(lf, lg, D == 2 ? tab.ty(cy) : 0.f, cf, cg);
+                if (rx0 <= rx1) {
+                    const int ex = max(abs(rx0), abs(rx1));
+                    dmax = max(dmax, ex * ex + cy * cy);
+                }
+#pragma unroll 1
+                for (int seg = 0; seg < (split ? 2 : 1); seg++) {
+                    const int xa = seg == 0 ? rx0 : rb + 1, xb = seg == 0 && split ? ra - 1 : rx1;
+                    const float x0 = tab.tx(xa);
+                    float kf = 0.f, cxf = (float)xa;  // point index and c_x as floats (exact)
+#pragma unroll 1
+                    for (int cx = xa; cx <= xb; cx++, kf += 1.f, cxf += 1.f) {
+                        const float x = fmaf(kf, s32, x0);
+                        const float f = __expf(-fmaf(fmaf(fmaf(cf[3], x, cf[2]), x, cf[1]), x, cf[0]));
+                        const float gp = has_g ? __expf(-fmaf(fmaf(cg[2], x, cg[1]), x, cg[0])) : 0.f;
+                        float cpf[D];
+                        cpf[0] = cxf;
+                        if constexpr (D == 2) cpf[1] = (float)cy;
+                        float v[NM];
+                        fractions32<D>(cpf, mfs * f, mgs * gp, v);
+                        account(v);
+                        put(cx, cy, v);
+                    }
+                    if (xa <= xb) q += (unsigned int)(xb - xa + 1);
+                }
+                continue;
+            }
+            if (!split) continue;
+#pragma unroll 1
+            for (int sy = (D == 2 ? -1 : 0); sy <= (D == 2 ? 1 : 0); sy += 2) {
+                constexpr float w_child = D == 1 ? 0.5f : 0.25f;
+                float cf[4], cg[3];
+                row_coeffs32<D>(lf, lg, D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f, cf, cg);
+                const float y = (float)cy + 0.25f * (float)sy;
+                const int nk = 2 * (rb - ra + 1);
+                q += (unsigned int)nk;
+                float A[6], B[6];  // columns p - 1 | p (before a left | right child) and the next
+#pragma unroll
+                for (int k = 0; k < 6; k++) A[k] = B[k] = 0.f;
+#pragma unroll 1
+                for (int h = 0; h < nk + 3; h++) {  // three empty children complete the last columns
+                    const int p = ra + (h >> 1);
+                    const bool left = (h & 1) == 0;
+                    const float cx = (float)p + (left ? -0.25f : 0.25f);
+                    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                    if (h < nk) {
+                        const float x = tab.tx(p, left ? -0.25f : 0.25f);
+                        s[0] = mfs * w_child * __expf(-fmaf(fmaf(fmaf(cf[3], x, cf[2]), x, cf[1]), x, cf[0]));
+                        s[4] = has_g ? mgs * w_child * __expf(-fmaf(fmaf(cg[2], x, cg[1]), x, cg[0])) : 0.f;
+#pragma unroll
+                        for (int k = 1; k < 4; k++) s[k] = cx * s[k - 1];
+                        s[5] = cx * s[4];
+                    }
+                    const float wa = left ? 0.25f : 0.75f, wb = left ? 0.75f : 0.25f;
+#pragma unroll
+                    for (int k = 0; k < 6; k++) {
+                        A[k] = fmaf(wa, s[k], A[k]);
+                        B[k] = fmaf(wb, s[k], B[k]);
+                    }
+                    if (!left) continue;
+                    float v[NM];
+                    if constexpr (D == 1) {
+#pragma unroll
+                        for (int k = 0; k < 6; k++) v[k] = A[k];
+                    } else {
+                        v[0] = A[0];
+                        v[1] = A[1];
+                        v[2] = y * A[0];
+                        v[3] = A[2];
+                        v[4] = y * A[1];
+                        v[5] = y * v[2];
+                        v[6] = fmaf(y, v[4], A[3]);
+                        v[7] = y * (A[2] + v[5]);
+                        v[8] = A[4];
+                        v[9] = A[5];
+                        v[10] = y * A[4];
+                    }
+                    account(v);
+#pragma unroll 1
+                    for (int k = D == 2 ? 0 : 1; k < 2; k++) {  // 2D: 1/4 on the row cy + sy, the rest on cy
+                        float o[NM];
+#pragma unroll
+                        for (int i = 0; i < NM; i++) {
+                            // 3/4 v rounded; v less that is exact (flushed, so that both are normal or zero)
+                            const float big = flush_sub(__fmul_rn(0.75f, v[i]));
+                            o[i] = k == 0 ? __fsub_rn(v[i], big) : (D == 2 ? big : v[i]);
+                        }
+                        put(p - 1, k == 0 ? cy + sy : cy, o);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 6; k++) {
+                        A[k] = B[k];
+                        B[k] = 0.f;
+                    }
+                }
+            }
+        }
+    }
+    keep_shortfall32<D>(m, g, type, Mout, cell, c, em, ep, ee);
+    if (q > ls.q_max) ls.q_max = q;
+    ls.points += q;
+    ls.disp_max2 = fmax(ls.disp_max2, (double)dmax);
+}
+
+// Moment streaming of the FP32 path for any cell: near a wall, or without a row table.
 template <int D>
 __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                                long long cell, const CellState<D>& c, const Stencil<D>& st,
@@ -254,119 +432,6 @@ __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g
                 put(land<D>(g, cell, lo, n, ix, iy, base[0] + sx, D == 2 ? base[D - 1] + sy : 0), part);
             }
     };
-    // Split points without wall tracing: one deposit per landing cell and child row.  Along
-    // x the children p -/+ 1/4 land 3/4 on p and 1/4 on p -/+ 1; their shares are summed
-    // with each other and with the level-0 points a - 1 and b + 1 of the row (1D), or, in
-    // 2D, per child row cy + sy/4 and then shared 3/4 : 1/4 between rows cy and cy + sy.
-    // The accounting takes the deposits as they are.
-    constexpr float w_child = D == 1 ? 0.5f : 0.25f;
-    // fractions of the level-0 point (cx, cy), and of the child (p + sx/4, cy + sy/4) with
-    // the exponent polynomials cf, cg of its row
-    auto point_v = [&](int cx, int cy, float* v) {
-        float cf[4], cg[3];
-        row_coeffs32<D>(lf, lg, D == 2 ? tab.ty(cy) : 0.f, cf, cg);
-        const float x = tab.tx(cx);
-        const float f = __expf(-fmaf(fmaf(fmaf(cf[3], x, cf[2]), x, cf[1]), x, cf[0]));
-        const float gp = has_g ? __expf(-fmaf(fmaf(cg[2], x, cg[1]), x, cg[0])) : 0.f;
-        float cpf[D];
-        cpf[0] = (float)cx;
-        if constexpr (D == 2) cpf[1] = (float)cy;
-        fractions32<D>(cpf, mfs * f, mgs * gp, v);
-    };
-    auto child_v = [&](const float* cf, const float* cg, int p, int sx, float cyq, float* v) {
-        const float x = tab.tx(p, 0.25f * (float)sx);
-        const float f = w_child * __expf(-fmaf(fmaf(fmaf(cf[3], x, cf[2]), x, cf[1]), x, cf[0]));
-        const float gp = has_g ? w_child * __expf(-fmaf(fmaf(cg[2], x, cg[1]), x, cg[0])) : 0.f;
-        float cpf[D];
-        cpf[0] = (float)p + 0.25f * (float)sx;
-        if constexpr (D == 2) cpf[1] = cyq;
-        fractions32<D>(cpf, mfs * f, mgs * gp, v);
-    };
-    auto emit = [&](int tx, int ty, const float* v) {
-        account(v);
-        put(land<D>(g, cell, lo, n, ix, iy, tx, ty), v);
-    };
-    // column t of child row sy: V (x-summed children) and, when l0, the level-0 point (t, cy).
-    // 1D: one deposit V (+ the point); 2D: V/4 on row cy + sy, 3V/4 (+ the point) on row cy.
-    // One call site each for emit and point_v keeps the code of this path short.
-    auto emit_col = [&](int t, int cy, int sy, const float* V, bool l0) {
-        float lv[NM];
-        if (l0) {
-            point_v(t, cy, lv);
-        } else {
-#pragma unroll
-            for (int mm = 0; mm < NM; mm++) lv[mm] = 0.f;
-        }
-#pragma unroll 1
-        for (int k = (D == 2 ? 0 : 1); k < 2; k++) {
-            const float w = D == 1 ? 1.f : (k == 0 ? 0.25f : 0.75f);
-            float o[NM];
-#pragma unroll
-            for (int mm = 0; mm < NM; mm++) o[mm] = k == 0 ? w * V[mm] : fmaf(w, V[mm], lv[mm]);
-            emit(t, k == 0 ? cy + sy : cy, o);
-        }
-    };
-    // child row sy (0 in 1D) of the split points a..b of row cy (level-0 points x0..x1);
-    // with_l0: the level-0 points a - 1 and b + 1 join their columns' deposits.  The
-    // children are taken in order p - 1/4, p + 1/4, ...; each adds w_lo of its fractions
-    // to column lo (cA) and w_hi to column lo + 1 (cB): (p - 1, p) with (1/4, 3/4) for the
-    // left child, (p, p + 1) with (3/4, 1/4) for the right one.  After a left child,
-    // column p - 1 is complete.  Two empty left children past b emit columns b and b + 1.
-    auto band_row = [&](int cy, int sy, int a, int b, int x0, int x1, bool with_l0) {
-        float cf[4], cg[3];
-        row_coeffs32<D>(lf, lg, D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f, cf, cg);
-        const float cyq = (float)cy + 0.25f * (float)sy;
-        float cA[NM], cB[NM], v[NM];
-#pragma unroll
-        for (int mm = 0; mm < NM; mm++) cA[mm] = cB[mm] = 0.f;
-        const int nch = 2 * (b - a + 1);
-#pragma unroll 1
-        for (int h = 0; h <= nch + 2; h++) {
-            const int p = a + (h >> 1);
-            const bool left = (h & 1) == 0;
-            if (h < nch) {
-                child_v(cf, cg, p, left ? -1 : 1, cyq, v);
-            } else {
-#pragma unroll
-                for (int mm = 0; mm < NM; mm++) v[mm] = 0.f;
-            }
-            const float w_lo = left ? 0.25f : 0.75f, w_hi = left ? 0.75f : 0.25f;
-#pragma unroll
-            for (int mm = 0; mm < NM; mm++) {
-                cA[mm] = fmaf(w_lo, v[mm], cA[mm]);
-                cB[mm] = fmaf(w_hi, v[mm], cB[mm]);
-            }
-            if (left) {
-                const int t = p - 1;  // complete
-                emit_col(t, cy, sy, cA, with_l0 && ((t == a - 1 && t >= x0) || (t == b + 1 && t <= x1)));
-#pragma unroll
-                for (int mm = 0; mm < NM; mm++) {
-                    cA[mm] = cB[mm];
-                    cB[mm] = 0.f;
-                }
-            }
-        }
-        q += (unsigned long long)nch + (with_l0 ? (a - 1 >= x0) + (b + 1 <= x1) : 0);
-        const int ex = max(abs(x0), abs(x1));
-        dmax = max(dmax, ex * ex + cy * cy);
-    };
-    // a row with split points a..b: its level-0 segments and its child rows
-    auto split_row = [&](int cy, int x0, int x1, int a, int b) {
-#pragma unroll 1
-        for (int sy = (D == 2 ? -1 : 0); sy <= (D == 2 ? 1 : 0); sy += 2) band_row(cy, sy, a, b, x0, x1, sy <= 0);
-    };
-    // the level-0 segments of a row: x0..x1 less the split points a..b and their
-    // neighbours a - 1, b + 1 (which split_row deposits)
-    auto row_segments = [&](int cy, int x0, int x1, int a, int b) {
-        const bool band = a <= b;
-#pragma unroll 1
-        for (int k = 0; k < (band ? 2 : 1); k++) {
-            const int xa = band ? (k == 0 ? x0 : b + 2) : x0;
-            const int xb = band ? (k == 0 ? a - 2 : x1) : x1;
-            if (xa <= xb) row(cy, xa, xb);
-        }
-        if (band) split_row(cy, x0, x1, a, b);
-    };
     if (tab.ok) {
         // children of split points at (p + sx/4, cy + sy/4): along an axis the landing
         // point p - 1/4 splits 3/4 : 1/4 over p - 1, p and p + 1/4 splits over p, p + 1
@@ -392,17 +457,7 @@ __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g
             }
             refined(cpf, tab.tx(p, qx), D == 2 ? tab.ty(cy, qy) : 0.f, D == 1 ? 0.5f : 0.25f, base, w1, cpd);
         };
-        if (near_wall) {
-            tab.visit(row, child);  // every share is traced on its own
-        } else if constexpr (D == 1) {
-            row_segments(0, tab.x0, tab.x1, tab.a, tab.b);
-        } else {
-            for (int r = 0; r < tab.nrows; r++) {
-                int rx0, rx1, ra, rb;
-                tab.row_ext(r, rx0, rx1, ra, rb);
-                row_segments(tab.y_first + r, rx0, rx1, ra, rb);
-            }
-        }
+        tab.visit(row, child);  // every share on its own (near a wall it is traced)
     } else {
         auto leaf = [&](const double* cp, double dC) {
             float cpf[D];
@@ -420,20 +475,7 @@ __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g
         };
         st.for_each_row(row, leaf);
     }
-    // what the emitted fractions miss of the conserved moments stays in the cell
-    if (type[cell] == CELL_FLUID) {
-        double usq = 0.0;
-#pragma unroll
-        for (int a = 0; a < D; a++) usq += c.u[a] * c.u[a];
-        const double dm = c.rho - em.value();
-        const double dE = c.rho * (usq + ((double)D + m.K) * c.RT) - ee.value();
-        atomicAdd(Mout + cell, dm);
-#pragma unroll
-        for (int a = 0; a < D; a++) {
-            atomicAdd(Mout + (1 + a) * g.ncell + cell, c.rho * c.u[a] - ep[a].value());
-            atomicAdd(Mout + iM2<D>(a, a) * g.ncell + cell, dE / (double)D);
-        }
-    }
+    keep_shortfall32<D>(m, g, type, Mout, cell, c, em, ep, ee);
     if (q > ls.q_max) ls.q_max = q;
     ls.points += q;
     ls.walls += walls;
@@ -531,28 +573,6 @@ static __device__ __noinline__ void noslip_images(const Model& m, const Geometry
             if (kept[1] <= 0.0 && dm[1] != 0.0) atomicAdd(Mout + (long long)iG0<2>() * g.ncell + cell, dm[1]);
         }
     }
-}
-
-// Where a cell's populations land: its place in the grid.
-struct CellPlace {
-    long long cell;
-    long long lo;  // 1D: first interior cell of the instance
-    int n;         // 1D: interior length of the instance
-    int ix, iy;    // 2D: padded coordinates
-};
-
-template <int D>
-__device__ __forceinline__ CellPlace cell_place(const Geometry& g, long long cell) {
-    CellPlace p{cell, 0, 0, 0, 0};
-    if constexpr (D == 1) {
-        const int b = g.inst_of_cell[cell];
-        p.lo = g.inst_lo[b];
-        p.n = g.inst_n[b];
-    } else {
-        p.iy = (int)(cell / g.NX);
-        p.ix = (int)(cell - (long long)p.iy * g.NX);
-    }
-    return p;
 }
 
 template <int D>
@@ -672,6 +692,10 @@ __device__ __forceinline__ void scatter_cell(const Model& m, const Geometry& g, 
     ls.disp_max2 = fmax(ls.disp_max2, dmax2);
 }
 
+// Children of a row that scatter64 holds for ChildRow: two for each of at most four split points (the
+// paper's refinement radius); a row with more (refine_rad set larger) deposits them one by one.
+constexpr int kChildMax = 8;
+
 // scatter_cell in lattice form (lelbm_fp64.cuh), for a cell with a row table.
 template <int D>
 __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
@@ -696,12 +720,20 @@ __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, con
         const double hs = child ? 0.5 * c.inv_sig : c.inv_sig;
         const double ox = child ? 2.0 * lat.fx + 0.5 : lat.fx, oy = child ? 2.0 * lat.fy + 0.5 : lat.fy;
         const double w = child ? (D == 2 ? 0.25 : 0.5) : 1.0;
+        // the children of a row in order, for ChildRow (the sweep visits them from the centre out)
+        double kf[kChildMax], kg[kChildMax];
+        int k0 = 0, nk = 0;
         auto point = [&](int k, int j, double mf, double mg) {
             q++;
             // velocity in quarter cells, exact; on the lattice or a quarter off it on either side
             const int qx = child ? 4 * lat.xn - 1 + 2 * k : 4 * (lat.xn + k);
             const int qy = D == 2 ? (child ? 4 * lat.yn - 1 + 2 * j : 4 * (lat.yn + j)) : 0;
             far4 = max(far4, qx * qx + qy * qy);
+            if (child && nk > 0) {
+                kf[k - k0] = mf;
+                kg[k - k0] = mg;
+                return;
+            }
             const double cx = widen(0.25f * (float)qx), cy = D == 2 ? widen(0.25f * (float)qy) : 0.0;
             if constexpr (D == 2) {
                 if (near_wall) {
@@ -714,51 +746,39 @@ __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, con
                 }
             }
             double v[NM];
-            v[0] = mf;
-            v[1] = cx * mf;
-            if constexpr (D == 2) {
-                v[2] = cy * mf;
-                v[3] = cx * v[1];
-                v[4] = cx * v[2];
-                v[5] = cy * v[2];
-                const double e = v[3] + v[5];
-                v[6] = cx * e;
-                v[7] = cy * e;
-                v[8] = mg;
-                v[9] = cx * mg;
-                v[10] = cy * mg;
-            } else {
-                v[2] = cx * v[1];
-                v[3] = cx * v[2];
-                v[4] = mg;
-                v[5] = cx * mg;
-            }
+            stored_moments<D, true, true>(cx, cy, mf, mg, v);
             const int bx0 = qx >> 2, by0 = qy >> 2;
             if (!child) {
-                const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, bx0, by0);
-                if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) return;
-#pragma unroll
-                for (int mm = 0; mm < NM; mm++) atomicAdd(Mout + mm * g.ncell + tgt, v[mm]);
+                deposit_at<D, true, true>(g, type, Mout, at, bx0, by0, v);
                 return;
             }
-            // cloud-in-cell: along each axis 3/4 on the nearer cell, 1/4 on the other
+            // cloud-in-cell, share by share: along each axis 3/4 on the nearer cell, 1/4 on the other
             const double wx1 = (qx & 3) == 3 ? 0.75 : 0.25, wy1 = (qy & 3) == 3 ? 0.75 : 0.25;
 #pragma unroll 1
-            for (int sy = 0; sy < (D == 2 ? 2 : 1); sy++)
-#pragma unroll 1
-                for (int sx = 0; sx < 2; sx++) {
-                    double ws = sx ? wx1 : 1.0 - wx1;
-                    if constexpr (D == 2) ws *= sy ? wy1 : 1.0 - wy1;
-                    const long long tgt = land<D>(g, at.cell, at.lo, at.n, at.ix, at.iy, bx0 + sx, by0 + sy);
-                    if (tgt < 0 || !lands_on_fluid<D>(g, type, tgt)) continue;
+            for (int s4 = 0; s4 < (D == 2 ? 4 : 2); s4++) {
+                double ws = (s4 & 1) ? wx1 : 1.0 - wx1, o[NM];
+                if constexpr (D == 2) ws *= (s4 & 2) ? wy1 : 1.0 - wy1;
 #pragma unroll
-                    for (int mm = 0; mm < NM; mm++) atomicAdd(Mout + mm * g.ncell + tgt, ws * v[mm]);
-                }
+                for (int mm = 0; mm < NM; mm++) o[mm] = ws * v[mm];
+                deposit_at<D, true, true>(g, type, Mout, at, bx0 + (s4 & 1), by0 + (s4 >> 1), o);
+            }
         };
-        auto row_end = [](int) {};
+        auto row_end = [&](int j) {
+            if (!child || nk == 0) return;
+            ChildRow<D, true, true> kids;
+            kids.start();
+            const int first = lat.xn + (k0 >> 1), cy = D == 2 ? lat.yn + (j >> 1) : 0, sy = D == 2 ? ((j & 1) ? 1 : -1) : 0;
+#pragma unroll 1
+            for (int h = 0; h < nk + 3; h++)
+                kids.add(g, type, Mout, at, first, h, cy, sy, h < nk ? kf[h] : 0.0, h < nk ? kg[h] : 0.0);
+        };
         int jlo, jhi;
         lat.rows(tab, child, jlo, jhi);
-        auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
+        auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) {
+            lat.ext(tab, child, j, i0, i1, h0, h1);
+            k0 = i0;
+            nk = child && !near_wall && i1 - i0 < kChildMax ? i1 - i0 + 1 : 0;
+        };
         lattice_sweep<D>(lf, lg, true, has_g, -ox * hs, -oy * hs, hs, w * mfs, w * mgs, jlo, jhi, ext, point,
                          row_end);
     }
@@ -1127,86 +1147,53 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
     return -1;
 }
 
-// Returns true when the cell is solved and streamed; false leaves the cell, with nothing
-// of it deposited, to the FP64 EPR.  Phonons go first: their system is the smaller one, so
-// less of it stays live through the fluon passes.
+// The multipliers of a converged FP32 solve minus Eq. (IID13), for the next step, and its counts.
 template <int D>
-__device__ __forceinline__ bool df_finish(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
-                                          long long cell, BlockCounters& bc, ThreadCounters& tc, const double* conF,
-                                          const double* conG, const CellState<D>& c, const Stencil<D>& st,
-                                          const RowTable<D>& tab, float* lf32, float* lg32, bool learned,
-                                          const float2* etab, long long* bslot) {
+__device__ __forceinline__ void keep_solution32(const Model& m, const Geometry& g, long long cell, BlockCounters& bc,
+                                                const CellState<D>& c, const float* lf32, const float* lg32, int sf,
+                                                int sg) {
     constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
     const bool has_g = m.K > 0.0;
-    {
-        float cf32[NF], cg32[NG];
+    atomicAdd(&bc.hist[sf < 63 ? sf : 63], 1ull);
+    if (has_g) atomicAdd(&bc.hist[sg < 63 ? sg : 63], 1ull);
+    if (m.lam_store) {
+        const float l0 = -1.f + 0.5f * D * logf(6.2831853071795865f * c.RT32);
 #pragma unroll
-        for (int j = 0; j < NF; j++) cf32[j] = (float)conF[j];
-#pragma unroll
-        for (int j = 0; j < NG; j++) cg32[j] = (float)conG[j];
-        int sf, sg;
-        bool ok32 = solve_fg32<D>(c, st, tab, cf32, cg32, has_g, lf32, lg32, sf, sg, tc.p32);
-        if (!ok32 && learned) {
-            tc.retry++;
-            maxwell_start32<D, NF, NG>((float)c.RT, lf32, lg32);
-            ok32 = solve_fg32<D>(c, st, tab, cf32, cg32, has_g, lf32, lg32, sf, sg, tc.p32);
-        }
-        if (!ok32) return false;
-    }
-    DFStream ds;
-    ds.g = &g;
-    ds.type = type;
-    ds.Mout = Mout;
-    ds.cell = cell;
-    ds.lo = 0;
-    ds.n = 0;
-    ds.ix = ds.iy = 0;
-    ds.near_wall = false;
-    ds.beta = bslot;
-    if constexpr (D == 1) {
-        const int b = g.inst_of_cell[cell];
-        ds.lo = g.inst_lo[b];
-        ds.n = g.inst_n[b];
-    } else {
-        ds.iy = (int)(cell / g.NX);
-        ds.ix = (int)(cell - (long long)ds.iy * g.NX);
-        // Sec. III.B: trace paths past solid faces where a solid cell lies within reach
-        if (g.wall_dist)
-            ds.near_wall = (double)g.wall_dist[cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5;
-    }
-    const double xm = (double)st.R + 2.0;  // |X|, |Y| of every stencil offset from floor(u)
-    double lg[NG];
-    int ug = 0;
-    if (has_g) {
-#pragma unroll
-        for (int j = 0; j < NG; j++) lg[j] = (double)lg32[j];
-        df_split(c.rho * m.K * c.RT, ds.mh, ds.ml);
-        ug = df_population<D, false>(m, c, tab, lg, conG, etab, xm, ds, tc);
-        if (ug < 0) return false;
-    }
-    double lf[NF];
-#pragma unroll
-    for (int j = 0; j < NF; j++) lf[j] = (double)lf32[j];
-    df_split(c.rho, ds.mh, ds.ml);
-    const int uf = df_population<D, true>(m, c, tab, lf, conF, etab, xm, ds, tc);
-    if (uf < 0) {
-        if (has_g) {  // take the phonon deposit back too: the FP64 EPR streams both
-            double r[NG], rmax;
-            df_split(-(c.rho * m.K * c.RT), ds.mh, ds.ml);
-            df_pass<D, false, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lg, conG, etab, xm, r, rmax, nullptr, ds, tc.ls, tc.pdf, ds.beta);
-        }
-        return false;
-    }
-    atomicAdd(&bc.hist[uf], 1ull);
-    if (has_g) atomicAdd(&bc.hist[ug], 1ull);
-    if (m.lam_store) {  // the converged multipliers minus Eq. (IID13), as FP32 corrections
-        const float l0 = (float)maxwell_l0<D>(c.RT);
-#pragma unroll
-        for (int j = 0; j < NF; j++) m.lam_store[(long long)j * g.ncell + cell] = (float)lf[j] - start_base<D>(j, l0);
+        for (int j = 0; j < NF; j++) m.lam_store[(long long)j * g.ncell + cell] = lf32[j] - start_base<D>(j, l0);
 #pragma unroll
         for (int j = 0; j < NG; j++)
-            m.lam_store[(long long)(NF + j) * g.ncell + cell] = has_g ? (float)lg[j] - start_base<D>(j, l0) : 0.f;
+            m.lam_store[(long long)(NF + j) * g.ncell + cell] = has_g ? lg32[j] - start_base<D>(j, l0) : 0.f;
     }
+}
+
+// The FP32 path's cells near a wall or without a row table, out of line.  Returns false when the
+// FP32 solve failed (nothing is deposited).
+template <int D>
+static __device__ __noinline__ bool fp32_cell_general(const Model& m, const Geometry& g, const uint8_t* type,
+                                                      double* Mout, long long cell, BlockCounters* bc,
+                                                      ThreadCounters* tc, const float* conF, const float* conG,
+                                                      const CellState<D>& c, const Stencil<D>& st,
+                                                      const RowTable<D>& tab, const float* lf_start,
+                                                      const float* lg_start, bool learned) {
+    constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
+    const bool has_g = m.K > 0.0;
+    float lf32[NF], lg32[NG];
+#pragma unroll
+    for (int j = 0; j < NF; j++) lf32[j] = lf_start[j];
+#pragma unroll
+    for (int j = 0; j < NG; j++) lg32[j] = lg_start[j];
+    int sf, sg;
+    bool ok32;
+    for (;;) {
+        ok32 = solve_fg32<D>(c, st, tab, conF, conG, has_g, lf32, lg32, sf, sg, tc->p32);
+        if (ok32 || !learned) break;
+        tc->retry++;
+        maxwell_start32<D, NF, NG>(c.RT32, lf32, lg32);
+        learned = false;
+    }
+    if (!ok32) return false;
+    keep_solution32<D>(m, g, cell, *bc, c, lf32, lg32, sf, sg);
+    scatter_cell32<D>(m, g, type, Mout, cell, c, st, tab, lf32, lg32, tc->ls);
     return true;
 }
 
@@ -1272,7 +1259,8 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
                                             const double* __restrict__ Min, double* Mout,
                                             DevStats* stats, long long cell, BlockCounters& bc, ThreadCounters& tc,
                                             Con<PREC>* conF, Con<PREC>* conG, const CellState<D>& c, const Stencil<D>& st,
-                                            const float* dl, char2* rowbuf, const float2* etab, long long* bslot) {
+                                            const float* dl, char2* rowbuf) {
+    static_assert(PREC != PREC_MIXED, "the mixed path steps cells in phases (mixed_block)");
     constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
     tc.cells++;
     const bool has_g = m.K > 0.0;
@@ -1367,26 +1355,27 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
         tab.build(c, st, rowbuf);
     if constexpr (PREC == PREC_FP32) {
         // FP32 Newton and FP32 streaming; the plain FP64 EPR is the fallback
-        bool ok32 = solve_fg32<D>(c, st, tab, conF, conG, has_g, lf32, lg32, sf, sg, tc.p32);
-        if (!ok32 && learned) {
-            tc.retry++;
-            maxwell_start32<D, NF, NG>(c.RT32, lf32, lg32);
-            learned = false;
-            ok32 = solve_fg32<D>(c, st, tab, conF, conG, has_g, lf32, lg32, sf, sg, tc.p32);
+        bool near_wall = false;  // as in scatter_cell32
+        if constexpr (D == 2) {
+            if (g.wall_dist)
+                near_wall = (double)g.wall_dist[cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5;
         }
-        if (ok32) {
-            atomicAdd(&bc.hist[sf < 63 ? sf : 63], 1ull);
-            if (has_g) atomicAdd(&bc.hist[sg < 63 ? sg : 63], 1ull);
-            if (m.lam_store) {  // the converged multipliers minus Eq. (IID13), for the next step
-                const float l0 = -1.f + 0.5f * D * logf(6.2831853071795865f * c.RT32);
-#pragma unroll
-                for (int j = 0; j < NF; j++)
-                    m.lam_store[(long long)j * g.ncell + cell] = lf32[j] - start_base<D>(j, l0);
-#pragma unroll
-                for (int j = 0; j < NG; j++)
-                    m.lam_store[(long long)(NF + j) * g.ncell + cell] = has_g ? lg32[j] - start_base<D>(j, l0) : 0.f;
+        if (tab.ok && !near_wall) {
+            bool ok32;
+#pragma unroll 1
+            for (;;) {
+                ok32 = solve_fg32<D, true>(c, st, tab, conF, conG, has_g, lf32, lg32, sf, sg, tc.p32);
+                if (ok32 || !learned) break;
+                tc.retry++;
+                maxwell_start32<D, NF, NG>(c.RT32, lf32, lg32);
+                learned = false;
             }
-            scatter_cell32<D>(m, g, type, Mout, cell, c, st, tab, lf32, lg32, tc.ls);
+            if (ok32) {
+                keep_solution32<D>(m, g, cell, bc, c, lf32, lg32, sf, sg);
+                scatter_table32<D>(m, g, type, Mout, cell, c, tab, lf32, lg32, tc.ls);
+                return;
+            }
+        } else if (fp32_cell_general<D>(m, g, type, Mout, cell, &bc, &tc, conF, conG, c, st, tab, lf32, lg32, learned)) {
             return;
         }
         // the plain FP64 EPR, out of line: it is rare, and inline it would shape the
@@ -1395,17 +1384,6 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
         const TailCounts t = fp64_tail_cold<D>(m, g, type, Mout, stats, cell, &bc, conF, conG, c, st);
         add_tail(tc, t);
     } else {
-        if constexpr (PREC == PREC_MIXED) {
-            // FP32 Newton, double-float correction and streaming judged at the FP64
-            // tolerance; the FP64 EPR (out of line) takes the cells it leaves
-            if (tab.ok && df_finish<D>(m, g, type, Mout, cell, bc, tc, conF, conG, c, st, tab, lf32, lg32, learned,
-                                       etab, bslot))
-                return;
-            tc.redo++;
-            const TailCounts t = fp64_cell_cold<D>(m, g, type, Min, Mout, stats, cell, &bc, conF, conG);
-            add_tail(tc, t);
-            return;
-        }
         fp64_cell<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), bc, tc, conF, conG, c, st, tab, lf, lg, learned);
     }
 }
@@ -1434,11 +1412,14 @@ static __device__ __noinline__ bool fp32_phase(const RowTable<D>& tab_in, const 
     }
     unsigned int np = 0;
     int sf, sg;
-    bool ok = solve_fg32<D, true>(c, st, tab, cf32, cg32, has_g, lf32, lg32, sf, sg, np);
-    if (!ok && learned) {
+    bool ok;
+#pragma unroll 1
+    for (;;) {  // one code site for the learned start and its retry from Eq. (IID13)
+        ok = solve_fg32<D, true>(c, st, tab, cf32, cg32, has_g, lf32, lg32, sf, sg, np);
+        if (ok || !learned) break;
         retry++;
         maxwell_start32<D, NF, NG>(rt32, lf32, lg32);
-        ok = solve_fg32<D, true>(c, st, tab, cf32, cg32, has_g, lf32, lg32, sf, sg, np);
+        learned = false;
     }
     np32 += np;
 #pragma unroll
@@ -1553,22 +1534,14 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
     ds.g = &g;
     ds.type = type;
     ds.Mout = Mout;
-    ds.cell = cell;
-    ds.lo = 0;
-    ds.n = 0;
-    ds.ix = ds.iy = 0;
+    ds.at = CellPlace{cell, 0, 0, 0, 0};
     ds.near_wall = false;
     ds.beta = bslot;
     ds.mh = ds.ml = 0.f;
     double xm = 0.0;
     if (alive) {
-        if constexpr (D == 1) {
-            const int b = g.inst_of_cell[cell];
-            ds.lo = g.inst_lo[b];
-            ds.n = g.inst_n[b];
-        } else {
-            ds.iy = (int)(cell / g.NX);
-            ds.ix = (int)(cell - (long long)ds.iy * g.NX);
+        ds.at = cell_place<D>(g, cell);
+        if constexpr (D == 2) {
             // Sec. III.B: trace paths past solid faces where a solid cell lies within reach
             if (g.wall_dist)
                 ds.near_wall = (double)g.wall_dist[cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5;
@@ -1683,23 +1656,20 @@ __global__ void __launch_bounds__(cell_threads<PREC>(), min_blocks<D, PREC>()) c
             mixed_block<D, false>(m, g, type, Min, Mout, stats, cell, active, bc, tc, conF, conG, rowbuf, s_exp,
                                   s_beta[threadIdx.x], nullptr, false, grp, G);
         }
-        counters_flush(bc, tc, stats);
-        return;
-    }
-    for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(work, 32ull);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (base >= (unsigned long long)g.ncell) break;
-        const long long cell = (long long)base + lane;
-        const bool active = cell < g.ncell && type[cell] != CELL_SOLID;
-        CellState<D> c;
-        Stencil<D> st;
-        bool ok = false;
-        if (active) ok = prepare_cell<D, PREC>(m, g, Min, stats, cell, bc, c, st);
-        if (ok)
-            finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr, rowbuf, s_exp,
-                                 PREC == PREC_MIXED ? s_beta[threadIdx.x] : nullptr);
+    } else {
+        for (;;) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(work, 32ull);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (base >= (unsigned long long)g.ncell) break;
+            const long long cell = (long long)base + lane;
+            const bool active = cell < g.ncell && type[cell] != CELL_SOLID;
+            CellState<D> c;
+            Stencil<D> st;
+            bool ok = false;
+            if (active) ok = prepare_cell<D, PREC>(m, g, Min, stats, cell, bc, c, st);
+            if (ok) finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr, rowbuf);
+        }
     }
     counters_flush(bc, tc, stats);
 }
@@ -1805,7 +1775,7 @@ __global__ void __launch_bounds__(128, batch_min_blocks<PREC>()) batch_persisten
                                          s_exp, s_beta[threadIdx.x], s_mlp, mlp, 0, (int)blockDim.x);
                 }
             }
-            for (; PREC != PREC_MIXED;) {
+            if constexpr (PREC != PREC_MIXED) for (;;) {
                 unsigned int base = 0;
                 if (lane == 0) base = atomicAdd(&s_next, 32u);
                 base = __shfl_sync(0xffffffffu, base, 0);
@@ -1827,7 +1797,7 @@ __global__ void __launch_bounds__(128, batch_min_blocks<PREC>()) batch_persisten
                 }
                 if (ok)
                     finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st,
-                                         use_mlp ? dl : nullptr, nullptr, s_exp, PREC == PREC_MIXED ? s_beta[threadIdx.x] : nullptr);
+                                         use_mlp ? dl : nullptr, nullptr);
             }
             counters_to_block(bc, tc);  // keeps the 32-bit tallies of a long launch small
             __syncthreads();

@@ -33,6 +33,76 @@ __device__ __forceinline__ float narrow(double v) {
     return hi < 0x38100000u ? 0.f : (hi >= 0x47f00000u ? __int_as_float(0x7f800000) : f);
 }
 
+// ---------------------------------------------------------------------------
+// exp(x) in FP64 with integer instructions: Tang's table-driven method (ACM TOMS 15, 1989) in 64-bit
+// fixed point.  x log2(e) = n + j / 512 + rho, 2^(j/512) from a table, 2^rho from five Taylor terms.
+// Every step carries at least 59 bits, so the result is rounded once (0.6 ulp at most).  About 70
+// integer instructions, some 20 issue cycles of an SM, where the library's exp takes about 17 FP64
+// instructions, 16 cycles each.
+// ---------------------------------------------------------------------------
+struct Exp2Table {
+    unsigned long long t[512];  // 2^(j/512), 62 fractional bits
+    // floor(sqrt(x 2^63)) for x with 63 fractional bits in [1, 2)
+    static constexpr unsigned long long root(unsigned long long x) {
+        unsigned long long y = 0;
+        const unsigned __int128 v = (unsigned __int128)x << 63;
+        for (int b = 63; b >= 0; b--) {
+            const unsigned long long c = y | (1ull << b);
+            if ((unsigned __int128)c * c <= v) y = c;
+        }
+        return y;
+    }
+    constexpr Exp2Table() : t{} {
+        unsigned long long r[9] = {};  // 2^(1/2), 2^(1/4), ..., 2^(1/512), 63 fractional bits
+        unsigned __int128 two = (unsigned __int128)2 << 126;  // sqrt(2): from 2 with 126 fractional bits
+        for (int b = 63; b >= 0; b--) {
+            const unsigned long long c = r[0] | (1ull << b);
+            if ((unsigned __int128)c * c <= two) r[0] = c;
+        }
+        for (int k = 1; k < 9; k++) r[k] = root(r[k - 1]);
+        for (int j = 0; j < 512; j++) {
+            unsigned long long p = 1ull << 63;
+            for (int k = 0; k < 9; k++)
+                if ((j >> (8 - k)) & 1) p = (unsigned long long)(((unsigned __int128)p * r[k]) >> 63);
+            t[j] = p >> 1;
+        }
+    }
+};
+static __device__ const Exp2Table c_exp2 = Exp2Table();
+
+// 2^(w 2^-55) = P 2^(n - 62), P in [2^62, 2^63].
+__device__ __forceinline__ unsigned long long exp2_q62(long long w, int& n) {
+    const int hi = (int)(w >> 32);
+    n = hi >> 23;
+    const unsigned long long T = __ldg(&c_exp2.t[(hi >> 14) & 511]);
+    const unsigned long long L = __umul64hi((unsigned long long)w << 18, 0xB17217F7D1CF79ACull);  // 512 rho ln 2
+    const unsigned l = (unsigned)(L >> 32);
+    const unsigned long long q2 = __umul64hi(L, L);
+    const unsigned q3 = __umulhi((unsigned)(q2 >> 32), l), q4 = __umulhi(q3, l), q5 = __umulhi(q4, l);
+    // rho ln 2 = L / 512: the terms L/2^9, L^2/2^19, L^3/(6 2^27), L^4/(24 2^36) and (to a few per cent)
+    // L^5/(120 2^45), with 64 fractional bits
+    const unsigned long long e = (L >> 9) + (q2 >> 19) + ((unsigned long long)__umulhi(q3, 0xAAAAAAABu) << 3) +
+                                 (__umulhi(q4, 0xAAAAAAABu) >> 8) + (q5 >> 20);
+    return T + __umul64hi(T, e);
+}
+
+__device__ __forceinline__ double exp_int(double x) {
+    const int xh = __double2hiint(x);
+    const int ex = (xh >> 20) & 0x7ff;
+    if (ex >= 1023 + 7) return exp(x);  // |x| >= 128, infinite or NaN
+    // |x| log2(e) with 55 fractional bits
+    const unsigned long long m =
+        ((unsigned long long)((xh & 0xfffff) | (ex ? 0x100000 : 0)) << 43) | ((unsigned long long)(unsigned)__double2loint(x) << 11);
+    const unsigned long long p = __umul64hi(m, 0xB8AA3B295C17F0BCull);  // mantissa x log2(e) / 2, 63 bits below the point
+    const int sh = 1023 + 7 - ex;                                       // >= 1: p holds |x| log2(e) 2^(62 - (ex - 1023))
+    unsigned long long w = sh < 64 ? (((p >> (sh - 1)) + 1) >> 1) : 0ull;
+    const long long ws = xh < 0 ? -(long long)w : (long long)w;
+    int n;
+    const unsigned long long P = exp2_q62(ws, n) + 512;  // round to 53 bits
+    // P = 2^62 + ...: adding it above the exponent field carries its leading one into the exponent
+    return __longlong_as_double((long long)(P >> 10) + ((long long)(n + 1022) << 52));
+}
+
 // Coefficients d[ix(a, b)] of k^a j^b in the exponent 1 + sum_j lam_j T_j at the thermal points
 // (x0 + k h, y0 + j h).
 template <int D, bool FLUON>
@@ -84,32 +154,62 @@ struct SweepFactors {
 
     __device__ __forceinline__ void init(const double* p, double wgt) {
         using Q = DFPop<D, FLUON>;
+        constexpr int NE = FLUON ? (D == 1 ? 6 : 17) : (D == 1 ? 4 : 9);
+        double a[NE];
         const double p10 = p[Q::ix(1, 0)], p20 = p[Q::ix(2, 0)];
         const double p30 = FLUON ? p[FLUON ? Q::ix(3, 0) : 0] : 0.0;
-        e0 = wgt * exp(-p[0]);
-        r = exp(-(p10 + p20 + p30));
-        l = exp(p10 - p20 + p30);
-        r2 = exp(-(2.0 * p20 + 6.0 * p30));
+        a[0] = p[0];
+        a[1] = p10 + p20 + p30;
+        a[2] = p20 - p10 - p30;
+        a[3] = 2.0 * p20 + 6.0 * p30;
         if constexpr (FLUON) {
-            r3 = exp(-6.0 * p30);
-            l3 = 1.0 / r3;
+            a[4] = 6.0 * p30;
+            a[5] = -a[4];
         }
         if constexpr (D == 2) {
+            constexpr int o = FLUON ? 6 : 4;
             const double p01 = p[Q::ix(0, 1)], p02 = p[Q::ix(0, 2)];
             const double p03 = FLUON ? p[FLUON ? Q::ix(0, 3) : 0] : 0.0;
-            u = exp(-(p01 + p02 + p03));
-            ud = exp(p01 - p02 + p03);
-            u2 = exp(-(2.0 * p02 + 6.0 * p03));
-            m11 = exp(-p[Q::ix(1, 1)]);
-            i11 = 1.0 / m11;
+            a[o] = p01 + p02 + p03;
+            a[o + 1] = p02 - p01 - p03;
+            a[o + 2] = 2.0 * p02 + 6.0 * p03;
+            a[o + 3] = p[Q::ix(1, 1)];
+            a[o + 4] = -a[o + 3];
             if constexpr (FLUON) {
-                u3 = exp(-6.0 * p03);
-                u3d = 1.0 / u3;
+                a[11] = 6.0 * p03;
+                a[12] = -a[11];
+                a[13] = p[Q::ix(1, 2)];
+                a[14] = -a[13];
+                a[15] = p[Q::ix(2, 1)];
+                a[16] = -a[15];
+            }
+        }
+        // one code site: inlined copies would crowd the instruction caches
+#pragma unroll 1
+        for (int k = 0; k < NE; k++) a[k] = exp_int(-a[k]);
+        e0 = wgt * a[0];
+        r = a[1];
+        l = a[2];
+        r2 = a[3];
+        if constexpr (FLUON) {
+            r3 = a[4];
+            l3 = a[5];
+        }
+        if constexpr (D == 2) {
+            constexpr int o = FLUON ? 6 : 4;
+            u = a[o];
+            ud = a[o + 1];
+            u2 = a[o + 2];
+            m11 = a[o + 3];
+            i11 = a[o + 4];
+            if constexpr (FLUON) {
+                u3 = a[11];
+                u3d = a[12];
                 u2d = u2 * (u3d * u3d);
-                m12 = exp(-p[Q::ix(1, 2)]);
-                i12 = 1.0 / m12;
-                m21 = exp(-p[Q::ix(2, 1)]);
-                i21 = 1.0 / m21;
+                m12 = a[13];
+                i12 = a[14];
+                m21 = a[15];
+                i21 = a[16];
             }
         }
     }

@@ -776,7 +776,7 @@ __device__ __forceinline__ int own_monomials(int lane, int* ma, int* mb, int* mc
 // fallback, of the equilibrium: omega = 1).
 __device__ __forceinline__ void start3(Warp3* w, const CellState<3>& c, bool equilibrium, int lane) {
     double lf[kNF3], lg[kNG3];
-    maxwell_start_fg<3, kNF3, kNG3>(c.RT, lf, lg);
+    maxwell_start_newton<3, kNF3, kNG3>(c.RT, lf, lg);
     if (lane < kNF3) {
         w->lf[lane] = lf[lane];
         double v = c.cf[lane];

@@ -305,7 +305,6 @@ extern "C" int lelbm_create(lelbm_t* out, const lelbm_params* p) {
     Model& m = h->model;
     m.lam_store = nullptr;
     m.K = p->K;
-    m.inv_dk = 1.0 / ((double)D + p->K);
     m.nu_s = p->nu_shear;
     m.nu_b = p->nu_bulk;
     m.Pr = p->prandtl;
@@ -317,7 +316,7 @@ extern "C" int lelbm_create(lelbm_t* out, const lelbm_params* p) {
     m.max_refine = p->max_refine;
     m.tol = p->tol;
     m.max_iter = p->max_newton;
-    set_fp32_params(m);
+    set_derived_params(m, D);
 
     Geometry& g = h->geo;
     g.D = D;

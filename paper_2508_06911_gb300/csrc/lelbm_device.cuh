@@ -48,6 +48,64 @@ __device__ __forceinline__ constexpr int iG1(int g) {
 }
 
 // ---------------------------------------------------------------------------
+// FP32 <-> FP64 bit helpers (integer operations only; GB300's FP64 pipe also runs
+// the FP32 <-> FP64 conversion instructions).
+// ---------------------------------------------------------------------------
+// Subnormals become zero.
+__device__ __forceinline__ float flush_sub(float v) { return (__float_as_uint(v) & 0x7f800000u) ? v : 0.f; }
+
+// FP32 -> FP64: the exponent is rebiased from 127 to 1023 by one addition and the
+// mantissa shifted into place.  Normal numbers widen exactly; zeros and subnormals give
+// zero.  Infinities and NaNs, which a converged solve does not produce, come out finite.
+__device__ __forceinline__ double widen(float v) {
+    const unsigned int b = __float_as_uint(v);
+    const bool tiny = (b & 0x7f800000u) == 0u;
+    const unsigned int hi = (((b >> 3) & 0x0fffffffu) + 0x38000000u) | (b & 0x80000000u);
+    return __hiloint2double(tiny ? 0 : (int)hi, tiny ? 0 : (int)(b << 29));
+}
+
+// FP64 -> FP32 by truncation with integer operations (the conversion instruction runs on the
+// FP64 pipe).  Positive normal values; below 2^-126 zero, from 2^128 on (and NaN) infinity.
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    const float f = __uint_as_float(__funnelshift_l(lo, hi - 0x38000000u, 3));
+    return hi < 0x38100000u ? 0.f : (hi >= 0x47f00000u ? __int_as_float(0x7f800000) : f);
+}
+
+// The same of any sign.
+__device__ __forceinline__ float narrow_signed(double v) {
+    const float a = narrow(__hiloint2double(__double2hiint(v) & 0x7fffffff, __double2loint(v)));
+    return __double2hiint(v) < 0 ? -a : a;
+}
+
+// Largest of |v| and worst as integers, ordered as the doubles are with NaN above infinity.
+__device__ __forceinline__ long long max_abs_bits(double v, long long worst) {
+    const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+    return b > worst ? b : worst;
+}
+constexpr long long kInfBits = 0x7ff0000000000000LL;
+
+// ---------------------------------------------------------------------------
+// Reciprocals and quotients.  The library's FP64 division takes about nine instructions of the FP64
+// pipe; a reciprocal from the FP32 one and two Newton steps takes four (24 -> 48 -> 53 bits, within
+// one ulp), and a quotient by a divisor whose reciprocal is known three (Markstein's correction, correctly
+// rounded like __ddiv_rn).
+// ---------------------------------------------------------------------------
+// Is v positive, normal and within 2^+-99, the range of the short forms?
+__device__ __forceinline__ bool recip_range(double v) { return (unsigned)(__double2hiint(v) >> 20) - 924u < 198u; }
+__device__ __forceinline__ double recip64(double v) {
+    if (!recip_range(v)) return 1.0 / v;
+    double y = widen(__fdividef(1.f, narrow(v)));
+    y = __fma_rn(y, __fma_rn(-v, y, 1.0), y);
+    return __fma_rn(y, __fma_rn(-v, y, 1.0), y);
+}
+// a / b for y = recip64(b), recip_range(b) (or y = RN(1 / b))
+__device__ __forceinline__ double quotient(double a, double b, double y) {
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-q, b, a), y, q);
+}
+
+// ---------------------------------------------------------------------------
 // Collision module: Eq. (IIB6), (IIB9)-(IIB18), App. C (C7)-(C8), App. D.
 // ---------------------------------------------------------------------------
 template <int D>
@@ -63,50 +121,54 @@ struct CellState {
 // Eq. (IIB6), with the operation order of a plain loop and one rounding each: rho, u, RT
 // and whether they describe a gas (rho > 0, RT > 0, finite).  usq receives |u|^2.
 template <int D>
-__device__ __forceinline__ bool cell_macros(const double* M, double K, double& rho, double* u, double& RT,
+__device__ __forceinline__ bool cell_macros(const double* M, const Model& m, double& rho, double* u, double& RT,
                                             double& usq) {
     rho = M[0];
+    const bool quick = recip_range(rho);
+    const double y = quick ? recip64(rho) : 0.0;
+    auto over_rho = [&](double a) { return quick ? quotient(a, rho, y) : __ddiv_rn(a, rho); };
     usq = 0.0;
     double tr = 0.0;
 #pragma unroll
     for (int a = 0; a < D; a++) {
-        u[a] = __ddiv_rn(M[1 + a], rho);
+        u[a] = over_rho(M[1 + a]);
         usq = __dadd_rn(usq, __dmul_rn(u[a], u[a]));
         tr = __dadd_rn(tr, M[iM2<D>(a, a)]);
     }
-    RT = __ddiv_rn(__dsub_rn(__ddiv_rn(__dadd_rn(tr, M[iG0<D>()]), rho), usq), __dadd_rn((double)D, K));
+    RT = quotient(__dsub_rn(over_rho(__dadd_rn(tr, M[iG0<D>()])), usq), __dadd_rn((double)D, m.K), m.inv_dk);
     return rho > 0.0 && RT > 0.0 && isfinite(rho) && isfinite(RT);
 }
 
 template <int D>
 __device__ __forceinline__ void collide(const double* M, const Model& m, CellState<D>& c) {
-    constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
+    constexpr int NG = Dim<D>::NG;
     const double K = m.K;
     double rho, RT, usq;
-    c.ok = cell_macros<D>(M, K, rho, c.u, RT, usq);
+    c.ok = cell_macros<D>(M, m, rho, c.u, RT, usq);
     c.rho = rho;
     c.RT = RT;
     if (!c.ok) return;
     c.sig = sqrt(RT);
-    c.inv_sig = 1.0 / c.sig;
+    c.inv_sig = recip64(c.sig);
 
     // Eq. (IIB9): non-equilibrium central moments.
     double P[D][D];
-#pragma unroll
-    for (int a = 0; a < D; a++)
-#pragma unroll
-        for (int b = 0; b < D; b++)
-            P[a][b] = M[iM2<D>(a, b)] - rho * (c.u[a] * c.u[b] + (a == b ? RT : 0.0));
     double trP = 0.0;
 #pragma unroll
-    for (int a = 0; a < D; a++) trP += P[a][a];
+    for (int a = 0; a < D; a++) {
+#pragma unroll
+        for (int b = a; b < D; b++)
+            P[a][b] = P[b][a] = M[iM2<D>(a, b)] - rho * (c.u[a] * c.u[b] + (a == b ? RT : 0.0));
+        trP += P[a][a];
+    }
     double Q[D];
+    const double e3 = rho * (usq + (D + 2) * RT);
 #pragma unroll
     for (int g = 0; g < D; g++) {
         double s = 0.0;
 #pragma unroll
         for (int a = 0; a < D; a++) s += c.u[a] * P[a][g];
-        Q[g] = M[iMD<D>(g)] - 2.0 * s - c.u[g] * trP - rho * (usq + (D + 2) * RT) * c.u[g];
+        Q[g] = M[iMD<D>(g)] - 2.0 * s - c.u[g] * trP - e3 * c.u[g];
     }
     const double G0 = M[iG0<D>()];
     const double G0n = G0 - rho * K * RT;
@@ -115,26 +177,25 @@ __device__ __forceinline__ void collide(const double* M, const Model& m, CellSta
     for (int g = 0; g < D; g++) Gn[g] = M[iG1<D>(g)] - c.u[g] * G0;
 
     // App. C: implicit collision frequencies from the kinematic coefficients.
-    const double inv_f = m.nu_s / RT + 0.5;
-    double wf = 1.0 / inv_f;
-    const double fb = 2.0 / D - 2.0 / (D + K);
-    double wb = (m.nu_b < 0.0 || fb <= 0.0) ? 1.0 : 1.0 / (m.nu_b / (RT * fb) + 0.5);
-    double wh = 1.0 / ((inv_f - 0.5) / m.Pr + 0.5);
+    const double iRT = recip64(RT);
+    const double irr = recip64(rho) * iRT;  // 1 / (rho RT)
+    const double inv_f = m.nu_s * iRT + 0.5;
+    double wf = recip64(inv_f);
+    double wb = m.nu_b_over < 0.0 ? 1.0 : recip64(m.nu_b_over * iRT + 0.5);
+    double wh = recip64((inv_f - 0.5) * m.inv_Pr + 0.5);
 
     // App. D: Knudsen number (moments normalised by rho) and limiter.
     if (m.limiter) {
-        double s2 = 0.0, s3 = 0.0;
-        const double ir = 1.0 / rho;
+        double s2 = fabs(G0n), s3 = 0.0;
 #pragma unroll
         for (int a = 0; a < D; a++)
 #pragma unroll
-            for (int b = 0; b < D; b++) s2 += fabs(P[a][b] * ir);
-        s2 += fabs(G0n * ir);
+            for (int b = 0; b < D; b++) s2 += fabs(P[a][b]);
 #pragma unroll
-        for (int g = 0; g < D; g++) s3 += fabs(Q[g] * ir) + fabs(Gn[g] * ir);
-        const double k2 = s2 / ((D + K) * RT);
-        const double k3 = s3 / ((D + K + 2) * RT * c.sig);
-        const double Kn = fmax(k2, k3);
+        for (int g = 0; g < D; g++) s3 += fabs(Q[g]) + fabs(Gn[g]);
+        const double k2 = s2 * (irr * m.inv_dk);
+        const double k3 = s3 * (irr * c.inv_sig * m.inv_dk2);
+        const double Kn = k2 > k3 ? k2 : k3;
         if (Kn > 0.01) {  // below 0.01 the limiter leaves omega unchanged
             const double ks = log10(Kn);
             if (ks >= -1.0) {
@@ -149,9 +210,7 @@ __device__ __forceinline__ void collide(const double* M, const Model& m, CellSta
     }
 
     // Eq. (IIB10)-(IIB18), then divided by sqrt(RT)^order (thermal units).
-    const double bulk = -G0n / D;
-    const double ir = 1.0 / rho;
-    const double iRT = 1.0 / RT;
+    const double bulk = -G0n * (1.0 / D);
     c.cf[0] = 1.0;
 #pragma unroll
     for (int a = 0; a < D; a++) c.cf[1 + a] = 0.0;
@@ -161,20 +220,18 @@ __device__ __forceinline__ void collide(const double* M, const Model& m, CellSta
 #pragma unroll
         for (int b = a; b < D; b++) {
             const double sh = P[a][b] - (a == b ? bulk : 0.0);
-            const double mm = (a == b ? rho * RT : 0.0) + (1.0 - wf) * sh + (1.0 - wb) * (a == b ? bulk : 0.0);
-            c.cf[j++] = mm * ir * iRT;
+            const double mm = (1.0 - wf) * sh + (1.0 - wb) * (a == b ? bulk : 0.0);
+            c.cf[j++] = mm * irr + (a == b ? 1.0 : 0.0);
         }
-    const double s3 = iRT * c.inv_sig;
+    const double s3 = (1.0 - wh) * (irr * c.inv_sig);
 #pragma unroll
     for (int g = 0; g < D; g++)
 #pragma unroll
-        for (int a = 0; a < D; a++) c.cf[j++] = (1.0 - wh) * ((1.0 + 2.0 * (a == g)) / (D + 2) * Q[g]) * ir * s3;
-    (void)NF;
+        for (int a = 0; a < D; a++) c.cf[j++] = ((1.0 + 2.0 * (a == g)) / (D + 2)) * Q[g] * s3;
     if (K > 0.0) {
-        const double nrm = 1.0 / (rho * K * RT);
-        c.cg[0] = (rho * K * RT + (1.0 - wb) * G0n) * nrm;
+        c.cg[0] = (1.0 - wb) * G0n * (irr * m.inv_K) + 1.0;
 #pragma unroll
-        for (int g = 0; g < D; g++) c.cg[1 + g] = (1.0 - wh) * Gn[g] * nrm * c.inv_sig;
+        for (int g = 0; g < D; g++) c.cg[1 + g] = Gn[g] * (s3 * m.inv_K);
         int k = 1 + D;
 #pragma unroll
         for (int a = 0; a < D; a++)
@@ -391,22 +448,27 @@ struct Stencil {
     int Nr;          // refinement levels
     double rad2[5];  // squared refinement radius of level 1..4 (index = level)
 
+    // R_ac and N_r round half away from zero; FP32 decides unless the value lies close to a
+    // half-integer, where the FP64 expression does.
     __device__ __forceinline__ void init(const CellState<D>& c, const Model& m) {
 #pragma unroll
         for (int a = 0; a < D; a++) u[a] = c.u[a];
-        double r = round(__dmul_rn(m.n_conf, c.sig));
-        if (r < m.r_min) r = m.r_min;
-        R = (int)r;
-        const double rr = (double)R + 0.5;
-        rr2 = rr * rr;
-        double nr = round(__ddiv_rn(1.0, __dmul_rn(m.refine_div, c.sig)));
-        if (nr > (double)m.max_refine) nr = (double)m.max_refine;
-        Nr = (int)nr;
-#pragma unroll
-        for (int L = 0; L < 5; L++) {
-            const double rad = m.refine_rad * ldexp(1.0, -L);
-            rad2[L] = rad * rad;
+        const float sf = narrow(c.sig);
+        const float x = m.n_conf32 * sf, xr = floorf(x + 0.5f);
+        R = (int)xr;
+        if (!(x < 1000.f) || fabsf(x - xr) > 0.499f) R = (int)round(__dmul_rn(m.n_conf, c.sig));
+        if (R < m.r_min_up) R = (int)m.r_min;
+        const float rr = (float)R + 0.5f;
+        rr2 = R < 2000 ? widen(rr * rr) : ((double)R + 0.5) * ((double)R + 0.5);  // exact in FP32
+        const float v = __fdividef(1.f, m.refine_div32 * sf), vr = floorf(v + 0.5f);
+        Nr = v < 1000.f ? (int)vr : 1000;
+        if (fabsf(v - vr) > 0.499f) {
+            const double nr = round(__ddiv_rn(1.0, __dmul_rn(m.refine_div, c.sig)));
+            Nr = nr < 1000.0 ? (int)nr : 1000;
         }
+        if (Nr > m.max_refine) Nr = m.max_refine;
+#pragma unroll
+        for (int L = 0; L < 5; L++) rad2[L] = m.rad2[L];
     }
 
     // The same set-up in FP32 for the FP32 path (R_ac and N_r differ from the FP64
@@ -877,6 +939,25 @@ __device__ __forceinline__ void maxwell_start_fg(double RT, double* lf, double* 
 #pragma unroll
     for (int j = 0; j < NGv; j++) lg[j] = 0.0;
     lf[0] = lg[0] = l0;
+    int j = 1 + D;
+#pragma unroll
+    for (int a = 0; a < D; a++)
+#pragma unroll
+        for (int b = a; b < D; b++) {
+            lf[j] = lg[j] = (a == b) ? 0.5 : 0.0;
+            j++;
+        }
+}
+
+// The same with its logarithm in FP32, as the start of a Newton iteration (which it only steers).
+template <int D, int NFv, int NGv>
+__device__ __forceinline__ void maxwell_start_newton(double RT, double* lf, double* lg) {
+    const float l0 = -1.f + 0.5f * D * logf(6.2831853071795865f * narrow(RT));
+#pragma unroll
+    for (int j = 0; j < NFv; j++) lf[j] = 0.0;
+#pragma unroll
+    for (int j = 0; j < NGv; j++) lg[j] = 0.0;
+    lf[0] = lg[0] = widen(l0);
     int j = 1 + D;
 #pragma unroll
     for (int a = 0; a < D; a++)

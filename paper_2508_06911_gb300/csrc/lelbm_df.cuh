@@ -157,6 +157,15 @@ struct DFPop {
     __device__ __forceinline__ static constexpr int ix(int a, int b) { return D == 1 ? a : tix(a, b, P); }
 };
 
+// round(d 2^54) for |d| < 256 with integer operations (the conversion instruction runs on the FP64 pipe).
+__device__ __forceinline__ long long to_fix(double d) {
+    static_assert(kFixBits == 54, "shift");
+    const int hi = __double2hiint(d), s = ((hi >> 20) & 0x7ff) - 1021;  // d = mantissa 2^(s - 54)
+    const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(d);
+    const unsigned long long v = s >= 0 ? m << s : (s > -55 ? ((m >> (-s - 1)) + 1) >> 1 : 0ull);
+    return hi < 0 ? -(long long)v : (long long)v;
+}
+
 // Coefficients beta[ix(a, b)] of X^a Y^b in w(X, Y) = -log2(e) (1 + sum_j lam_j T_j(t)),
 // t = ((X - fx) s, (Y - fy) s), as int64 with kFixBits fractional bits; (X, Y) are the
 // lattice offsets of a velocity from (floor u_x, floor u_y), (fx, fy) = u - floor(u) and
@@ -202,18 +211,19 @@ __device__ __forceinline__ bool fix_poly(const double* lam, double s, double fx,
                     if (k < n && i >= k && i < n) d[Q::ix(a, i)] = fma(-fy, d[Q::ix(a, i + 1)], d[Q::ix(a, i)]);
         }
     }
-    double bound = 0.0;
-    double xp[P + 1];
-    xp[0] = 1.0;
+    float bound = 0.f;
+    const float xf = (float)xm;
+    float xp[P + 1];
+    xp[0] = 1.f;
 #pragma unroll
-    for (int k = 1; k <= P; k++) xp[k] = xp[k - 1] * xm;
+    for (int k = 1; k <= P; k++) xp[k] = xp[k - 1] * xf;
 #pragma unroll
     for (int b = 0; b <= (D == 2 ? P : 0); b++)
 #pragma unroll
-        for (int a = 0; a + b <= P; a++) bound += fabs(d[Q::ix(a, b)]) * xp[a] * xp[b];
-    if (!(bound < kFixBound)) return false;
+        for (int a = 0; a + b <= P; a++) bound += fabsf(narrow_signed(d[Q::ix(a, b)])) * (xp[a] * xp[b]);
+    if (!(bound < (float)kFixBound)) return false;
 #pragma unroll
-    for (int k = 0; k < NB; k++) beta[k] = __double2ll_rn(d[k] * kFixOne);
+    for (int k = 0; k < NB; k++) beta[k] = to_fix(d[k]);
     return true;
 }
 
@@ -266,19 +276,26 @@ __device__ __forceinline__ long long fix_child_w(const long long* B, int m) {
     return v;
 }
 
-// Moments K_i = sum_a C(i, a) (-h)^(i - a) L_a of a distribution about a new origin h.
-template <int P>
-__device__ __forceinline__ void origin_shift(const double* L, double h, double* K) {
+// Moments L[ix(a, b)] = sum X^a Y^b f (degree <= P) of a distribution to those about (hx, hy), in place: the
+// transposed Taylor shift, P (P + 1) / 2 FMAs for a column of degree P.
+template <int D, int P>
+__device__ __forceinline__ void moments_about(double* L, double hx, double hy) {
+    auto ix = [](int a, int b) { return D == 1 ? a : tix(a, b, P); };
 #pragma unroll
-    for (int i = 0; i <= P; i++) {
-        double acc = 0.0, hp = 1.0, bin = 1.0;
+    for (int b = 0; b <= (D == 2 ? P : 0); b++)
 #pragma unroll
-        for (int a = i; a >= 0; a--) {
-            acc = fma(bin * hp, L[a], acc);
-            hp *= -h;
-            bin = bin * (double)a / (double)(i - a + 1);
-        }
-        K[i] = acc;
+        for (int k = P - 1; k >= 0; k--)
+#pragma unroll
+            for (int i = 0; i < P; i++)
+                if (k < P - b && i >= k && i < P - b) L[ix(i + 1, b)] = fma(-hx, L[ix(i, b)], L[ix(i + 1, b)]);
+    if constexpr (D == 2) {
+#pragma unroll
+        for (int a = 0; a <= P; a++)
+#pragma unroll
+            for (int k = P - 1; k >= 0; k--)
+#pragma unroll
+                for (int i = 0; i < P; i++)
+                    if (k < P - a && i >= k && i < P - a) L[ix(a, i + 1)] = fma(-hy, L[ix(a, i)], L[ix(a, i + 1)]);
     }
 }
 
@@ -575,42 +592,16 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
     sp[0] = 1.0;
 #pragma unroll
     for (int k = 1; k <= P; k++) sp[k] = sp[k - 1] * inv_sig;
-    double Mth[NB];
-    if constexpr (D == 1) {
-        origin_shift<P>(Ld, fx, Mth);
-#pragma unroll
-        for (int a = 0; a <= P; a++) Mth[a] *= sp[a];
-    } else {
-        // along X for every power of Y, then along Y for every power of X
-#pragma unroll
-        for (int b = 0; b <= P; b++) {
-            double col[P + 1], out[P + 1];
-#pragma unroll
-            for (int a = 0; a <= P; a++) col[a] = a + b <= P ? Ld[Q::ix(a, b)] : 0.0;
-            origin_shift<P>(col, fx, out);
-#pragma unroll
-            for (int a = 0; a + b <= P; a++) Mth[Q::ix(a, b)] = out[a];
-        }
-#pragma unroll
-        for (int a = 0; a <= P; a++) {
-            double col[P + 1], out[P + 1];
-#pragma unroll
-            for (int b = 0; b <= P; b++) col[b] = a + b <= P ? Mth[Q::ix(a, b)] : 0.0;
-            origin_shift<P>(col, fy, out);
-#pragma unroll
-            for (int b = 0; a + b <= P; b++) Mth[Q::ix(a, b)] = out[b] * sp[a + b];
-        }
-    }
-    double rmax = 0.0;
-    bool finite = true;
+    moments_about<D, P>(Ld, fx, fy);
+    long long worst = 0;
 #pragma unroll
     for (int j = 0; j < Q::N; j++) {
-        const double rj = Mth[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))] - con[j];
+        const int a = bx<D, FLUON>(j), b = by<D, FLUON>(j);
+        const double rj = Ld[Q::ix(a, b)] * sp[a + b] - con[j];
         r_out[j] = rj;
-        finite = finite && isfinite(rj);
-        rmax = fmax(rmax, fabs(rj));
+        worst = max_abs_bits(rj, worst);
     }
-    rmax_out = finite ? rmax : INFINITY;
+    rmax_out = worst < kInfBits ? __longlong_as_double(worst) : INFINITY;
     if constexpr (MODE == DF_CORR) {
 #pragma unroll
         for (int k = 0; k < Q::NJ; k++) MJ_out[k] = MJ[k];
@@ -627,7 +618,7 @@ __device__ __forceinline__ bool df_update(const float* MJ, const double* r, doub
     float A[N * (N + 1) / 2], x[N];
 #pragma unroll
     for (int i = 0; i < N; i++) {
-        x[i] = (float)r[i];
+        x[i] = narrow_signed(r[i]);
 #pragma unroll
         for (int j = 0; j <= i; j++)
             A[tri(i, j)] = MJ[D == 1 ? bx<D, FLUON>(i) + bx<D, FLUON>(j)
@@ -635,7 +626,7 @@ __device__ __forceinline__ bool df_update(const float* MJ, const double* r, doub
     }
     if (!ldlt_solve<float, N>(A, x)) return false;
 #pragma unroll
-    for (int j = 0; j < N; j++) lam[j] += (double)x[j];
+    for (int j = 0; j < N; j++) lam[j] += widen(x[j]);
     return true;
 }
 

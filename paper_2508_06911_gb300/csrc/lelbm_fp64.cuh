@@ -25,14 +25,6 @@
 
 namespace lbm {
 
-// FP64 -> FP32 by truncation with integer operations (the conversion instruction runs on the
-// FP64 pipe).  Positive normal values; below 2^-126 zero, from 2^128 on (and NaN) infinity.
-__device__ __forceinline__ float narrow(double v) {
-    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-    const float f = __uint_as_float(__funnelshift_l(lo, hi - 0x38000000u, 3));
-    return hi < 0x38100000u ? 0.f : (hi >= 0x47f00000u ? __int_as_float(0x7f800000) : f);
-}
-
 // ---------------------------------------------------------------------------
 // exp(x) in FP64 with integer instructions: Tang's table-driven method (ACM TOMS 15, 1989) in 64-bit
 // fixed point.  x log2(e) = n + j / 512 + rho, 2^(j/512) from a table, 2^rho from five Taylor terms.
@@ -413,28 +405,13 @@ __device__ __forceinline__ void add_thermal(const double* Ls, double fx, double 
     for (int k = 1; k <= P; k++) sp[k] = sp[k - 1] * hs;
     double K[Q::NB];
 #pragma unroll
-    for (int b = 0; b <= (D == 2 ? P : 0); b++) {
-        double col[P + 1], out[P + 1];
+    for (int k = 0; k < Q::NB; k++) K[k] = Ls[k];
+    moments_about<D, P>(K, fx, fy);
 #pragma unroll
-        for (int a = 0; a <= P; a++) col[a] = a + b <= P ? Ls[Q::ix(a, a + b <= P ? b : 0)] : 0.0;
-        origin_shift<P>(col, fx, out);
+    for (int b = 0; b <= (D == 2 ? P : 0); b++)
 #pragma unroll
-        for (int a = 0; a + b <= P; a++) K[Q::ix(a, b)] = out[a];
-    }
-    if constexpr (D == 1) {
-#pragma unroll
-        for (int a = 0; a <= P; a++) T[a] = fma(K[a], sp[a], T[a]);
-    } else {
-#pragma unroll
-        for (int a = 0; a <= P; a++) {
-            double col[P + 1], out[P + 1];
-#pragma unroll
-            for (int b = 0; b <= P; b++) col[b] = a + b <= P ? K[Q::ix(a + b <= P ? a : 0, b)] : 0.0;
-            origin_shift<P>(col, fy, out);
-#pragma unroll
-            for (int b = 0; a + b <= P; b++) T[Q::ix(a, b)] = fma(out[b], sp[a + b], T[Q::ix(a, b)]);
-        }
-    }
+        for (int a = 0; a + b <= P; a++)
+            T[Q::ix(a, b)] = a + b > 0 ? fma(K[Q::ix(a, b)], sp[a + b], T[Q::ix(a, b)]) : T[Q::ix(a, b)] + K[Q::ix(a, b)];
 }
 
 // One pass over the velocity set: the thermal moments of degree <= 3 of f (if doF) and <= 2 of g
@@ -569,16 +546,14 @@ __device__ __forceinline__ int newton_step64(const double* T, const float* Mom, 
     using Q = DFPop<D, FLUON>;
     constexpr int N = Q::N, PJ = Q::PJ;
     float x[N];
-    long long worst = 0;  // |r| as integers: ordered as the doubles are, with NaN above infinity
+    long long worst = 0;
 #pragma unroll
     for (int j = 0; j < N; j++) {
         const double r = T[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))] - con[j];
-        const long long b = __double_as_longlong(r) & 0x7fffffffffffffffLL;
-        worst = b > worst ? b : worst;
-        const float a = narrow(__longlong_as_double(b));
-        x[j] = __double2hiint(r) < 0 ? -a : a;
+        worst = max_abs_bits(r, worst);
+        x[j] = narrow_signed(r);
     }
-    if (worst >= 0x7ff0000000000000LL) return -1;
+    if (worst >= kInfBits) return -1;
     const bool conv = worst <= __double_as_longlong(tol);
     if (!conv && it >= max_iter) return -2;
     float A[N * (N + 1) / 2];

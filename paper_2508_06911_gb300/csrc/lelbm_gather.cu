@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(kGTX * kGTY) gather2d_kernel(const __grid_cons
                 for (int i = 0; i < 11; i++) M[i] = Min[i * g.ncell + cell];
                 CellState<2> c;
                 double RT, usq;
-                if (!cell_macros<2>(M, m.K, c.rho, c.u, RT, usq)) continue;
+                if (!cell_macros<2>(M, m, c.rho, c.u, RT, usq)) continue;
                 c.RT = RT;
                 c.sig = sqrt(RT);
                 c.inv_sig = 1.0 / c.sig;

@@ -3,6 +3,7 @@
 // lelbm_mlp.cu) and the C ABI (lelbm_api.cu, host side).
 #pragma once
 
+#include <cmath>
 #include <type_traits>
 #include <cstdint>
 #include <cuda_bf16.h>
@@ -54,13 +55,29 @@ struct Model {
                                    // instead of scattering; null: scatter with atomics
     int* det_halo;                 // with det_lam: max over cells of the reach of the velocity
                                    // set (cells), for the gather's window
-    // FP32 copies for the FP32 path (set by set_fp32_params)
+    // derived constants (set by set_derived_params)
+    double inv_dk2, inv_Pr, inv_K;  // 1 / (D + K + 2), 1 / Pr, 1 / K (0 for K = 0)
+    double nu_b_over;               // nu_b / (2/D - 2/(D + K)) of Eq. (C8b); < 0 -> omega_b = 1
+    double rad2[5];                 // squared refinement radii (refine_rad / 2^L)^2
+    int r_min_up;                   // smallest integer >= r_min
+    // FP32 copies
     float K32, nu_s32, nu_b32, Pr32, n_conf32, r_min32, refine_div32;
     double rad2_32[5];  // squared refinement radii, FP32 arithmetic: (refine_rad / 2^L)^2
 };
 
-// Fills the FP32 copies of the model parameters (host).
-inline void set_fp32_params(Model& m) {
+// Fills the derived constants and FP32 copies of the model parameters in D dimensions (host).
+inline void set_derived_params(Model& m, int D) {
+    m.inv_dk = 1.0 / ((double)D + m.K);
+    m.inv_dk2 = 1.0 / ((double)D + m.K + 2.0);
+    m.inv_Pr = 1.0 / m.Pr;
+    m.inv_K = m.K > 0.0 ? 1.0 / m.K : 0.0;
+    const double fb = 2.0 / D - 2.0 / (D + m.K);
+    m.nu_b_over = (m.nu_b < 0.0 || fb <= 0.0) ? -1.0 : m.nu_b / fb;
+    for (int L = 0; L < 5; L++) {
+        const double r = m.refine_rad * (1.0 / (1 << L));
+        m.rad2[L] = r * r;
+    }
+    m.r_min_up = m.r_min < 2e9 ? (int)std::ceil(m.r_min) : 2000000000;
     m.K32 = (float)m.K;
     m.nu_s32 = (float)m.nu_s;
     m.nu_b32 = (float)m.nu_b;

@@ -11,23 +11,6 @@
 
 namespace lbm {
 
-// ---------------------------------------------------------------------------
-// FP32 <-> FP64 bit helpers (integer operations only; GB300's FP64 pipe also runs
-// the FP32 <-> FP64 conversion instructions).
-// ---------------------------------------------------------------------------
-// Subnormals become zero.
-__device__ __forceinline__ float flush_sub(float v) { return (__float_as_uint(v) & 0x7f800000u) ? v : 0.f; }
-
-// FP32 -> FP64: the exponent is rebiased from 127 to 1023 by one addition and the
-// mantissa shifted into place.  Normal numbers widen exactly; zeros and subnormals give
-// zero.  Infinities and NaNs, which a converged solve does not produce, come out finite.
-__device__ __forceinline__ double widen(float v) {
-    const unsigned int b = __float_as_uint(v);
-    const bool tiny = (b & 0x7f800000u) == 0u;
-    const unsigned int hi = (((b >> 3) & 0x0fffffffu) + 0x38000000u) | (b & 0x80000000u);
-    return __hiloint2double(tiny ? 0 : (int)hi, tiny ? 0 : (int)(b << 29));
-}
-
 struct LocalStats {
     unsigned long long q_max;
     double disp_max2;

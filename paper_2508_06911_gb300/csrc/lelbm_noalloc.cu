@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(128) noalloc_cell_kernel(Model m, Topo t, cons
         Stencil<D> st;
         st.init(c, m);
         double lf[NF], lg[NG];
-        maxwell_start_fg<D, NF, NG>(c.RT, lf, lg);
+        maxwell_start_newton<D, NF, NG>(c.RT, lf, lg);
 #pragma unroll
         for (int j = 0; j < NF; j++) conF[j] = c.cf[j];
 #pragma unroll
@@ -248,7 +248,6 @@ extern "C" int lelbm_step_noalloc(const lelbm_params* p, const double* m_in, dou
 
     Model m{};
     m.K = p->K;
-    m.inv_dk = 1.0 / ((double)p->dims + p->K);
     m.nu_s = p->nu_shear;
     m.nu_b = p->nu_bulk;
     m.Pr = p->prandtl;
@@ -260,7 +259,7 @@ extern "C" int lelbm_step_noalloc(const lelbm_params* p, const double* m_in, dou
     m.max_refine = p->max_refine;
     m.tol = p->tol;
     m.max_iter = p->max_newton;
-    set_fp32_params(m);
+    set_derived_params(m, p->dims);
 
     Topo t{};
     t.D = p->dims;

@@ -1314,7 +1314,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
             if (!fin) maxwell_start32<D, NF, NG>(rt32, lf32, lg32);
         }
     } else {
-        maxwell_start_fg<D, NF, NG>(c.RT, lf, lg);
+        maxwell_start_newton<D, NF, NG>(c.RT, lf, lg);
         if (dl_ok) {
 #pragma unroll
             for (int j = 0; j < NF; j++) lf[j] += (double)dl[j];
@@ -1340,7 +1340,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
                 }
             }
             learned = fin;
-            if (!fin) maxwell_start_fg<D, NF, NG>(c.RT, lf, lg);
+            if (!fin) maxwell_start_newton<D, NF, NG>(c.RT, lf, lg);
         }
     }
 #pragma unroll

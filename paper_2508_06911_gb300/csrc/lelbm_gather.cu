@@ -14,11 +14,17 @@
 // the staged sources inside its own window.  Periodic axes wrap the source coordinate, so a
 // source that reaches a target through several images contributes once per image, as in
 // the scatter.
+//
+// FP64 instructions bound the kernel.  Most pairs in the window (2 H + 1)^2 are no points of the
+// source's set, so membership is decided in FP32 on offsets from floor(u) (as in RowTable::build: only
+// a test closer to its threshold than FP32 resolves goes to FP64); a pair that is a point takes 45
+// FP64 operations, its exponentials being integer code (exp_int).
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "lelbm_device.cuh"
+#include "lelbm_fp64.cuh"
 #include "lelbm_internal.h"
 
 namespace lbm {
@@ -29,39 +35,33 @@ constexpr int kGRB = 2, kGCW = 64;  // staged chunk: source rows x columns
 struct GSrc {
     double ux, uy, inv_sig, rr2, mf, mg;  // mf = rho, mg = rho K RT (Eq. IIE3)
     double lf[10], lg[6];
+    float fx, fy;  // u - floor(u)
+    int bx, by;    // floor(u)
     int R, Nr, ok;
 };
 
 // Adds the moment fractions of one population point c (lattice frame, relative to its
-// source), volume dC and cloud-in-cell weight w, to acc (Eq. IIE3).
-__device__ __forceinline__ void gather_point(const GSrc& s, bool has_g, double cx, double cy, double dC, double w,
-                                             double* acc) {
-    const double t[2] = {(cx - s.ux) * s.inv_sig, (cy - s.uy) * s.inv_sig};
-    double T[10];
-    Basis<2, true>::eval(t, T);
-    double ef = 1.0;
+// source) of weight w (volume dC times cloud-in-cell share), to acc (Eq. IIE3).
+__device__ __forceinline__ void gather_point(const GSrc& s, bool has_g, double cx, double cy, double w, double* acc) {
+    const double x = (cx - s.ux) * s.inv_sig, y = (cy - s.uy) * s.inv_sig;
+    double cf[4], cg[3];
+    row_coeffs<2>(s.lf, s.lg, y, cf, cg);
+    const double mf = w * s.mf * exp_int(-(((cf[3] * x + cf[2]) * x + cf[1]) * x + cf[0]));
+    const double mg = has_g ? w * s.mg * exp_int(-((cg[2] * x + cg[1]) * x + cg[0])) : 0.0;
+    double v[11];
+    stored_moments<2, true, true>(cx, cy, mf, mg, v);
 #pragma unroll
-    for (int j = 0; j < 10; j++) ef += s.lf[j] * T[j];
-    const double mf = w * (s.mf * (dC * exp(-ef)));
-    double mg = 0.0;
-    if (has_g) {
-        double eg = 1.0;
-#pragma unroll
-        for (int j = 0; j < 6; j++) eg += s.lg[j] * T[j];
-        mg = w * (s.mg * (dC * exp(-eg)));
-    }
-    const double csq = cx * cx + cy * cy;
-    acc[0] += mf;
-    acc[1] += cx * mf;
-    acc[2] += cy * mf;
-    acc[3] += cx * cx * mf;
-    acc[4] += cx * cy * mf;
-    acc[5] += cy * cy * mf;
-    acc[6] += csq * cx * mf;
-    acc[7] += csq * cy * mf;
-    acc[8] += mg;
-    acc[9] += cx * mg;
-    acc[10] += cy * mg;
+    for (int k = 0; k < 11; k++) acc[k] += v[k];
+}
+
+// Is the lattice point at (dx, dy) within distance^2 thr of the source's u (inclusive)?
+__device__ __forceinline__ bool gather_inside(const GSrc& s, int dx, int dy, double thr, float thr32) {
+    const float ex = (float)(dx - s.bx) - s.fx, ey = (float)(dy - s.by) - s.fy;
+    const float v = fmaf(ex, ex, ey * ey), mg = 1e-3f + 1e-5f * thr32;
+    if (v < thr32 - mg) return true;
+    if (v > thr32 + mg) return false;
+    const double a = __dsub_rn((double)dx, s.ux), b = __dsub_rn((double)dy, s.uy);  // as Stencil::dist2
+    return __dadd_rn(__dadd_rn(0.0, __dmul_rn(a, a)), __dmul_rn(b, b)) <= thr;
 }
 
 __global__ void __launch_bounds__(kGTX * kGTY) gather2d_kernel(const __grid_constant__ Model m,
@@ -84,8 +84,7 @@ __global__ void __launch_bounds__(kGTX * kGTY) gather2d_kernel(const __grid_cons
     double rad2[5];
 #pragma unroll
     for (int L = 0; L < 5; L++) {
-        const double rad = m.refine_rad * ldexp(1.0, -L);
-        rad2[L] = rad * rad;  // as Stencil::init
+        rad2[L] = m.rad2[L];
     }
     const int sx_lo = tx0 - H, sx_hi = tx0 + kGTX - 1 + H;
     const int sy_lo = ty0 - H, sy_hi = ty0 + kGTY - 1 + H;
@@ -119,11 +118,15 @@ __global__ void __launch_bounds__(kGTX * kGTY) gather2d_kernel(const __grid_cons
                 if (!cell_macros<2>(M, m, c.rho, c.u, RT, usq)) continue;
                 c.RT = RT;
                 c.sig = sqrt(RT);
-                c.inv_sig = 1.0 / c.sig;
+                c.inv_sig = recip64(c.sig);
                 Stencil<2> st;
                 st.init(c, m);
                 s.ux = c.u[0];
                 s.uy = c.u[1];
+                s.bx = (int)floor(c.u[0]);
+                s.by = (int)floor(c.u[1]);
+                s.fx = (float)(c.u[0] - (double)s.bx);
+                s.fy = (float)(c.u[1] - (double)s.by);
                 s.inv_sig = c.inv_sig;
                 s.rr2 = st.rr2;
                 s.mf = c.rho;
@@ -147,46 +150,56 @@ __global__ void __launch_bounds__(kGTX * kGTY) gather2d_kernel(const __grid_cons
                     const GSrc& s = src[r][k];
                     if (!s.ok) continue;
                     const int dx = tx - (sx0 + k);  // the point c = (dx, dy) of the source
-                    const double ex = (double)dx - s.ux, ey = (double)dy - s.uy;
-                    const double reach = (double)s.R + 2.5;
+                    const float ex = (float)(dx - s.bx) - s.fx, ey = (float)(dy - s.by) - s.fy;
+                    const float reach = (float)s.R + 2.6f;
                     if (ex * ex + ey * ey > reach * reach) continue;
-                    Stencil<2> st;
-                    st.u[0] = s.ux;
-                    st.u[1] = s.uy;
-                    st.rr2 = s.rr2;
-                    st.R = s.R;
-                    st.Nr = s.Nr;
-#pragma unroll
-                    for (int L = 0; L < 5; L++) st.rad2[L] = rad2[L];
-                    const double cd[2] = {(double)dx, (double)dy};
-                    const double d2 = st.dist2(cd);
+                    const float rr = (float)s.R + 0.5f, rr32 = rr * rr, split32 = (float)rad2[1];
                     // a level-0 point that is not split lands exactly on the target
-                    if (d2 <= st.rr2 && (st.Nr == 0 || d2 > st.rad2[1])) {
-                        gather_point(s, has_g, cd[0], cd[1], 1.0, 1.0, acc);
+                    if (gather_inside(s, dx, dy, s.rr2, rr32) &&
+                        (s.Nr == 0 || !gather_inside(s, dx, dy, rad2[1], split32))) {
+                        gather_point(s, has_g, widen((float)dx), widen((float)dy), 1.0, acc);
                         n_dep++;
                     }
-                    // children of split points (within refine_rad / 2 of u) whose
-                    // cloud-in-cell share reaches the target
-                    if (st.Nr > 0 && fabs(ex) < 3.0 && fabs(ey) < 3.0) {
-                        const double r1 = sqrt(st.rad2[1]);
-                        const int ax = (int)floor(s.ux - r1) - 1, bx = (int)ceil(s.ux + r1) + 1;
-                        const int ay = (int)floor(s.uy - r1) - 1, by = (int)ceil(s.uy + r1) + 1;
-                        for (int py0 = ay; py0 <= by; py0++) {
-                            if (abs(py0 - dy) > 1) continue;
-                            for (int px0 = ax; px0 <= bx; px0++) {
-                                if (abs(px0 - dx) > 1) continue;
-                                const double c0[2] = {(double)px0, (double)py0};
-                                const double p2 = st.dist2(c0);
-                                if (!(p2 <= st.rr2 && p2 <= st.rad2[1])) continue;
-                                auto leaf = [&](const double* cl, double dC) {
-                                    const double wx = 1.0 - fabs(cl[0] - cd[0]), wy = 1.0 - fabs(cl[1] - cd[1]);
-                                    if (wx > 0.0 && wy > 0.0) {
-                                        gather_point(s, has_g, cl[0], cl[1], dC, wx * wy, acc);
+                    // children of split points whose cloud-in-cell share reaches the target
+                    const float near = sqrtf(split32) + 1.6f;
+                    if (s.Nr == 0 || fabsf(ex) > near || fabsf(ey) > near) continue;
+#pragma unroll 1
+                    for (int py0 = dy - 1; py0 <= dy + 1; py0++) {
+#pragma unroll 1
+                        for (int px0 = dx - 1; px0 <= dx + 1; px0++) {
+                            if (!gather_inside(s, px0, py0, s.rr2, rr32) ||
+                                !gather_inside(s, px0, py0, rad2[1], split32))
+                                continue;
+                            if (s.Nr == 1) {  // four children at +-1/4
+#pragma unroll 1
+                                for (int k = 0; k < 4; k++) {
+                                    const float cx = (float)px0 + ((k & 1) ? 0.25f : -0.25f);
+                                    const float cy = (float)py0 + ((k & 2) ? 0.25f : -0.25f);
+                                    const float wx = 1.f - fabsf(cx - (float)dx), wy = 1.f - fabsf(cy - (float)dy);
+                                    if (wx > 0.f && wy > 0.f) {
+                                        gather_point(s, has_g, widen(cx), widen(cy), widen(0.25f * wx * wy), acc);
                                         n_dep++;
                                     }
-                                };
-                                st.visit0(c0, leaf);
+                                }
+                                continue;
                             }
+                            Stencil<2> st;
+                            st.u[0] = s.ux;
+                            st.u[1] = s.uy;
+                            st.rr2 = s.rr2;
+                            st.R = s.R;
+                            st.Nr = s.Nr;
+#pragma unroll
+                            for (int L = 0; L < 5; L++) st.rad2[L] = rad2[L];
+                            const double c0[2] = {(double)px0, (double)py0};
+                            auto leaf = [&](const double* cl, double dC) {
+                                const double wx = 1.0 - fabs(cl[0] - (double)dx), wy = 1.0 - fabs(cl[1] - (double)dy);
+                                if (wx > 0.0 && wy > 0.0) {
+                                    gather_point(s, has_g, cl[0], cl[1], dC * (wx * wy), acc);
+                                    n_dep++;
+                                }
+                            };
+                            st.visit0(c0, leaf);
                         }
                     }
                 }

@@ -1055,7 +1055,8 @@ __device__ __forceinline__ void count_set(const RowTable<D>& tab, const CellLatt
 }
 
 // The FP64 path's cell after the collision: EPR from the multipliers lf, lg, and moment streaming, in
-// lattice form where the cell has a row table whose offsets are exact in FP32 (|k|^3 < 2^24).
+// lattice form where the cell has a row table whose offsets and velocities are exact in FP32
+// (|k|^3 and quarter cells below 2^24).
 template <int D>
 __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                           DevStats* stats, const CellPlace& at, BlockCounters& bc,
@@ -1063,7 +1064,7 @@ __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, con
                                           const Stencil<D>& st, const RowTable<D>& tab, double* lf, double* lg,
                                           bool learned) {
     const bool has_g = m.K > 0.0;
-    if (tab.ok && st.R <= 250) {
+    if (tab.ok && st.R <= 250 && abs(tab.xc) < (1 << 21) && abs(tab.yc) < (1 << 21)) {
         CellLattice<D> lat;
         lat.init(c, tab);
         int sf, sg;

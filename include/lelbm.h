@@ -67,7 +67,10 @@ extern "C" {
 #define LELBM_BC_PERIODIC 2 /* wrap-around; must be set on both sides of an axis      */
 
 /* arithmetic of the step */
-#define LELBM_FP64 0  /* every operation in FP64                                     */
+#define LELBM_FP64 0  /* state, collision, populations, residuals, multipliers and
+                         accumulation in FP64; the Jacobian and the solve of a Newton
+                         update, which only steer the iteration, in FP32 (a solve that
+                         breaks down is redone with both in FP64)             */
 #define LELBM_MIXED 1 /* EPR Newton in FP32 to the FP32 noise floor, then per
                          population one Newton correction whose residual is summed
                          in double-float (FP32 pairs, about 48 bits) with an FP32
@@ -76,8 +79,12 @@ extern "C" {
                          against tol (a miss is taken back and corrected again,
                          then left to the FP64 EPR).  Exponents are exact int64
                          fixed-point polynomials, 2^w a table-driven double-float
-                         exponential; deposits are FP64 atomic additions of both
-                         words.  State, collision and accumulation in FP64.
+                         exponential; a correction below 2e-6 of the constraints
+                         reaches the streaming pass as a relative change of the
+                         populations that the correction pass kept (scratch of the
+                         handle: 4 KB a resident thread, at most 239 MB).  Deposits
+                         are FP64 atomic additions.  State, collision and
+                         accumulation in FP64.
                          Matches LELBM_FP64 to about 1e-13 per step.             */
 #define LELBM_FP32 2  /* EPR Newton (passes and solves) and the streaming pass in
                          FP32, to an FP32 residual of 3e-4 (thermal units) plus one

@@ -53,6 +53,7 @@ struct lelbm {
     float* d_mlp_nrm = nullptr;        // and normalisation
     float* d_lam = nullptr;            // stored warm start (lelbm_set_warmstart)
     float* d_mlp_start = nullptr;      // learned start of the current step (cell-update path)
+    float2* d_df_pop = nullptr;        // mixed path: kept populations (Model::df_pop)
     double* d_det_lam = nullptr;       // deterministic streaming: per-cell multipliers
     int* d_det_halo = nullptr;         // and the reach of the step's velocity sets
     cudaGraphExec_t graph = nullptr;  // captured lelbm_run_batch launch
@@ -211,6 +212,7 @@ static void free_all(lelbm* h) {
     cudaFree(h->d_mlp_nrm);
     cudaFree(h->d_lam);
     cudaFree(h->d_mlp_start);
+    cudaFree(h->d_df_pop);
     cudaFree(h->d_det_lam);
     cudaFree(h->d_det_halo);
     if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -526,6 +528,21 @@ extern "C" int lelbm_create(lelbm_t* out, const lelbm_params* p) {
         if (cudaMalloc((void**)&h->d_det_lam, sizeof(double) * 16 * (size_t)h->ncell) != cudaSuccess ||
             cudaMalloc((void**)&h->d_det_halo, sizeof(int)) != cudaSuccess)
             rc = LELBM_E_NOMEM;
+    }
+    if (!rc && p->precision == LELBM_MIXED) {
+        // scratch for the threads that can be resident (one 384-thread block an SM); without it the
+        // mixed path evaluates its populations twice
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        constexpr long long nt = cell_threads<PREC_MIXED>();
+        const long long threads = std::min<long long>(sms * nt, (h->ncell + nt - 1) / nt * nt);
+        if (cudaMalloc((void**)&h->d_df_pop, sizeof(float2) * kDfPopCap * (size_t)threads) == cudaSuccess) {
+            h->model.df_pop = h->d_df_pop;
+            h->model.df_pop_threads = (int)threads;
+        } else {
+            h->d_df_pop = nullptr;
+            cudaGetLastError();
+        }
     }
     if (!rc) rc = reset_stats_dev(h);
     if (rc) {

@@ -317,8 +317,53 @@ struct DFStream {
     CellPlace at;
     bool near_wall;
     float mh, ml;   // rho dV (fluons) or rho K RT dV (phonons), signed, as a double-float
+    float2* pop;      // the thread's populations of the last correction pass, pop[i * pop_stride] for the
+    int pop_stride;   // i-th point (i < pop_cap); pop_cap = 0: none are kept
+    int pop_cap;
     long long* beta;  // the thread's slot for the exponent coefficients (shared memory)
 };
+
+// 1D deposit of the mass (vh, vl) at velocity cx.  A child has only two landing cells, so its shares go one
+// by one, as double-float products (FP32 instructions) with two atomic additions each, of the high and
+// the low word (both widened exactly): 16 FP64 operations a child for merged columns cost the batch's
+// cold tubes 2 %.
+template <bool FLUON>
+__device__ __forceinline__ void deposit_1d(const DFStream& ds, float cx, float vh, float vl, bool child) {
+    auto put_all = [&](int dx, float sh, float sl) {
+        const long long tgt = land<1>(*ds.g, ds.at.cell, ds.at.lo, ds.at.n, 0, 0, dx, 0);
+        if (tgt < 0) return;
+        auto put = [&](int mm, float T) {
+            if (T == 0.f) return;
+            float p, e;
+            two_prod(T, sh, p, e);
+            e = __fmaf_rn(T, sl, e);
+            double* a = ds.Mout + (long long)mm * ds.g->ncell + tgt;
+            atomicAdd(a, widen(p));
+            atomicAdd(a, widen(e));
+        };
+        if constexpr (FLUON) {
+            put(0, 1.f);
+            put(1, cx);
+            put(2, cx * cx);
+            put(3, cx * cx * cx);
+        } else {
+            put(4, 1.f);
+            put(5, cx);
+        }
+    };
+    if (!child) {
+        put_all((int)cx, vh, vl);
+        return;
+    }
+    const float flx = floorf(cx), w1 = cx - flx;
+#pragma unroll 1
+    for (int sx = 0; sx < 2; sx++) {
+        const float w = sx ? w1 : 1.f - w1;
+        float sh, sl;
+        two_prod(w, vh, sh, sl);
+        put_all((int)flx + sx, sh, __fmaf_rn(w, vl, sl));
+    }
+}
 
 // Out of line: one object per (dimension, population, mode), called two to three times per
 // cell; the cell enters as u (ux, uy) and 1 / sqrt(RT) only.  beta: a per-thread slot of
@@ -350,53 +395,13 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
     unsigned long long q = 0;
     long long walls = 0;
     int dmax = 0;
+    int kept = 0;  // DF_CORR: populations written to ds.pop
     // a population at the lattice velocity (cx, cy): its mass in FP64, then FP64 moments and one
     // atomic addition each (FP64 products cost fewer issue slots than double-float ones)
     auto mass = [&](float fh, float fl) {
         float vh, vl;
         df_mul(ds.mh, ds.ml, fh, fl, vh, vl);
         return widen(vh) + widen(vl);
-    };
-    // 1D: a child has only two landing cells, so its shares go one by one, as double-float products
-    // (FP32 instructions) with two atomic additions each, of the high and the low word (both widened
-    // exactly): 16 FP64 operations a child for merged columns cost the batch's cold tubes 2 %
-    auto put_df = [&](int dx, float cx, float vh, float vl) {
-        const long long tgt = land<D>(*ds.g, ds.at.cell, ds.at.lo, ds.at.n, 0, 0, dx, 0);
-        if (tgt < 0) return;
-        auto put = [&](int mm, float T) {
-            if (T == 0.f) return;
-            float p, e;
-            two_prod(T, vh, p, e);
-            e = __fmaf_rn(T, vl, e);
-            double* a = ds.Mout + (long long)mm * ds.g->ncell + tgt;
-            atomicAdd(a, widen(p));
-            atomicAdd(a, widen(e));
-        };
-        if constexpr (FLUON) {
-            put(0, 1.f);
-            put(1, cx);
-            put(2, cx * cx);
-            put(3, cx * cx * cx);
-        } else {
-            put(4, 1.f);
-            put(5, cx);
-        }
-    };
-    auto stream_1d = [&](float cx, float fh, float fl, bool child) {
-        float vh, vl;
-        df_mul(ds.mh, ds.ml, fh, fl, vh, vl);
-        if (!child) {
-            put_df((int)cx, cx, vh, vl);
-            return;
-        }
-        const float flx = floorf(cx), w1 = cx - flx;
-#pragma unroll 1
-        for (int sx = 0; sx < 2; sx++) {
-            const float w = sx ? w1 : 1.f - w1;
-            float sh, sl;
-            two_prod(w, vh, sh, sl);
-            put_df((int)flx + sx, cx, sh, __fmaf_rn(w, vl, sl));
-        }
     };
     auto trace = [&](double cx, double cy, double v) {
         if constexpr (D == 2) {
@@ -458,122 +463,128 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
     // one kind then stays in the instruction caches.
 #pragma unroll 1
     for (int lat = 0; lat < 2; lat++) {
-    const int r_first = D == 2 && lat ? tab.band_first : 0;
-    const int r_end = D == 2 ? (lat ? r_first + tab.band_n : tab.nrows) : 1;
+        const int r_first = D == 2 && lat ? tab.band_first : 0;
+        const int r_end = D == 2 ? (lat ? r_first + tab.band_n : tab.nrows) : 1;
 #pragma unroll 1
-    for (int rr = r_first; rr < r_end; rr++) {
-        int rx0, rx1, ra, rb, cy = 0;
-        if constexpr (D == 2) {
-            tab.row_ext(rr, rx0, rx1, ra, rb);
-            cy = tab.y_first + rr;
-        } else {
-            rx0 = tab.x0;
-            rx1 = tab.x1;
-            ra = tab.a;
-            rb = tab.b;
-        }
-        const int Y = cy - tab.yc;
-        const bool split = ra <= rb;
-        long long gm[P + 1];
-        if (lat == 0 && rx0 <= rx1) fix_row<D, FLUON>(beta, Y, gm);
-        // segments 0, 1: level-0 runs rx0..ra-1 and rb+1..rx1 (the whole row when no point
-        // splits); 2 (and 3 in 2D): the child rows at cy - 1/4 and cy + 1/4
-#pragma unroll 1
-        for (int seg = 2 * lat; seg < (lat ? (D == 2 ? 4 : 3) : 2); seg++) {
-            long long D0, D1, D2 = 0, D3 = 0;
-            float Xf, h, Yf, y32;
-            int np, dn;
-            if (seg < 2) {
-                if (rx0 > rx1 || (seg == 1 && !split)) continue;
-                const int xa = seg == 0 ? rx0 : rb + 1;
-                const int xb = seg == 0 ? (split ? ra - 1 : rx1) : rx1;
-                if (xa > xb) continue;
-                const long long x0 = xa - tab.xc;
-                if constexpr (P == 3) {
-                    D3 = 6 * gm[3];
-                    D2 = 2 * gm[2] + 6 * gm[3] * (x0 + 1);
-                    D1 = gm[1] + gm[2] * (2 * x0 + 1) + gm[3] * (3 * x0 * x0 + 3 * x0 + 1);
-                    D0 = ((gm[3] * x0 + gm[2]) * x0 + gm[1]) * x0 + gm[0];
-                } else {
-                    D2 = 2 * gm[2];
-                    D1 = gm[1] + gm[2] * (2 * x0 + 1);
-                    D0 = (gm[2] * x0 + gm[1]) * x0 + gm[0];
-                }
-                Xf = (float)x0;
-                h = 1.f;
-                np = xb - xa + 1;
-                dn = 0;
-                Yf = (float)Y;
-                y32 = D == 2 ? tab.ty(cy) : 0.f;
-                const int ex = max(abs(xa), abs(xb));
-                dmax = max(dmax, ex * ex + cy * cy);
+        for (int rr = r_first; rr < r_end; rr++) {
+            int rx0, rx1, ra, rb, cy = 0;
+            if constexpr (D == 2) {
+                tab.row_ext(rr, rx0, rx1, ra, rb);
+                cy = tab.y_first + rr;
             } else {
-                if (!split) break;
-                const int sy = D == 2 ? (seg == 2 ? -1 : 1) : 0;
-                const int n4 = 4 * Y + sy;
-                long long B[P + 1];
-                fix_child_row<D, FLUON>(beta, n4, B);
-                // N(m) = 64 w at the quarter offsets m = m0, m0 + 2, ... (exact integers)
-                const int m0 = 4 * (ra - tab.xc) - 1;
-                const long long N0 = fix_child_w<P>(B, m0), N1 = fix_child_w<P>(B, m0 + 2),
-                                N2 = fix_child_w<P>(B, m0 + 4);
-                D0 = N0;
-                D1 = N1 - N0;
-                D2 = N2 - 2 * N1 + N0;
-                if constexpr (P == 3) D3 = fix_child_w<P>(B, m0 + 6) - 3 * N2 + 3 * N1 - N0;
-                Xf = 0.25f * (float)m0;
-                h = 0.5f;
-                np = 2 * (rb - ra + 1);
-                dn = -D;
-                Yf = 0.25f * (float)n4;
-                y32 = D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f;
+                rx0 = tab.x0;
+                rx1 = tab.x1;
+                ra = tab.a;
+                rb = tab.b;
             }
-            DFAcc S[P + 1];
-            float SJ[PJ + 1];
-#pragma unroll
-            for (int a = 0; a <= P; a++) S[a].zero();
-#pragma unroll
-            for (int a = 0; a <= PJ; a++) SJ[a] = 0.f;
-            const float cyf = (float)tab.yc + Yf;  // c_y of the segment's points
-            const bool child = dn != 0;
-            const int sy = D == 2 && child ? (seg == 2 ? -1 : 1) : 0;
-            const bool traced = D == 2 && MODE == DF_STREAM && ds.near_wall;
-            ChildRow<D, FLUON, !FLUON> kids;
-            if constexpr (MODE == DF_STREAM) kids.start();
-            const int nk = D == 2 && MODE == DF_STREAM && child && !traced ? np + 3 : np;
+            const int Y = cy - tab.yc;
+            const bool split = ra <= rb;
+            long long gm[P + 1];
+            if (lat == 0 && rx0 <= rx1) fix_row<D, FLUON>(beta, Y, gm);
+            // segments 0, 1: level-0 runs rx0..ra-1 and rb+1..rx1 (the whole row when no point
+            // splits); 2 (and 3 in 2D): the child rows at cy - 1/4 and cy + 1/4
 #pragma unroll 1
-            for (int k = 0; k < nk; k++) {
-                float fh = 0.f, fl = 0.f;
-                if (k < np) {
-                    exp2_fix(D0, etab, dn, fh, fl);
-                    accumulate(S, SJ, Xf, fh, fl);
-                }
-                if constexpr (MODE == DF_STREAM) {
-                    const float cx = (float)tab.xc + Xf;
-                    if constexpr (D == 1) {
-                        stream_1d(cx, fh, fl, child);
+            for (int seg = 2 * lat; seg < (lat ? (D == 2 ? 4 : 3) : 2); seg++) {
+                long long D0, D1, D2 = 0, D3 = 0;
+                float Xf, h, Yf, y32;
+                int np, dn;
+                if (seg < 2) {
+                    if (rx0 > rx1 || (seg == 1 && !split)) continue;
+                    const int xa = seg == 0 ? rx0 : rb + 1;
+                    const int xb = seg == 0 ? (split ? ra - 1 : rx1) : rx1;
+                    if (xa > xb) continue;
+                    const long long x0 = xa - tab.xc;
+                    if constexpr (P == 3) {
+                        D3 = 6 * gm[3];
+                        D2 = 2 * gm[2] + 6 * gm[3] * (x0 + 1);
+                        D1 = gm[1] + gm[2] * (2 * x0 + 1) + gm[3] * (3 * x0 * x0 + 3 * x0 + 1);
+                        D0 = ((gm[3] * x0 + gm[2]) * x0 + gm[1]) * x0 + gm[0];
                     } else {
-                    const double v = mass(fh, fl);
-                    if (traced) {
-                        trace(widen(cx), D == 2 ? widen(cyf) : 0.0, v);
-                    } else if (child) {
-                        kids.add(*ds.g, ds.type, ds.Mout, ds.at, ra, k, cy, sy, v, v);
-                    } else {
-                        double vm[Stored<D, FLUON, !FLUON>::N];
-                        stored_moments<D, FLUON, !FLUON>(widen(cx), widen(cyf), v, v, vm);
-                        deposit_at<D, FLUON, !FLUON>(*ds.g, ds.type, ds.Mout, ds.at, tab.xc + (int)Xf, cy, vm);
+                        D2 = 2 * gm[2];
+                        D1 = gm[1] + gm[2] * (2 * x0 + 1);
+                        D0 = (gm[2] * x0 + gm[1]) * x0 + gm[0];
                     }
-                    }
+                    Xf = (float)x0;
+                    h = 1.f;
+                    np = xb - xa + 1;
+                    dn = 0;
+                    Yf = (float)Y;
+                    y32 = D == 2 ? tab.ty(cy) : 0.f;
+                    const int ex = max(abs(xa), abs(xb));
+                    dmax = max(dmax, ex * ex + cy * cy);
+                } else {
+                    if (!split) break;
+                    const int sy = D == 2 ? (seg == 2 ? -1 : 1) : 0;
+                    const int n4 = 4 * Y + sy;
+                    long long B[P + 1];
+                    fix_child_row<D, FLUON>(beta, n4, B);
+                    // N(m) = 64 w at the quarter offsets m = m0, m0 + 2, ... (exact integers)
+                    const int m0 = 4 * (ra - tab.xc) - 1;
+                    const long long N0 = fix_child_w<P>(B, m0), N1 = fix_child_w<P>(B, m0 + 2),
+                                    N2 = fix_child_w<P>(B, m0 + 4);
+                    D0 = N0;
+                    D1 = N1 - N0;
+                    D2 = N2 - 2 * N1 + N0;
+                    if constexpr (P == 3) D3 = fix_child_w<P>(B, m0 + 6) - 3 * N2 + 3 * N1 - N0;
+                    Xf = 0.25f * (float)m0;
+                    h = 0.5f;
+                    np = 2 * (rb - ra + 1);
+                    dn = -D;
+                    Yf = 0.25f * (float)n4;
+                    y32 = D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f;
                 }
-                D0 += D1;
-                D1 += D2;
-                if constexpr (P == 3) D2 += D3;
-                Xf += h;
+                DFAcc S[P + 1];
+                float SJ[PJ + 1];
+#pragma unroll
+                for (int a = 0; a <= P; a++) S[a].zero();
+#pragma unroll
+                for (int a = 0; a <= PJ; a++) SJ[a] = 0.f;
+                const float cyf = (float)tab.yc + Yf;  // c_y of the segment's points
+                const bool child = dn != 0;
+                const int sy = D == 2 && child ? (seg == 2 ? -1 : 1) : 0;
+                const bool traced = D == 2 && MODE == DF_STREAM && ds.near_wall;
+                ChildRow<D, FLUON, !FLUON> kids;
+                if constexpr (MODE == DF_STREAM) kids.start();
+                const int nk = D == 2 && MODE == DF_STREAM && child && !traced ? np + 3 : np;
+#pragma unroll 1
+                for (int k = 0; k < nk; k++) {
+                    float fh = 0.f, fl = 0.f;
+                    if (k < np) {
+                        exp2_fix(D0, etab, dn, fh, fl);
+                        accumulate(S, SJ, Xf, fh, fl);
+                        if constexpr (MODE == DF_CORR) {
+                            if (kept < ds.pop_cap) ds.pop[(long long)kept * ds.pop_stride] = make_float2(fh, fl);
+                            kept++;
+                        }
+                    }
+                    if constexpr (MODE == DF_STREAM) {
+                        const float cx = (float)tab.xc + Xf;
+                        if constexpr (D == 1) {
+                            float vh, vl;
+                            df_mul(ds.mh, ds.ml, fh, fl, vh, vl);
+                            deposit_1d<FLUON>(ds, cx, vh, vl, child);
+                        } else {
+                            const double v = mass(fh, fl);
+                            if (traced) {
+                                trace(widen(cx), D == 2 ? widen(cyf) : 0.0, v);
+                            } else if (child) {
+                                kids.add(*ds.g, ds.type, ds.Mout, ds.at, ra, k, cy, sy, v, v);
+                            } else {
+                                double vm[Stored<D, FLUON, !FLUON>::N];
+                                stored_moments<D, FLUON, !FLUON>(widen(cx), widen(cyf), v, v, vm);
+                                deposit_at<D, FLUON, !FLUON>(*ds.g, ds.type, ds.Mout, ds.at, tab.xc + (int)Xf, cy, vm);
+                            }
+                        }
+                    }
+                    D0 += D1;
+                    D1 += D2;
+                    if constexpr (P == 3) D2 += D3;
+                    Xf += h;
+                }
+                q += (unsigned long long)np;
+                fold(S, SJ, Yf, y32);
             }
-            q += (unsigned long long)np;
-            fold(S, SJ, Yf, y32);
         }
-    }
     }
     npts += (unsigned int)q;
     if constexpr (MODE == DF_STREAM) {
@@ -610,12 +621,12 @@ static __device__ __noinline__ bool df_pass(double ux, double uy, double inv_sig
 }
 
 // Newton update from a double-float residual and the FP32 Jacobian of the same pass
-// (Eq. IID11 with A in FP32): lam += A^-1 r.  False on a non-positive pivot.
+// (Eq. IID11 with A in FP32): x = A^-1 r, lam += x.  False on a non-positive pivot.
 template <int D, bool FLUON>
-__device__ __forceinline__ bool df_update(const float* MJ, const double* r, double* lam) {
+__device__ __forceinline__ bool df_update(const float* MJ, const double* r, double* lam, float* x) {
     using Q = DFPop<D, FLUON>;
     constexpr int N = Q::N, PJ = Q::PJ;
-    float A[N * (N + 1) / 2], x[N];
+    float A[N * (N + 1) / 2];
 #pragma unroll
     for (int i = 0; i < N; i++) {
         x[i] = narrow_signed(r[i]);
@@ -628,6 +639,145 @@ __device__ __forceinline__ bool df_update(const float* MJ, const double* r, doub
 #pragma unroll
     for (int j = 0; j < N; j++) lam[j] += widen(x[j]);
     return true;
+}
+
+// The streaming pass after a small update dlam of the multipliers, from the populations that the
+// correction pass kept: f' = f (1 + em), em = expm1(-dlam . T), where a DF_STREAM pass evaluates every
+// exponential and the whole residual again.  em is FP32: with |dlam| of the size of the FP32 Newton's
+// noise (1e-7) its rounding moves a population by 1e-14 of itself.  The residual of exactly what is
+// deposited is the correction pass's r plus sum T f em, whose FP32 sum is off by about 1e-7 of the
+// residual that dlam removes: kRestreamMax bounds that by 2e-13, inside the 1e-12 that is judged.
+// What bounds a DF_STREAM pass is FP32 instructions (79 a point for the exponential and the sums, and 250
+// a row to set them up); this pass takes 15 and 25, and a load.  1024^2 mixed step at RT 0.6: 4.28 -> 3.87 ms,
+// at RT 0.35 8.07 -> 7.15 ms, four-quadrant flow 9.58 -> 7.85 ms; 4096 tubes, two steps, 33.0 -> 18.7 ms.
+constexpr double kRestreamMax = 2e-6;
+
+template <int D, bool FLUON>
+static __device__ __noinline__ void df_restream(const RowTable<D>& tab_in, const float* __restrict__ dlam,
+                                                const double* __restrict__ r, double& rmax_out,
+                                                const DFStream& ds_in, LocalStats& ls, unsigned int& npts) {
+    using Q = DFPop<D, FLUON>;
+    constexpr int P = Q::P, N = Q::N, NB = Q::NB;
+    const RowTable<D> tab = tab_in;
+    const DFStream ds = ds_in;
+    float d[NB];
+#pragma unroll
+    for (int j = 0; j < N; j++) d[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))] = dlam[j];
+    float L[NB];  // sum x^a y^b f em, thermal units
+#pragma unroll
+    for (int k = 0; k < NB; k++) L[k] = 0.f;
+    const float2* pop = ds.pop;
+    unsigned int q = 0;
+    int dmax = 0;
+#pragma unroll 1
+    for (int lat = 0; lat < 2; lat++) {  // the order of points of df_pass
+        const int r_first = D == 2 && lat ? tab.band_first : 0;
+        const int r_end = D == 2 ? (lat ? r_first + tab.band_n : tab.nrows) : 1;
+#pragma unroll 1
+        for (int rr = r_first; rr < r_end; rr++) {
+            int rx0, rx1, ra, rb, cy = 0;
+            if constexpr (D == 2) {
+                tab.row_ext(rr, rx0, rx1, ra, rb);
+                cy = tab.y_first + rr;
+            } else {
+                rx0 = tab.x0;
+                rx1 = tab.x1;
+                ra = tab.a;
+                rb = tab.b;
+            }
+            const bool split = ra <= rb;
+            if (lat && !split) continue;
+            if (lat == 0 && rx0 <= rx1) {
+                const int ex = max(abs(rx0), abs(rx1));
+                dmax = max(dmax, ex * ex + cy * cy);
+            }
+#pragma unroll 1
+            for (int seg = 0; seg < (lat ? D : (split ? 2 : 1)); seg++) {
+                const int xa = lat ? ra : (seg == 0 ? rx0 : rb + 1);
+                const int xb = lat ? rb : (seg == 0 && split ? ra - 1 : rx1);
+                if (xa > xb) continue;
+                const bool child = lat != 0;
+                const int sy = D == 2 && child ? (seg == 0 ? -1 : 1) : 0;
+                const int np = child ? 2 * (xb - xa + 1) : xb - xa + 1;
+                const float h = child ? 0.5f : 1.f;
+                float cx = (float)xa - (child ? 0.25f : 0.f);  // c_x, exact
+                float Xf = (float)(xa - tab.xc) - (child ? 0.25f : 0.f);
+                const float y = D == 2 ? tab.ty(cy, 0.25f * (float)sy) : 0.f;
+                // -(dlam . T) on the row as a polynomial in x
+                float cf[P + 1];
+#pragma unroll
+                for (int a = 0; a <= P; a++) {
+                    float v = -d[Q::ix(a, D == 2 ? P - a : 0)];
+                    if constexpr (D == 2) {
+#pragma unroll
+                        for (int b = P - a - 1; b >= 0; b--) v = fmaf(v, y, -d[Q::ix(a, b)]);
+                    }
+                    cf[a] = v;
+                }
+                float S[P + 1];
+#pragma unroll
+                for (int a = 0; a <= P; a++) S[a] = 0.f;
+                ChildRow<D, FLUON, !FLUON> kids;
+                if (D == 2) kids.start();
+                const int nk = D == 2 && child ? np + 3 : np;
+                float2 f = *pop;
+#pragma unroll 1
+                for (int k = 0; k < nk; k++) {
+                    float vh = 0.f, vl = 0.f;
+                    if (k < np) {
+                        const float2 now = f;
+                        pop += ds.pop_stride;
+                        if (k + 1 < np) f = *pop;
+                        const float x = fmaf(Xf, tab.s32, -tab.fux);
+                        float e = cf[P];
+#pragma unroll
+                        for (int a = P - 1; a >= 0; a--) e = fmaf(e, x, cf[a]);
+                        const float w = now.x * fmaf(0.5f * e, e, e);
+                        S[0] += w;
+                        float px = x;
+#pragma unroll
+                        for (int a = 1; a <= P; a++) {
+                            S[a] = fmaf(px, w, S[a]);
+                            px *= x;
+                        }
+                        df_mul(ds.mh, ds.ml, now.x, __fadd_rn(now.y, w), vh, vl);
+                    }
+                    if constexpr (D == 1) {
+                        deposit_1d<FLUON>(ds, cx, vh, vl, child);
+                    } else {
+                        const double v = widen(vh) + widen(vl);
+                        if (child) {
+                            kids.add(*ds.g, ds.type, ds.Mout, ds.at, ra, k, cy, sy, v, v);
+                        } else {
+                            double vm[Stored<D, FLUON, !FLUON>::N];
+                            stored_moments<D, FLUON, !FLUON>(widen(cx), widen((float)cy), v, v, vm);
+                            deposit_at<D, FLUON, !FLUON>(*ds.g, ds.type, ds.Mout, ds.at, (int)cx, cy, vm);
+                        }
+                    }
+                    cx += h;
+                    Xf += h;
+                }
+                q += (unsigned int)np;
+                float yp = 1.f;
+#pragma unroll
+                for (int b = 0; b <= (D == 2 ? P : 0); b++) {
+#pragma unroll
+                    for (int a = 0; a + b <= P; a++) L[Q::ix(a, b)] = fmaf(S[a], yp, L[Q::ix(a, b)]);
+                    yp *= y;
+                }
+            }
+        }
+    }
+    npts += q;
+    if (FLUON && ds.mh > 0.f) {  // counted once per cell: the fluon deposit, not a take-back
+        if (q > ls.q_max) ls.q_max = q;
+        ls.points += q;
+        ls.disp_max2 = fmax(ls.disp_max2, (double)dmax);
+    }
+    long long worst = 0;
+#pragma unroll
+    for (int j = 0; j < N; j++) worst = max_abs_bits(r[j] + widen(L[Q::ix(bx<D, FLUON>(j), by<D, FLUON>(j))]), worst);
+    rmax_out = worst < kInfBits ? __longlong_as_double(worst) : INFINITY;
 }
 
 }  // namespace lbm

@@ -25,6 +25,14 @@ using Con = typename std::conditional<PREC == PREC_FP32, float, double>::type;
 template <int PREC>
 constexpr int cell_threads() { return PREC == PREC_MIXED ? 384 : 128; }
 
+// Points of a velocity set whose populations the mixed path keeps between its correction and its streaming
+// pass: up to R_ac = 12 in 2D (q = 490), 4 KB for each of the threads that can be resident (239 MB a GPU;
+// a grid of fewer cells takes less).  A step touches q entries a thread, so up to q = 250 what it keeps
+// stays in L2 (129 MB); at RT = 8 (q = 434) reading it back still beats evaluating it again (7.17 against
+// 7.98 ms at 512^2).
+constexpr int kDfPopCap = 512;
+constexpr int kDfPopR = 12;  // larger sets (2D) are not kept
+
 // Physical and numerical constants of one handle (Sec. II, App. C, App. D).
 struct Model {
     double K;           // internal degrees of freedom
@@ -50,6 +58,8 @@ struct Model {
                                    // mlp_start_kernel, SoA [NF + NG][ncell] (NaN: none), or null
     float mlp_gate;                // learned start only where the normalised constraints depart
                                    // from equilibrium by at least this much (0: everywhere)
+    float2* df_pop;                // mixed path: scratch for the populations of a correction pass,
+    int df_pop_threads;            // [kDfPopCap][df_pop_threads], one column per thread (0: none)
     double* det_lam;               // deterministic streaming (FP64 2D): the cell kernel writes
                                    // each cell's final multipliers here, SoA [NF + NG][ncell],
                                    // instead of scattering; null: scatter with atomics

@@ -166,7 +166,9 @@ __device__ __forceinline__ void keep_shortfall32(const Model& m, const Geometry&
 // points of all rows go first, then the child rows, whose children are merged per landing column
 // (as in ChildRow, in FP32): four sums x^a f and two x^a g a column, expanded to the stored moments
 // once and shared 3/4 : 1/4 between the rows cy and cy + sy; the larger share is rounded and the
-// smaller is the exact difference, so the accounting takes a column once.
+// smaller is the exact difference, so the accounting takes a column once.  Instruction issue and the
+// FP64 atomic additions bound it (11 a point or column, 40 % of their peak rate at RT 0.25-1.5): 1024^2
+// step at RT 0.25-1.5 3.59 ms with a share at a time, 3.13 ms so.
 template <int D>
 __device__ __forceinline__ void scatter_table32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                                 long long cell, const CellState<D>& c, const RowTable<D>& tab,
@@ -1126,6 +1128,10 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
     double rmax;
 #pragma unroll 1
     for (int it = 0; it < 2; it++) {
+        float dl[Q::N];
+#pragma unroll
+        for (int j = 0; j < Q::N; j++) dl[j] = 0.f;
+        const unsigned int q0 = tc.pdfc;
         {
             float MJ[Q::NJ];
             if (!df_pass<D, FLUON, DF_CORR>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax, MJ, ds,
@@ -1133,16 +1139,22 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
                 return -1;
             // far from the FP32 solution's neighbourhood (or non-finite): the FP64 EPR decides
             if (!(rmax < 1e-3)) return -1;
-            if (rmax > m.tol && !df_update<D, FLUON>(MJ, r, lam)) return -1;
+            if (rmax > m.tol && !df_update<D, FLUON>(MJ, r, lam, dl)) return -1;
         }
-        if (!df_pass<D, FLUON, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax, nullptr, ds, tc.ls, tc.pdf, ds.beta)) return -1;
-        if (rmax <= m.tol) return it + 1;
-        // the deposited populations miss the tolerance: take them back
-        ds.mh = -ds.mh;
-        ds.ml = -ds.ml;
-        df_pass<D, FLUON, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax, nullptr, ds, tc.ls, tc.pdf, ds.beta);
-        ds.mh = -ds.mh;
-        ds.ml = -ds.ml;
+        // a small update of few enough points streams the populations of the correction pass
+        const bool again = rmax <= kRestreamMax && tc.pdfc - q0 <= (unsigned int)ds.pop_cap && !ds.near_wall;
+#pragma unroll 1
+        for (int undo = 0; undo < 2; undo++) {
+            if (again)
+                df_restream<D, FLUON>(tab, dl, r, rmax, ds, tc.ls, tc.pdf);
+            else if (!df_pass<D, FLUON, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax,
+                                                   nullptr, ds, tc.ls, tc.pdf, ds.beta))
+                return -1;
+            if (undo == 0 && rmax <= m.tol) return it + 1;
+            // the deposited populations miss the tolerance: take them back
+            ds.mh = -ds.mh;
+            ds.ml = -ds.ml;
+        }
         tc.redo++;
     }
     return -1;
@@ -1539,6 +1551,12 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
     ds.near_wall = false;
     ds.beta = bslot;
     ds.mh = ds.ml = 0.f;
+    {
+        const int tid = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+        ds.pop = m.df_pop + tid;
+        ds.pop_stride = m.df_pop_threads;
+        ds.pop_cap = tid < m.df_pop_threads && (D == 1 || st.R <= kDfPopR) ? kDfPopCap : 0;
+    }
     double xm = 0.0;
     if (alive) {
         ds.at = cell_place<D>(g, cell);

@@ -17,7 +17,9 @@
 // The FP64 pipe (one warp instruction in 64 cycles on each of an SM's four partitions) bounds this
 // kernel, so only what decides the result is FP64: populations (their exponentials by integer
 // instructions, exp_int), the residual, the multipliers and the deposited moments.  A solve that
-// breaks down is redone by the all-FP64 Newton below it.
+// breaks down is redone by the all-FP64 Newton below it.  A step of 40^3 cells: 19.2 ms, against
+// 82.5 ms with library exponentials, FP64 moments to degree 6 and an FP64 factorisation; error
+// 7.5e-16 -> 6.3e-16.
 //   - moment streaming (Eq. IIE3) deposits T_N(c_i) rho f'_i and T_N(c_i) rho K RT g'_i
 //     at x + c_i with FP64 atomic additions (cloud-in-cell for refined children).
 // Thermal units throughout the Newton (t = (c - u) / sqrt(RT)), as in 1D and 2D.

@@ -88,8 +88,9 @@ constexpr long long kInfBits = 0x7ff0000000000000LL;
 // ---------------------------------------------------------------------------
 // Reciprocals and quotients.  The library's FP64 division takes about nine instructions of the FP64
 // pipe; a reciprocal from the FP32 one and two Newton steps takes four (24 -> 48 -> 53 bits, within
-// one ulp), and a quotient by a divisor whose reciprocal is known three (Markstein's correction, correctly
-// rounded like __ddiv_rn).
+// one ulp), and a quotient by a divisor whose reciprocal is known three (Markstein's correction, the
+// rounding of __ddiv_rn but in rare cases, where it is off by one ulp).  With the other per-cell FP64
+// savings beside them: 512^2 FP64 step at RT 0.6 3.54 -> 3.26 ms, 1024^2 mixed step 4.83 -> 4.29 ms.
 // ---------------------------------------------------------------------------
 // Is v positive, normal and within 2^+-99, the range of the short forms?
 __device__ __forceinline__ bool recip_range(double v) { return (unsigned)(__double2hiint(v) >> 20) - 924u < 198u; }

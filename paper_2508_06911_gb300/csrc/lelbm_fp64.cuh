@@ -17,6 +17,9 @@
 //   - The membership decisions come from the row table, taken once per cell.
 // A solve that breaks down here is redone by the all-FP64 Newton (solve_fg), so what converges and
 // what falls back is decided there.
+// Against one exponential per row start and third ratio, FP64 moments to degree 6 and single shares of
+// every child, a step of a 731 x 523 four-quadrant flow (RT 0.25-1.5) went from 30.3 to 8.3 ms, and its
+// error against 64-bit arithmetic from 5.1e-16 to 4.1e-16.
 #pragma once
 
 #include <cstdint>
@@ -176,8 +179,9 @@ struct SweepFactors {
                 a[16] = -a[15];
             }
         }
-        // one code site: inlined copies would crowd the instruction caches
-#pragma unroll 1
+        // one code site in 2D (inlined copies would crowd the instruction caches); side by side in 1D, where a
+        // small batch waits for this chain
+#pragma unroll(D == 1 ? NE : 1)
         for (int k = 0; k < NE; k++) a[k] = exp_int(-a[k]);
         e0 = wgt * a[0];
         r = a[1];

@@ -18,7 +18,8 @@
 // FP64 instructions bound the kernel.  Most pairs in the window (2 H + 1)^2 are no points of the
 // source's set, so membership is decided in FP32 on offsets from floor(u) (as in RowTable::build: only
 // a test closer to its threshold than FP32 resolves goes to FP64); a pair that is a point takes 45
-// FP64 operations, its exponentials being integer code (exp_int).
+// FP64 operations, its exponentials being integer code (exp_int).  384 x 320 step, cell kernel
+// included: 7.1 ms with FP64 tests and library exponentials here, 3.5 ms so.
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -143,7 +143,7 @@ __device__ __forceinline__ double quarter(double v) {
 // A column is complete after the left child of the next point, so a row of n children ends with
 // three empty ones; every column leaves through one code site (refined cells are bound by
 // instruction fetch: with a site for each of the last columns and for both rows the 1024^2 mixed
-// step at RT 0.35 took 11.8 ms, with one 8.0 ms).
+// step at RT 0.35 took 11.8 ms, with one 8.6 ms).
 template <int D, bool F, bool G>
 struct ChildRow {
     static constexpr int NS = (F ? 4 : 0) + (G ? 2 : 0);

@@ -44,7 +44,9 @@ __global__ void to_bf16_kernel(const float* src, __nv_bfloat16* dst, int n) {
 // derivatives of SiLU wait in registers.  Blocks are persistent: each keeps the whole gradient in
 // registers (a tile's sums are formed on their own, then added) and adds it to grad once, instead of
 // one atomic addition per parameter and 64 samples.  Two blocks share an SM, so one computes while the
-// other waits at a barrier.  2^20 pairs in 2D: see the launch bounds' note for times.
+// other waits at a barrier.  FP32 FMAs and
+// the shared-memory loads between them bound it (35 kFLOP a sample): 2^20 pairs in 2D take 1.29 ms, 28 TFLOP/s,
+// where one thread per sample took 9.17 ms.
 constexpr int kGradThreads = 128;
 constexpr int kLD = TB + 4;  // row stride of the transposed tiles: float4 rows that start 4 banks apart
 
@@ -82,8 +84,8 @@ __device__ __forceinline__ void store_column(float* row, const float (&v)[8][4],
     *reinterpret_cast<float4*>(row + 4) = make_float4(v[4][c], v[5][c], v[6][c], v[7][c]);
 }
 
-// Sums over the tile's samples of A[ia][s] B[ib + 16... ][s]: out[r] += sum_s a[s] B_r[s], R rows of B
-// LDB floats apart.
+// out[r] += sum_s a[s] B[r][s] over the samples s of a tile: one row a, R rows of B that lie
+// ldb floats apart.
 template <int R>
 __device__ __forceinline__ void sample_sums(const float* a, const float* B, int ldb, float (&out)[R]) {
     float t[R];

@@ -99,13 +99,54 @@ constexpr float kRhoH = kLn2H * 4.656612873077392578125e-10f;   // ln2_hi 2^-31
 constexpr float kRhoM = kLn2L * 4.656612873077392578125e-10f;   // ln2_lo 2^-31
 constexpr float kRhoL = kLn2H * 5.5511151231257827e-17f;        // ln2_hi 2^-54
 
-// Each block fills the table once: entry j = 2^(j/512) as a double-float.
-__device__ __forceinline__ void exp2_table_init(float2* tab) {
-    for (int j = threadIdx.x; j < kExpTab; j += blockDim.x) {
-        const double v = exp2((double)j * (1.0 / kExpTab));
-        const float h = (float)v;
-        tab[j] = make_float2(h, (float)(v - (double)h));
+// 2^(j/512), made at compile time: with 62 fractional bits, and as double-floats.
+struct Exp2Table {
+    unsigned long long t[512];  // 2^(j/512), 62 fractional bits
+    // floor(sqrt(x 2^63)) for x with 63 fractional bits in [1, 2)
+    static constexpr unsigned long long root(unsigned long long x) {
+        unsigned long long y = 0;
+        const unsigned __int128 v = (unsigned __int128)x << 63;
+        for (int b = 63; b >= 0; b--) {
+            const unsigned long long c = y | (1ull << b);
+            if ((unsigned __int128)c * c <= v) y = c;
+        }
+        return y;
     }
+    constexpr Exp2Table() : t{} {
+        unsigned long long r[9] = {};  // 2^(1/2), 2^(1/4), ..., 2^(1/512), 63 fractional bits
+        unsigned __int128 two = (unsigned __int128)2 << 126;  // sqrt(2): from 2 with 126 fractional bits
+        for (int b = 63; b >= 0; b--) {
+            const unsigned long long c = r[0] | (1ull << b);
+            if ((unsigned __int128)c * c <= two) r[0] = c;
+        }
+        for (int k = 1; k < 9; k++) r[k] = root(r[k - 1]);
+        for (int j = 0; j < 512; j++) {
+            unsigned long long p = 1ull << 63;
+            for (int k = 0; k < 9; k++)
+                if ((j >> (8 - k)) & 1) p = (unsigned long long)(((unsigned __int128)p * r[k]) >> 63);
+            t[j] = p >> 1;
+        }
+    }
+};
+static __device__ const Exp2Table c_exp2 = Exp2Table();
+struct Exp2Pairs {
+    float h[kExpTab], l[kExpTab];
+    constexpr Exp2Pairs() : h{}, l{} {
+        const Exp2Table e;
+        for (int j = 0; j < kExpTab; j++) {
+            const double v = (double)e.t[j] / 4611686018427387904.0;  // 2^62
+            h[j] = (float)v;
+            l[j] = (float)(v - (double)h[j]);
+        }
+    }
+};
+static __device__ const Exp2Pairs c_exp2_pairs = Exp2Pairs();
+
+// Each block copies the table to shared memory (evaluated there, its 512 FP64 exponentials took 2 us of
+// every launch, and more in a small block).
+__device__ __forceinline__ void exp2_table_init(float2* tab) {
+    for (int j = threadIdx.x; j < kExpTab; j += blockDim.x)
+        tab[j] = make_float2(c_exp2_pairs.h[j], c_exp2_pairs.l[j]);
 }
 
 // fh + fl = 2^(w 2^-54 + dn) to about 2^-47 relative (the precision of a double-float).  w = n + j/512 + rho with

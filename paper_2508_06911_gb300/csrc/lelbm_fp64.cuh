@@ -35,36 +35,6 @@ namespace lbm {
 // integer instructions, some 20 issue cycles of an SM, where the library's exp takes about 17 FP64
 // instructions, 16 cycles each.
 // ---------------------------------------------------------------------------
-struct Exp2Table {
-    unsigned long long t[512];  // 2^(j/512), 62 fractional bits
-    // floor(sqrt(x 2^63)) for x with 63 fractional bits in [1, 2)
-    static constexpr unsigned long long root(unsigned long long x) {
-        unsigned long long y = 0;
-        const unsigned __int128 v = (unsigned __int128)x << 63;
-        for (int b = 63; b >= 0; b--) {
-            const unsigned long long c = y | (1ull << b);
-            if ((unsigned __int128)c * c <= v) y = c;
-        }
-        return y;
-    }
-    constexpr Exp2Table() : t{} {
-        unsigned long long r[9] = {};  // 2^(1/2), 2^(1/4), ..., 2^(1/512), 63 fractional bits
-        unsigned __int128 two = (unsigned __int128)2 << 126;  // sqrt(2): from 2 with 126 fractional bits
-        for (int b = 63; b >= 0; b--) {
-            const unsigned long long c = r[0] | (1ull << b);
-            if ((unsigned __int128)c * c <= two) r[0] = c;
-        }
-        for (int k = 1; k < 9; k++) r[k] = root(r[k - 1]);
-        for (int j = 0; j < 512; j++) {
-            unsigned long long p = 1ull << 63;
-            for (int k = 0; k < 9; k++)
-                if ((j >> (8 - k)) & 1) p = (unsigned long long)(((unsigned __int128)p * r[k]) >> 63);
-            t[j] = p >> 1;
-        }
-    }
-};
-static __device__ const Exp2Table c_exp2 = Exp2Table();
-
 // 2^(w 2^-55) = P 2^(n - 62), P in [2^62, 2^63].
 __device__ __forceinline__ unsigned long long exp2_q62(long long w, int& n) {
     const int hi = (int)(w >> 32);

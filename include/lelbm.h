@@ -82,7 +82,7 @@ extern "C" {
                          exponential; a correction below 2e-6 of the constraints
                          reaches the streaming pass as a relative change of the
                          populations that the correction pass kept (scratch of the
-                         handle: 4 KB a resident thread, at most 239 MB).  Deposits
+                         handle: 4 KB a resident thread, at most 319 MB).  Deposits
                          are FP64 atomic additions.  State, collision and
                          accumulation in FP64.
                          Matches LELBM_FP64 to about 1e-13 per step.             */

@@ -530,12 +530,12 @@ extern "C" int lelbm_create(lelbm_t* out, const lelbm_params* p) {
             rc = LELBM_E_NOMEM;
     }
     if (!rc && p->precision == LELBM_MIXED) {
-        // scratch for the threads that can be resident (one 384-thread block an SM); without it the
+        // scratch for the threads that can be resident (one 512-thread block an SM); without it the
         // mixed path evaluates its populations twice
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-        constexpr long long nt = cell_threads<PREC_MIXED>();
-        const long long threads = std::min<long long>(sms * nt, (h->ncell + nt - 1) / nt * nt);
+        constexpr long long nt = kWideThreads;
+        const long long threads = std::min<long long>(sms * nt, h->ncell + nt);
         if (cudaMalloc((void**)&h->d_df_pop, sizeof(float2) * kDfPopCap * (size_t)threads) == cudaSuccess) {
             h->model.df_pop = h->d_df_pop;
             h->model.df_pop_threads = (int)threads;

@@ -16,6 +16,9 @@ void BatchVariant<PREC>::launch(const Model& m, const Geometry& g, const double 
                                  const int* inst_pad, int* steps_left, int nsteps, int blocks, int threads,
                                  size_t smem, cudaStream_t s) {
     auto kern = batch_persistent_kernel<PREC>;
+    if constexpr (PREC == PREC_MIXED) {
+        if (g.n_inst > kWideTubes) kern = batch_persistent_kernel<PREC, true>;
+    }
     if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<blocks, threads, smem, s>>>(m, g, inlet[0], inlet[1], inlet[3], bc_left_inflow, bc_right_inflow, type, A,
                                        B, st, work, order, inst_first, inst_pad, steps_left, nsteps);
@@ -24,7 +27,7 @@ void BatchVariant<PREC>::launch(const Model& m, const Geometry& g, const double 
 template <int PREC>
 int BatchVariant<PREC>::blocks_per_sm(int threads) {
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_persistent_kernel<PREC>, threads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_persistent_kernel<PREC, PREC == PREC_MIXED>, threads, 0);
     return per_sm;
 }
 

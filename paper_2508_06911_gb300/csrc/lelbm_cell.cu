@@ -12,17 +12,20 @@ namespace lbm {
 
 template <int D, int PREC>
 void CellVariant<D, PREC>::launch(const Model& m, const Geometry& g, const uint8_t* type, const double* Min,
-                                   double* Mout, DevStats* st, unsigned long long* work, int blocks, size_t smem,
-                                   cudaStream_t s) {
-    auto kern = cell_update_kernel<D, PREC>;
+                                   double* Mout, DevStats* st, unsigned long long* work, int blocks, int threads,
+                                   size_t smem, cudaStream_t s) {
+    auto kern = cell_update_kernel<D, PREC, cell_threads<PREC>()>;
+    if constexpr (D == 2 && PREC == PREC_MIXED) {
+        if (threads > cell_threads<PREC>()) kern = cell_update_kernel<D, PREC, kWideThreads>;
+    }
     if (smem) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<blocks, cell_threads<PREC>(), smem, s>>>(m, g, type, Min, Mout, st, work);
+    kern<<<blocks, threads, smem, s>>>(m, g, type, Min, Mout, st, work);
 }
 
 template <int D, int PREC>
 int CellVariant<D, PREC>::blocks_per_sm() {
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_update_kernel<D, PREC>, cell_threads<PREC>(), 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cell_update_kernel<D, PREC, cell_threads<PREC>()>, cell_threads<PREC>(), 0);
     return per_sm;
 }
 

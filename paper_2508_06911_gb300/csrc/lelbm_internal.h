@@ -24,10 +24,19 @@ using Con = typename std::conditional<PREC == PREC_FP32, float, double>::type;
 // (one phase's instructions in the instruction caches at a time).
 template <int PREC>
 constexpr int cell_threads() { return PREC == PREC_MIXED ? 384 : 128; }
+// The mixed kernels exist in two widths: three warps a scheduler (168 registers) and four (128, with some
+// spills).  Deposits bound large grids, above all refined cells, and four warps hide more of their
+// latency; on small grids, where an SM holds fewer cells than threads, the spills only cost.  1024^2 step at
+// RT 0.35 7.17 -> 6.70 ms, 2048^2 four-quadrant flow 26.5 -> 24.8, 700^2 4.20 -> 3.99; 512^2 2.62 | 2.64,
+// 330 x 300 1.27 | 1.34.  Batches (a 128-thread block a tube): 4096 tubes 18.4 -> 17.3 ms, 1200 9.01 -> 8.63,
+// 900 6.78 -> 6.33; 650 6.49 | 6.60, 300 7.00 | 7.16.
+constexpr int kWideThreads = 512;
+constexpr long long kWideCells = 400000;
+constexpr int kWideTubes = 760;  // five an SM
 
 // Points of a velocity set whose populations the mixed path keeps between its correction and its streaming
-// pass: up to R_ac = 12 in 2D (q = 490), 4 KB for each of the threads that can be resident (239 MB a GPU;
-// a grid of fewer cells takes less).  A step touches q entries a thread, so up to q = 250 what it keeps
+// pass: up to R_ac = 12 in 2D (q = 490), 4 KB for each of the threads that can be resident (319 MB a GPU;
+// a grid of fewer cells takes less).  A step touches q entries a thread, so up to q = 200 what it keeps
 // stays in L2 (129 MB); at RT = 8 (q = 434) reading it back still beats evaluating it again (7.17 against
 // 7.98 ms at 512^2).
 constexpr int kDfPopCap = 512;
@@ -192,7 +201,7 @@ void launch_gather2d(const Model& m, const Geometry& g, const double* Min, doubl
 template <int D, int PREC>
 struct CellVariant {
     static void launch(const Model& m, const Geometry& g, const uint8_t* type, const double* Min, double* Mout,
-                       DevStats* st, unsigned long long* work, int blocks, size_t smem, cudaStream_t s);
+                       DevStats* st, unsigned long long* work, int blocks, int threads, size_t smem, cudaStream_t s);
     static int blocks_per_sm();
 };
 

@@ -3,6 +3,7 @@
 // kernels live in lelbm_cell.cu (cell update) and lelbm_batch.cu (persistent
 // 1D batch), one object per variant.
 
+#include <algorithm>
 #include <cstdint>
 
 #include "lelbm_device.cuh"
@@ -145,26 +146,32 @@ int cell_update_blocks(int D, int prec, int device) {
 
 template <int D>
 static void cell_launch(int prec, const Model& m, const Geometry& g, const uint8_t* type, const double* Min,
-                        double* Mout, DevStats* st, unsigned long long* work, int blocks, size_t sm, cudaStream_t s) {
+                        double* Mout, DevStats* st, unsigned long long* work, int blocks, int threads, size_t sm,
+                        cudaStream_t s) {
     if (prec == PREC_MIXED)
-        CellVariant<D, PREC_MIXED>::launch(m, g, type, Min, Mout, st, work, blocks, sm, s);
+        CellVariant<D, PREC_MIXED>::launch(m, g, type, Min, Mout, st, work, blocks, threads, sm, s);
     else if (prec == PREC_FP32)
-        CellVariant<D, PREC_FP32>::launch(m, g, type, Min, Mout, st, work, blocks, sm, s);
+        CellVariant<D, PREC_FP32>::launch(m, g, type, Min, Mout, st, work, blocks, threads, sm, s);
     else
-        CellVariant<D, PREC_FP64>::launch(m, g, type, Min, Mout, st, work, blocks, sm, s);
+        CellVariant<D, PREC_FP64>::launch(m, g, type, Min, Mout, st, work, blocks, threads, sm, s);
 }
 
 void launch_cell_update(const Model& m, const Geometry& g, const uint8_t* type, const double* Min, double* Mout,
                         DevStats* st, unsigned long long* work, int grid_blocks, int prec, cudaStream_t s) {
-    const int nt = prec == PREC_MIXED ? cell_threads<PREC_MIXED>() : 128;
-    long long need = (g.ncell + nt - 1) / nt;
-    int blocks = (int)(need < grid_blocks ? need : grid_blocks);
-    if (blocks < 1) blocks = 1;
+    // A grid too small to fill the resident blocks is dealt out to all SMs in smaller ones: 60 x 50 mixed
+    // step 0.76 -> 0.69 ms.
+    const int full = prec != PREC_MIXED                    ? 128
+                     : g.D == 2 && g.ncell >= kWideCells ? kWideThreads
+                                                         : cell_threads<PREC_MIXED>();
+    const long long share = (g.ncell + grid_blocks - 1) / grid_blocks;
+    const int nt = share >= full ? full : share > 32 ? ((int)share + 63) / 64 * 64 : 32;
+    const long long need = (g.ncell + nt - 1) / nt;
+    const int blocks = (int)std::max<long long>(1, std::min<long long>(need, grid_blocks));
     const size_t sm = 0;  // the learned start runs in mlp_start_kernel, not in the cell update
     if (g.D == 1)
-        cell_launch<1>(prec, m, g, type, Min, Mout, st, work, blocks, sm, s);
+        cell_launch<1>(prec, m, g, type, Min, Mout, st, work, blocks, nt, sm, s);
     else
-        cell_launch<2>(prec, m, g, type, Min, Mout, st, work, blocks, sm, s);
+        cell_launch<2>(prec, m, g, type, Min, Mout, st, work, blocks, nt, sm, s);
 }
 
 void launch_eq_state(int D, double K, const uint8_t* type, const double* rho, const double* u, const double* RT,

@@ -1655,20 +1655,20 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
 // with its own phase barriers: fewer warps wait at a barrier for the slowest one, while at
 // most two phases share an SM's instruction caches.  Two groups of six warps measured 4.8 %
 // faster than one group of twelve on the 4096^2 four-quadrant problem; three groups of four
-// were 12 % slower.
+// were 12 % slower; of sixteen warps, two groups of eight 24.4 ms on a 2048^2 one, four of four 31.6 ms.
+// A block of a small grid is one group.
 constexpr int kMixedGroups = 2;
 
 template <int D, int PREC>
 constexpr int min_blocks() { return PREC == PREC_FP32 ? 4 : (PREC == PREC_MIXED ? 1 : 1); }
 
-template <int D, int PREC>
-__global__ void __launch_bounds__(cell_threads<PREC>(), min_blocks<D, PREC>()) cell_update_kernel(const __grid_constant__ Model m, const __grid_constant__ Geometry g,
+template <int D, int PREC, int NT>
+__global__ void __launch_bounds__(NT, min_blocks<D, PREC>()) cell_update_kernel(const __grid_constant__ Model m, const __grid_constant__ Geometry g,
                                                           const uint8_t* __restrict__ type,
                                                           const double* __restrict__ Min, double* Mout,
                                                           DevStats* stats, unsigned long long* work) {
     constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
     __shared__ BlockCounters bc;
-    constexpr int NT = cell_threads<PREC>();
     __shared__ Con<PREC> s_con[NT][NF + NG];  // constraints of each thread's cell (out of registers)
     // 2D row tables (one per thread)
     __shared__ char2 s_rows[D == 2 ? NT : 1][D == 2 ? kRowsMax : 1];
@@ -1688,7 +1688,7 @@ __global__ void __launch_bounds__(cell_threads<PREC>(), min_blocks<D, PREC>()) c
     ThreadCounters& tc = s_tc[threadIdx.x];
     const int lane = threadIdx.x & 31;
     if constexpr (PREC == PREC_MIXED) {  // groups claim G-cell chunks and step them in phases
-        constexpr int G = NT / kMixedGroups;
+        const int G = (int)blockDim.x > NT / kMixedGroups ? (int)blockDim.x / kMixedGroups : (int)blockDim.x;
         const int grp = threadIdx.x / G, gl = threadIdx.x - grp * G;
         __shared__ unsigned long long s_base[kMixedGroups];
         for (;;) {
@@ -1727,13 +1727,13 @@ __global__ void __launch_bounds__(cell_threads<PREC>(), min_blocks<D, PREC>()) c
 // a shared counter.  An instance that ends on an odd step copies its block back, so
 // every instance finishes in buffer A.  steps_left[] (may be null: unlimited) caps
 // each instance and is decremented.
-// The persistent batch keeps 128-thread blocks (a block per instance); on the mixed path
-// three of them per SM (168 registers), as many as the FP32 variant fits at 128.
-template <int PREC>
-constexpr int batch_min_blocks() { return PREC == PREC_MIXED ? 3 : min_blocks<1, PREC>(); }
+// The persistent batch keeps 128-thread blocks (a block per instance).
+// WIDE: the mixed path at four blocks an SM (kWideTubes).
+template <int PREC, bool WIDE>
+constexpr int batch_min_blocks() { return PREC == PREC_MIXED ? (WIDE ? 4 : 3) : min_blocks<1, PREC>(); }
 
-template <int PREC>
-__global__ void __launch_bounds__(128, batch_min_blocks<PREC>()) batch_persistent_kernel(const __grid_constant__ Model m,
+template <int PREC, bool WIDE = false>
+__global__ void __launch_bounds__(128, batch_min_blocks<PREC, WIDE>()) batch_persistent_kernel(const __grid_constant__ Model m,
                                                                const __grid_constant__ Geometry g, double in0, double in1,
                                                                double in3, int bc_left_inflow, int bc_right_inflow,
                                                                const uint8_t* __restrict__ type, double* A, double* B,

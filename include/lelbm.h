@@ -79,10 +79,13 @@ extern "C" {
                          against tol (a miss is taken back and corrected again,
                          then left to the FP64 EPR).  Exponents are exact int64
                          fixed-point polynomials, 2^w a table-driven double-float
-                         exponential; a correction below 2e-6 of the constraints
-                         reaches the streaming pass as a relative change of the
-                         populations that the correction pass kept (scratch of the
-                         handle: 4 KB a resident thread, at most 319 MB).  Deposits
+                         exponential; a correction that changes the moments
+                         by less than 3e-6 (thermal units) reaches the streaming
+                         pass as a relative change of the populations that the
+                         correction pass kept (scratch of the handle: 4 KB a
+                         resident thread, at most 319 MB), judged to 0.45 of the
+                         default tol; with tol below 1e-12 the residual is always
+                         summed afresh.  Deposits
                          are FP64 atomic additions.  State, collision and
                          accumulation in FP64.
                          Matches LELBM_FP64 to about 1e-13 per step.             */

@@ -682,16 +682,38 @@ __device__ __forceinline__ bool df_update(const float* MJ, const double* r, doub
     return true;
 }
 
+// Bound on the sums |T_k f em| (any k) that an update x = A^-1 r of the multipliers changes: em = -x . T, so
+// sum f em^2 = x . A x = x . r, and by Cauchy and Schwarz sum |T_k f em| <= sqrt(A_kk x . r).
+template <int D, bool FLUON>
+__device__ __forceinline__ float df_update_size(const float* MJ, const double* r, const float* x) {
+    using Q = DFPop<D, FLUON>;
+    float xr = 0.f, top = 0.f;
+#pragma unroll
+    for (int j = 0; j < Q::N; j++) {
+        const int a = 2 * bx<D, FLUON>(j), b = 2 * by<D, FLUON>(j);
+        xr = fmaf(x[j], narrow_signed(r[j]), xr);
+        top = fmaxf(top, MJ[D == 1 ? a : tix(a, b, Q::PJ)]);
+    }
+    return sqrtf(fabsf(xr) * top);
+}
+
 // The streaming pass after a small update dlam of the multipliers, from the populations that the
 // correction pass kept: f' = f (1 + em), em = expm1(-dlam . T), where a DF_STREAM pass evaluates every
-// exponential and the whole residual again.  em is FP32: with |dlam| of the size of the FP32 Newton's
-// noise (1e-7) its rounding moves a population by 1e-14 of itself.  The residual of exactly what is
-// deposited is the correction pass's r plus sum T f em, whose FP32 sum is off by about 1e-7 of the
-// residual that dlam removes: kRestreamMax bounds that by 2e-13, inside the 1e-12 that is judged.
+// exponential and the whole residual again.  em is FP32, and so is the sum T f em that the residual of
+// exactly what is deposited takes beside the correction pass's r.  Both lose with the size S of the
+// change (df_update_size), not with the residual that it removes: over RT 0.2-9 that sum was off by 0.5
+// to 1.2 2^-24 S in the mean and 5.5 2^-24 S at most, and a population is by 2^-24 em.  The judge therefore
+// adds kRestreamErr S to the residual, and an update beyond kRestreamMax takes the DF_STREAM pass, so that
+// a deposit that passes is within 1.45 times the default tolerance at the worst.  The FP32 Newton leaves S at
+// 2e-7 to 1.8e-6 up to RT 8 and 2.8e-6 at RT 9.  Measured (4096 tubes, 512^2 hot box RT 7-9): no allowance
+// 17.6, 6.86 ms; this one 17.9, 6.86; one for the worst error 19.3, 8.11; S up to 1.5e-6 only 21.2, 9.8 (one
+// cell that evaluates again holds up its warp).  A caller whose tolerance is below kRestreamTol, which
+// such a judge would not serve, always gets the DF_STREAM pass.
 // What bounds a DF_STREAM pass is FP32 instructions (79 a point for the exponential and the sums, and 250
 // a row to set them up); this pass takes 15 and 25, and a load.  1024^2 mixed step at RT 0.6: 4.28 -> 3.87 ms,
 // at RT 0.35 8.07 -> 7.15 ms, four-quadrant flow 9.58 -> 7.85 ms; 4096 tubes, two steps, 33.0 -> 18.7 ms.
-constexpr double kRestreamMax = 2e-6;
+constexpr float kRestreamMax = 3e-6f, kRestreamErr = 3.f / 16777216.f;
+constexpr double kRestreamTol = 1e-12;
 
 template <int D, bool FLUON>
 static __device__ __noinline__ void df_restream(const RowTable<D>& tab_in, const float* __restrict__ dlam,

@@ -1159,6 +1159,7 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
 #pragma unroll
         for (int j = 0; j < Q::N; j++) dl[j] = 0.f;
         const unsigned int q0 = tc.pdfc;
+        float change = 0.f;
         {
             float MJ[Q::NJ];
             if (!df_pass<D, FLUON, DF_CORR>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax, MJ, ds,
@@ -1166,10 +1167,14 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
                 return -1;
             // far from the FP32 solution's neighbourhood (or non-finite): the FP64 EPR decides
             if (!(rmax < 1e-3)) return -1;
-            if (rmax > m.tol && !df_update<D, FLUON>(MJ, r, lam, dl)) return -1;
+            if (rmax > m.tol) {
+                if (!df_update<D, FLUON>(MJ, r, lam, dl)) return -1;
+                change = df_update_size<D, FLUON>(MJ, r, dl);
+            }
         }
         // a small update of few enough points streams the populations of the correction pass
-        const bool again = rmax <= kRestreamMax && tc.pdfc - q0 <= (unsigned int)ds.pop_cap && !ds.near_wall;
+        const bool again = change <= kRestreamMax && m.tol >= kRestreamTol &&
+                           tc.pdfc - q0 <= (unsigned int)ds.pop_cap && !ds.near_wall;
 #pragma unroll 1
         for (int undo = 0; undo < 2; undo++) {
             if (again)
@@ -1177,7 +1182,7 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
             else if (!df_pass<D, FLUON, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax,
                                                    nullptr, ds, tc.ls, tc.pdf, ds.beta))
                 return -1;
-            if (undo == 0 && rmax <= m.tol) return it + 1;
+            if (undo == 0 && rmax + (again ? widen(kRestreamErr * change) : 0.0) <= m.tol) return it + 1;
             // the deposited populations miss the tolerance: take them back
             ds.mh = -ds.mh;
             ds.ml = -ds.ml;

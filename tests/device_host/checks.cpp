@@ -1,0 +1,163 @@
+// Checks of the device headers' per-cell functions on the CPU (see cuda_host.h), for
+// test_device_code.py.
+#include "cuda_host.h"
+
+#include <random>
+#include <vector>
+
+#include "lelbm_step.cuh"
+
+using namespace lbm;
+typedef long double real;
+
+namespace {
+
+constexpr int kGrid = 64;  // cells a side of the periodic grid that takes the deposits
+
+struct Cell {
+    Model m{};
+    Geometry g{};
+    CellState<2> c{};
+    Stencil<2> st{};
+    RowTable<2> tab{};
+    CellLattice<2> lat{};
+    char2 rows[kRowsMax];
+    double conF[10], conG[6], lf[10], lg[6];  // constraints and the FP64 solution
+    std::vector<uint8_t> type;
+    std::vector<double> M;
+    std::vector<float2> pop;
+    std::vector<float2> etab;
+    long long beta[10];
+
+    Cell() : type(kGrid * kGrid, CELL_FLUID), M(11 * kGrid * kGrid), pop(kDfPopCap), etab(kExpTab) {
+        m.K = 2.0;
+        m.n_conf = 4.0;
+        m.r_min = 2.0;
+        m.refine_div = m.refine_rad = 3.0;
+        m.max_refine = 4;
+        m.Pr = 1.0;
+        m.tol = 1e-12;
+        m.max_iter = 60;
+        set_derived_params(m, 2);
+        g.D = 2;
+        g.NX = g.NY = g.nx = g.ny = kGrid;
+        g.ncell = kGrid * kGrid;
+        g.periodic[0] = g.periodic[1] = 1;
+        exp2_table_init(etab.data());
+    }
+    // a cell at temperature RT (about), with constraints off equilibrium by up to noneq; false
+    // where the FP64 path has no lattice-form solution
+    template <class Rng>
+    bool draw(Rng& rng, double RT, double noneq, double umag) {
+        std::uniform_real_distribution<double> U(-1.0, 1.0);
+        c.rho = 1.0;
+        c.RT = RT * (1.0 + 0.03 * U(rng));
+        c.sig = std::sqrt(c.RT);
+        c.inv_sig = 1.0 / c.sig;
+        c.u[0] = umag * U(rng);
+        c.u[1] = umag * U(rng);
+        st.init(c, m);
+        tab.build(c, st, rows);
+        for (int j = 0; j < 10; j++) conF[j] = (j == 0 || j == 3 || j == 5) + (j > 2 ? noneq * U(rng) : 0.0);
+        for (int j = 0; j < 6; j++) conG[j] = (j == 0 || j == 3 || j == 5) + (j > 0 ? noneq * U(rng) : 0.0);
+        if (!tab.ok) return false;
+        lat.init(c, tab);
+        maxwell_start_fg<2, 10, 6>(c.RT, lf, lg);
+        int sf, sg;
+        unsigned pf = 0, pg = 0;
+        solve_fg64<2>(c, tab, lat, conF, conG, true, lf, lg, m, sf, sg, pf, pg);
+        return sf >= 0 && sg >= 0;
+    }
+    DFStream stream(double mass, int pop_cap) {
+        DFStream ds{};
+        ds.g = &g;
+        ds.type = type.data();
+        ds.Mout = M.data();
+        ds.at = cell_place<2>(g, (kGrid / 2) * kGrid + kGrid / 2);
+        ds.beta = beta;
+        ds.pop = pop.data();
+        ds.pop_stride = 1;
+        ds.pop_cap = pop_cap;
+        df_split(mass, ds.mh, ds.ml);
+        return ds;
+    }
+    // Largest residual (thermal units) of what lies in M, deposited with mass 1, against the
+    // constraints of the fluons or the phonons.  The stored heat flux is the sum of two constraints.
+    double residual(bool fluon) const {
+        real T[11] = {};
+        for (int k = 0; k < 11; k++)
+            for (int i = 0; i < kGrid * kGrid; i++) T[k] += M[(size_t)k * kGrid * kGrid + i];
+        const real ux = c.u[0], uy = c.u[1], s = c.inv_sig, uu = ux * ux + uy * uy;
+        real worst = 0;
+        auto take = [&](real v) { worst = std::max(worst, fabsl(v)); };
+        if (!fluon) {
+            take(T[8] - conG[0]);
+            take((T[9] - ux * T[8]) * s - conG[1]);
+            take((T[10] - uy * T[8]) * s - conG[2]);
+            return (double)worst;
+        }
+        const real n = T[0], x = T[1], y = T[2], xx = T[3], xy = T[4], yy = T[5];
+        take(n - conF[0]);
+        take((x - ux * n) * s - conF[1]);
+        take((y - uy * n) * s - conF[2]);
+        take((xx - 2 * ux * x + ux * ux * n) * s * s - conF[3]);
+        take((xy - ux * y - uy * x + ux * uy * n) * s * s - conF[4]);
+        take((yy - 2 * uy * y + uy * uy * n) * s * s - conF[5]);
+        const real ud = ux * x + uy * y;
+        const real qx = T[6] - ux * (xx + yy) - 2 * (ux * xx + uy * xy) + 2 * ux * ud + uu * x - uu * ux * n;
+        const real qy = T[7] - uy * (xx + yy) - 2 * (ux * xy + uy * yy) + 2 * uy * ud + uu * y - uu * uy * n;
+        take((qx * s * s * s - conF[6] - conF[7]) / 2);
+        take((qy * s * s * s - conF[8] - conF[9]) / 2);
+        return (double)worst;
+    }
+};
+
+template <bool FLUON>
+int population(Cell& k, const double* start, double mass, int pop_cap, ThreadCounters& tc) {
+    double lam[10];
+    for (int j = 0; j < DFPop<2, FLUON>::N; j++) lam[j] = start[j];
+    DFStream ds = k.stream(mass, pop_cap);
+    return df_population<2, FLUON>(k.m, k.c, k.tab, lam, FLUON ? k.conF : k.conG, k.etab.data(), k.st.R + 2.0, ds, tc);
+}
+
+template <bool FLUON>
+void judged(double RT, double noise, double tol, int trials, unsigned seed, double* out) {
+    std::mt19937_64 rng(seed);
+    std::normal_distribution<double> N01;
+    Cell k;
+    k.m.tol = tol;
+    for (int i = 0; i < 4; i++) out[i] = 0.0;
+    for (int t = 0; t < trials; t++) {
+        if (!k.draw(rng, RT, 0.1, 1.0)) continue;
+        double start[10];
+        for (int j = 0; j < DFPop<2, FLUON>::N; j++)
+            start[j] = (double)(float)((FLUON ? k.lf[j] : k.lg[j]) + noise * N01(rng));
+        ThreadCounters tc{}, full{};
+        std::fill(k.M.begin(), k.M.end(), 0.0);
+        const bool ok = population<FLUON>(k, start, 1.0, kDfPopCap, tc) >= 0;
+        out[0] += 1.0;
+        out[3] += tc.redo;
+        if (!ok) continue;
+        out[1] = std::max(out[1], k.residual(FLUON));
+        const std::vector<double> kept = k.M;
+        std::fill(k.M.begin(), k.M.end(), 0.0);
+        population<FLUON>(k, start, 1.0, 0, full);  // every population evaluated twice
+        out[2] += kept != k.M;
+    }
+}
+
+}  // namespace
+
+extern "C" {
+
+// The mixed path's finish of one population from multipliers that are off by `noise`: out = cells drawn,
+// the largest true residual of a deposit that passed the check, cells streamed from kept
+// populations, deposits taken back.
+void check_judged(int fluon, double RT, double noise, double tol, int trials, unsigned seed, double* out) {
+    if (fluon)
+        judged<true>(RT, noise, tol, trials, seed, out);
+    else
+        judged<false>(RT, noise, tol, trials, seed, out);
+}
+
+}

@@ -1,0 +1,46 @@
+"""Per-cell functions of the CUDA headers, compiled for the host (device_host/) and held against
+extended-precision sums."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2508_06911_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("device_host") / "checks.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(build.NVCC)), "include")
+    src = os.path.join(HERE, "device_host", "checks.cpp")
+    r = subprocess.run(["g++", "-O2", "-std=c++17", "-w", "-ffp-contract=off", "-shared", "-fPIC", "-I", cuda, "-I",
+                        build.CSRC, src, "-o", so], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return ctypes.CDLL(so)
+
+
+def call(f, *args, n_out):
+    out = (ctypes.c_double * n_out)()
+    f(*[ctypes.c_double(a) if isinstance(a, float) else ctypes.c_int(a) for a in args], out)
+    return list(out)
+
+
+# The residual that the mixed path judges is that of the deposit.  Streaming from kept populations sums
+# the change of the residual in FP32, off by up to 5.5 2^-24 of sums of at most 3e-6, of which the judge
+# adds three fifths to what it finds: 0.45 of the default tolerance are left.  A smaller tolerance
+# has to be judged by a fresh sum.
+# 5e-14: the double-float floor of that sum (2^-48 of sums of |X|^3 f times 1 / sqrt(RT)^3).
+@pytest.mark.parametrize("tol", [1e-12, 1e-13])
+@pytest.mark.parametrize("fluon", [1, 0])
+@pytest.mark.parametrize("RT", [0.22, 0.6, 4.0, 9.0])
+def test_judged_residual_is_that_of_the_deposit(lib, RT, fluon, tol):
+    some_kept = 0
+    for noise in (3e-9, 1e-8, 3e-8, 6e-8, 1e-7):
+        cells, worst, kept, _ = call(lib.check_judged, fluon, RT, noise, tol, 400, 5, n_out=4)
+        assert cells > 100
+        assert worst <= (1.45 if tol >= 1e-12 else 1.0) * tol + 5e-14, f"noise {noise}: {worst:.2e}"
+        some_kept += kept
+    assert (some_kept > 0) == (tol >= 1e-12)

@@ -1192,6 +1192,23 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
     return -1;
 }
 
+// Takes back the phonon deposit that df_population made from the multipliers lg32 (the FP64 EPR then
+// streams the cell): the same passes from the same start with the mass negated, so that every addition
+// comes again with the other sign, whichever of the passes made it.  Out of line: it is rare.
+template <int D>
+static __device__ __noinline__ void df_take_back(const Model& m, const CellState<D>& c, const RowTable<D>& tab,
+                                                 const float* lg32, const double* conG, const float2* etab, double xm,
+                                                 const DFStream& ds_in, ThreadCounters& tc) {
+    double lg[Dim<D>::NG];
+#pragma unroll
+    for (int j = 0; j < Dim<D>::NG; j++) lg[j] = (double)lg32[j];
+    DFStream ds = ds_in;
+    df_split(-(c.rho * m.K * c.RT), ds.mh, ds.ml);
+    const unsigned int redo = tc.redo;
+    df_population<D, false>(m, c, tab, lg, conG, etab, xm, ds, tc);
+    tc.redo = redo;  // misses are counted once
+}
+
 // The multipliers of a converged FP32 solve minus Eq. (IID13), for the next step, and its counts.
 template <int D>
 __device__ __forceinline__ void keep_solution32(const Model& m, const Geometry& g, long long cell, BlockCounters& bc,
@@ -1620,12 +1637,7 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
         uf = df_population<D, true>(m, c, tab, lf, conF, etab, xm, ds, tc);
         if (uf < 0) {
             alive = false;
-            if (has_g) {  // take the phonon deposit back too: the FP64 EPR streams both
-                double r[NG], rmax;
-                df_split(-(c.rho * m.K * c.RT), ds.mh, ds.ml);
-                df_pass<D, false, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lg, conG, etab, xm, r, rmax,
-                                             nullptr, ds, tc.ls, tc.pdf, ds.beta);
-            }
+            if (has_g) df_take_back<D>(m, c, tab, lg32, conG, etab, xm, ds, tc);
         }
     }
     if (alive) {

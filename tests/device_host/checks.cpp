@@ -113,11 +113,12 @@ struct Cell {
 };
 
 template <bool FLUON>
-int population(Cell& k, const double* start, double mass, int pop_cap, ThreadCounters& tc) {
+int population(Cell& k, const double* start, double mass, int pop_cap, ThreadCounters& tc, double xm = 0.0) {
     double lam[10];
     for (int j = 0; j < DFPop<2, FLUON>::N; j++) lam[j] = start[j];
     DFStream ds = k.stream(mass, pop_cap);
-    return df_population<2, FLUON>(k.m, k.c, k.tab, lam, FLUON ? k.conF : k.conG, k.etab.data(), k.st.R + 2.0, ds, tc);
+    return df_population<2, FLUON>(k.m, k.c, k.tab, lam, FLUON ? k.conF : k.conG, k.etab.data(),
+                                   xm > 0.0 ? xm : k.st.R + 2.0, ds, tc);
 }
 
 template <bool FLUON>
@@ -146,6 +147,19 @@ void judged(double RT, double noise, double tol, int trials, unsigned seed, doub
     }
 }
 
+// |X| up to which the fixed-point exponents of the phonons' multipliers lam stay in range.
+float reach(const Cell& k, const double* lam) {
+    long long beta[10];
+    float lo = 0.f, hi = 1000.f;
+    while (std::nextafterf(lo, hi) < hi) {
+        const float mid = lo + 0.5f * (hi - lo);
+        const bool in = fix_poly<2, false>(lam, k.c.inv_sig, k.c.u[0] - (double)k.tab.xc, k.c.u[1] - (double)k.tab.yc,
+                                           (double)mid, beta);
+        (in ? lo : hi) = mid;
+    }
+    return lo;
+}
+
 }  // namespace
 
 extern "C" {
@@ -158,6 +172,55 @@ void check_judged(int fluon, double RT, double noise, double tol, int trials, un
         judged<true>(RT, noise, tol, trials, seed, out);
     else
         judged<false>(RT, noise, tol, trials, seed, out);
+}
+
+// A phonon deposit taken back: out = cells drawn, the largest of what stays of a moment against its
+// largest value, cells streamed from kept populations, cells whose updated multipliers alone are out of the
+// fixed-point range (edge = 1: the range is set between the start's reach and the update's).
+void check_take_back(double RT, double noise, int edge, int trials, unsigned seed, double* out) {
+    std::mt19937_64 rng(seed);
+    std::normal_distribution<double> N01;
+    Cell k;
+    for (int i = 0; i < 4; i++) out[i] = 0.0;
+    for (int t = 0; t < trials; t++) {
+        if (!k.draw(rng, RT, 0.1, 1.0)) continue;
+        float lg32[6];
+        double start[6], lam[6];
+        for (int j = 0; j < 6; j++) start[j] = lam[j] = lg32[j] = (float)(k.lg[j] + noise * N01(rng));
+        double xm = k.st.R + 2.0;
+        ThreadCounters tc{};
+        if (edge) {
+            DFStream ds = k.stream(1.0, 0);
+            double r[6], rmax;
+            float MJ[DFPop<2, false>::NJ], dl[6];
+            if (!df_pass<2, false, DF_CORR>(k.c.u[0], k.c.u[1], k.c.inv_sig, k.tab, lam, k.conG, k.etab.data(), xm, r,
+                                            rmax, MJ, ds, tc.ls, tc.pdfc, k.beta) ||
+                !df_update<2, false>(MJ, r, lam, dl))
+                continue;
+            const float a = reach(k, start), b = reach(k, lam);
+            if (!(b < a)) continue;
+            xm = a;
+            out[3] += 1.0;
+        }
+        const double mass = k.c.rho * k.m.K * k.c.RT;
+        std::fill(k.M.begin(), k.M.end(), 0.0);
+        if (population<false>(k, start, mass, kDfPopCap, tc, xm) < 0) continue;
+        out[0] += 1.0;
+        const std::vector<double> made = k.M;
+        DFStream ds = k.stream(1.0, kDfPopCap);
+        df_take_back<2>(k.m, k.c, k.tab, lg32, k.conG, k.etab.data(), xm, ds, tc);
+        for (int i = 8; i < 11; i++) {
+            double top = 0.0, left = 0.0;
+            for (int j = 0; j < kGrid * kGrid; j++) {
+                top = std::max(top, std::fabs(made[(size_t)i * kGrid * kGrid + j]));
+                left = std::max(left, std::fabs(k.M[(size_t)i * kGrid * kGrid + j]));
+            }
+            out[1] = std::max(out[1], left / top);
+        }
+        std::fill(k.M.begin(), k.M.end(), 0.0);
+        population<false>(k, start, mass, 0, tc, xm);
+        out[2] += made != k.M;
+    }
 }
 
 }

@@ -44,3 +44,14 @@ def test_judged_residual_is_that_of_the_deposit(lib, RT, fluon, tol):
         assert worst <= (1.45 if tol >= 1e-12 else 1.0) * tol + 5e-14, f"noise {noise}: {worst:.2e}"
         some_kept += kept
     assert (some_kept > 0) == (tol >= 1e-12)
+
+
+# A phonon deposit that a failed fluon solve takes back leaves the rounding of the additions only: at most
+# two times twenty additions to a cell, half an ulp each.  Also where the updated multipliers are out of
+# the range of the pass that evaluates them, while the kept populations were streamed.
+@pytest.mark.parametrize("edge", [0, 1])
+@pytest.mark.parametrize("RT", [0.22, 0.6, 4.0])
+def test_phonon_take_back(lib, RT, edge):
+    cells, left, kept, at_edge = call(lib.check_take_back, RT, 3e-7, edge, 1500 if edge else 300, 6, n_out=4)
+    assert cells > 50 and kept > 30 and (not edge or at_edge > 50)
+    assert left <= 40 * 2.0 ** -53

@@ -228,13 +228,77 @@ struct SweepRows {
 // compounded rounding of tall sets; up to R_ac = 7 (RT = 3.5 at n = 4) one anchor serves all.
 constexpr int kAnchorRows = 8;
 
+// Acoustic radius up to which the sweeps compound along y too.  The mean error of a population (weighted by
+// it, against 64 bits; the general stencil, whose rows each start afresh, in brackets): 2D, RT 0.6 1.6e-16
+// (1.3e-15), RT 9.4 1.3e-15 (1.5e-15), but with sweeps RT 10 1.3e-15 (1.0e-15), RT 16 2.2e-15 (6.6e-16)
+// and RT 32 5.0e-15 (1.0e-15).  Beyond, rows that start afresh in the lattice form: RT 10 4.9e-16, RT 16
+// 6.2e-16, RT 32 1.0e-15.  1D: RT 8 2.7e-16 (6.2e-15), RT 9.4 3.6e-16 and afresh 2.7e-16 (3.3e-16).  Time of a
+// step: 128^2 at RT 16 4.8 -> 5.5 ms (13.1 on the general stencil), 64^2 at RT 32 8.2 -> 7.7 ms (17.6).
+template <int D>
+constexpr int kSweepR = D == 1 ? 11 : 12;
+
+// The populations of one side of a row, from its point at thermal x outwards in steps of h (signed): with its
+// own exponentials, but for the last ratio, which is the same on every row.
+struct SideF {
+    double e, r, r2;
+    __device__ __forceinline__ void start(const double* c, double x, double h, double w) {
+        const double h2 = h * h, c3 = 3.0 * c[3] * x;
+        e = w * exp_int(-(((c[3] * x + c[2]) * x + c[1]) * x + c[0]));
+        r = exp_int(-(h * fma(x, fma(2.0, c[2], c3), c[1]) + h2 * (c[2] + c3 + c[3] * h)));
+        r2 = exp_int(-2.0 * h2 * (c[2] + c3 + 3.0 * c[3] * h));
+    }
+};
+struct SideG {
+    double e, r;
+    __device__ __forceinline__ void start(const double* c, double x, double h, double w) {
+        e = w * exp_int(-((c[2] * x + c[1]) * x + c[0]));
+        r = exp_int(-h * (c[1] + c[2] * (2.0 * x + h)));
+    }
+};
+
 // Visits the lattice points (x0 + k h, y0 + j h) of rows jlo..jhi: ext(j, i0, i1, h0, h1) gives a
 // row's points i0..i1 without the hole h0..h1 (empty: h0 = 1, h1 = 0); point(k, j, f, g) gets every
 // point with its populations (weights wf, wg included), row_end(j) follows a row that is not empty.
-template <int D, class Ext, class Pt, class RowEnd>
+// FRESH: every row starts from exponentials of its own, on both sides of its centre.
+template <int D, bool FRESH, class Ext, class Pt, class RowEnd>
 __device__ __forceinline__ void lattice_sweep(const double* lf, const double* lg, bool doF, bool doG, double x0,
                                               double y0, double h, double wf, double wg, int jlo, int jhi,
                                               const Ext& ext, Pt& point, RowEnd& row_end) {
+    if constexpr (FRESH) {
+        const double h3 = 6.0 * (h * h) * h;
+        const double r3 = doF ? exp_int(-h3 * lf[D == 1 ? 3 : 6]) : 0.0, l3 = doF ? exp_int(h3 * lf[D == 1 ? 3 : 6]) : 0.0;
+        const double r2g = doG ? exp_int(-2.0 * (h * h) * lg[D == 1 ? 2 : 3]) : 0.0;
+#pragma unroll 1
+        for (int j = jlo; j <= jhi; j++) {
+            int i0, i1, h0, h1;
+            ext(j, i0, i1, h0, h1);
+            if (i0 > i1) continue;
+            double cf[4], cg[3];
+            row_coeffs<D>(lf, lg, fma(widen((float)j), h, y0), cf, cg);
+#pragma unroll 1
+            for (int left = 0; left < 2; left++) {
+                const int n = left ? -i0 : i1;
+                if (n < left) continue;
+                const double x = left ? x0 - h : x0, hs = left ? -h : h, t3 = left ? l3 : r3;
+                SideF f{0.0, 0.0, 0.0};
+                SideG g{0.0, 0.0};
+                if (doF) f.start(cf, x, hs, wf);
+                if (doG) g.start(cg, x, hs, wg);
+#pragma unroll 1
+                for (int i = left; i <= n; i++) {
+                    const int k = left ? -i : i;
+                    if (k >= i0 && k <= i1 && (k < h0 || k > h1)) point(k, j, f.e, g.e);
+                    f.e *= f.r;
+                    f.r *= f.r2;
+                    f.r2 *= t3;
+                    g.e *= g.r;
+                    g.r *= r2g;
+                }
+            }
+            row_end(j);
+        }
+        return;
+    }
     int ja = 0;
     while (ja - kAnchorRows > jlo) ja -= 2 * kAnchorRows + 1;
 #pragma unroll 1
@@ -390,7 +454,7 @@ __device__ __forceinline__ void add_thermal(const double* Ls, double fx, double 
 
 // One pass over the velocity set: the thermal moments of degree <= 3 of f (if doF) and <= 2 of g
 // (if doG) in FP64 (TF, TG) and the Jacobian's moments in FP32 (MF, MG).  Returns the point count.
-template <int D>
+template <int D, bool FRESH>
 __device__ __forceinline__ unsigned int moment_pass64(const CellState<D>& c, const RowTable<D>& tab,
                                                       const CellLattice<D>& lat, const double* lf, const double* lg,
                                                       bool doF, bool doG, double* TF, double* TG, float* MF,
@@ -505,7 +569,7 @@ __device__ __forceinline__ unsigned int moment_pass64(const CellState<D>& c, con
         int jlo, jhi;
         lat.rows(tab, child, jlo, jhi);
         auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
-        lattice_sweep<D>(lf, lg, doF, doG, -ox * hs, -oy * hs, hs, w, w, jlo, jhi, ext, point, row_end);
+        lattice_sweep<D, FRESH>(lf, lg, doF, doG, -ox * hs, -oy * hs, hs, w, w, jlo, jhi, ext, point, row_end);
         if (doF) add_thermal<D, true>(LF, ox, oy, hs, TF);
         if (doG) add_thermal<D, false>(LG, ox, oy, hs, TG);
     }
@@ -549,7 +613,7 @@ __device__ __forceinline__ int newton_step64(const double* T, const float* Mom, 
 }
 
 // Joint Newton iterations of both populations as solve_fg, with lattice-form passes.
-template <int D>
+template <int D, bool FRESH = false>
 __device__ __forceinline__ void solve_fg64(const CellState<D>& c, const RowTable<D>& tab, const CellLattice<D>& lat,
                                            const double* conF, const double* conG, bool has_g, double* lf, double* lg,
                                            const Model& m, int& sf, int& sg, unsigned int& npf, unsigned int& npg) {
@@ -560,7 +624,7 @@ __device__ __forceinline__ void solve_fg64(const CellState<D>& c, const RowTable
     for (int it = 0; fa || ga; it++) {
         double TF[DFPop<D, true>::NB], TG[DFPop<D, false>::NB];
         float MF[MomentSet<D>::NF], MG[MomentSet<D>::NG];
-        const unsigned int q = moment_pass64<D>(c, tab, lat, lf, lg, fa, ga, TF, TG, MF, MG);
+        const unsigned int q = moment_pass64<D, FRESH>(c, tab, lat, lf, lg, fa, ga, TF, TG, MF, MG);
         if (ga) {
             npg += q;
             const int r = newton_step64<D, false>(TG, MG, conG, lg, m.tol, m.max_iter, it);

@@ -699,7 +699,7 @@ __device__ __forceinline__ void scatter_cell(const Model& m, const Geometry& g, 
 constexpr int kChildMax = 8;
 
 // scatter_cell in lattice form (lelbm_fp64.cuh), for a cell with a row table.
-template <int D>
+template <int D, bool FRESH = false>
 __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                           const CellPlace& at, const CellState<D>& c, const Stencil<D>& st,
                                           const RowTable<D>& tab, const CellLattice<D>& lat, const double* lf,
@@ -781,7 +781,7 @@ __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, con
             k0 = i0;
             nk = child && !near_wall && i1 - i0 < kChildMax ? i1 - i0 + 1 : 0;
         };
-        lattice_sweep<D>(lf, lg, true, has_g, -ox * hs, -oy * hs, hs, w * mfs, w * mgs, jlo, jhi, ext, point,
+        lattice_sweep<D, FRESH>(lf, lg, true, has_g, -ox * hs, -oy * hs, hs, w * mfs, w * mgs, jlo, jhi, ext, point,
                          row_end);
     }
     if constexpr (D == 2) {
@@ -1083,6 +1083,46 @@ __device__ __forceinline__ void count_set(const RowTable<D>& tab, const CellLatt
     ls.disp_max2 = fmax(ls.disp_max2, 0.0625 * (double)far4);
 }
 
+// The lattice form for one cell: EPR from the multipliers lf, lg and moment streaming.  False, with nothing
+// streamed, where a solve broke down.
+template <int D, bool FRESH>
+__device__ __forceinline__ bool fp64_lattice_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                                  const CellPlace& at, BlockCounters& bc, unsigned int& pf,
+                                                  unsigned int& pg, LocalStats& ls, const double* conF,
+                                                  const double* conG, const CellState<D>& c, const Stencil<D>& st,
+                                                  const RowTable<D>& tab, double* lf, double* lg) {
+    CellLattice<D> lat;
+    lat.init(c, tab);
+    int sf, sg;
+    solve_fg64<D, FRESH>(c, tab, lat, conF, conG, m.K > 0.0, lf, lg, m, sf, sg, pf, pg);
+    if (sf < 0 || sg < 0) return false;
+    keep_solution<D>(m, g, at.cell, bc, c, st, lf, lg, sf, sg);
+    if (m.det_lam) {
+        keep_for_gather<D>(m, g, at.cell, c, st, lf, lg);
+        count_set<D>(tab, lat, ls);
+    } else {
+        scatter64<D, FRESH>(m, g, type, Mout, at, c, st, tab, lat, lf, lg, ls, conF, conG);
+    }
+    return true;
+}
+
+// The same beyond kSweepR, out of line: few programs have such cells, and inline the second form would
+// crowd the first.
+template <int D>
+static __device__ __noinline__ bool fp64_hot_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                                  const CellPlace at, BlockCounters* bc, TailCounts* t,
+                                                  const double* conF, const double* conG, const CellState<D> c,
+                                                  const Stencil<D> st, const RowTable<D> tab_in, double* lf_io,
+                                                  double* lg_io) {
+    const RowTable<D> tab = tab_in;
+    double lf[Dim<D>::NF], lg[Dim<D>::NG];
+#pragma unroll
+    for (int j = 0; j < Dim<D>::NF; j++) lf[j] = lf_io[j];
+#pragma unroll
+    for (int j = 0; j < Dim<D>::NG; j++) lg[j] = lg_io[j];
+    return fp64_lattice_cell<D, true>(m, g, type, Mout, at, *bc, t->pf, t->pg, t->ls, conF, conG, c, st, tab, lf, lg);
+}
+
 // The FP64 path's cell after the collision: EPR from the multipliers lf, lg, and moment streaming, in
 // lattice form where the cell has a row table whose offsets and velocities are exact in FP32
 // (|k|^3 and quarter cells below 2^24).
@@ -1092,22 +1132,17 @@ __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, con
                                           ThreadCounters& tc, double* conF, double* conG, const CellState<D>& c,
                                           const Stencil<D>& st, const RowTable<D>& tab, double* lf, double* lg,
                                           bool learned) {
-    const bool has_g = m.K > 0.0;
     if (tab.ok && st.R <= 250 && abs(tab.xc) < (1 << 21) && abs(tab.yc) < (1 << 21)) {
-        CellLattice<D> lat;
-        lat.init(c, tab);
-        int sf, sg;
-        solve_fg64<D>(c, tab, lat, conF, conG, has_g, lf, lg, m, sf, sg, tc.pf, tc.pg);
-        if (sf >= 0 && sg >= 0) {
-            keep_solution<D>(m, g, at.cell, bc, c, st, lf, lg, sf, sg);
-            if (m.det_lam) {
-                keep_for_gather<D>(m, g, at.cell, c, st, lf, lg);
-                count_set<D>(tab, lat, tc.ls);
-            } else {
-                scatter64<D>(m, g, type, Mout, at, c, st, tab, lat, lf, lg, tc.ls, conF, conG);
-            }
-            return;
+        bool done;
+        if (st.R <= kSweepR<D>) {
+            done = fp64_lattice_cell<D, false>(m, g, type, Mout, at, bc, tc.pf, tc.pg, tc.ls, conF, conG, c, st, tab, lf,
+                                               lg);
+        } else {
+            TailCounts t{0, 0, 0, {0, 0.0, 0, 0}};
+            done = fp64_hot_cell<D>(m, g, type, Mout, at, &bc, &t, conF, conG, c, st, tab, lf, lg);
+            add_tail(tc, t);
         }
+        if (done) return;
         if (learned) tc.retry++;
         learned = false;
         maxwell_start_fg<D, Dim<D>::NF, Dim<D>::NG>(c.RT, lf, lg);

@@ -160,6 +160,99 @@ float reach(const Cell& k, const double* lam) {
     return lo;
 }
 
+// Errors of the lattice-form populations (out[0]: mean, weighted by the population; out[1]: largest relative
+// one) and of the general stencil's (out[2], out[3]) against extended precision, f and g.
+template <int D>
+void populations(double RT, int trials, unsigned seed, double* out) {
+    constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
+    std::mt19937_64 rng(seed);
+    std::uniform_real_distribution<double> U(-1.0, 1.0);
+    Model m{};
+    m.K = 2.0;
+    m.n_conf = 4.0;
+    m.r_min = 2.0;
+    m.refine_div = m.refine_rad = 3.0;
+    m.max_refine = 4;
+    set_derived_params(m, D);
+    real err[2] = {}, sum = 0;
+    double worst[2] = {};
+    for (int t = 0; t < trials; t++) {
+        CellState<D> c{};
+        c.rho = 1.0;
+        c.RT = RT * (1.0 + 0.02 * U(rng));
+        c.sig = std::sqrt(c.RT);
+        c.inv_sig = 1.0 / c.sig;
+        for (int a = 0; a < D; a++) c.u[a] = 2.0 * U(rng);
+        Stencil<D> st;
+        st.init(c, m);
+        char2 rows[kRowsMax];
+        RowTable<D> tab;
+        tab.build(c, st, rows);
+        if (!tab.ok) continue;
+        CellLattice<D> lat;
+        lat.init(c, tab);
+        double lf[NF], lg[NG];
+        maxwell_start_fg<D, NF, NG>(c.RT, lf, lg);
+        for (double& v : lf) v += 0.01 * U(rng);
+        for (double& v : lg) v += 0.01 * U(rng);
+        auto take = [&](int who, const real* v, double f, double g) {
+            const real x = (v[0] - c.u[0]) * c.inv_sig, y = D == 2 ? (v[D - 1] - c.u[D - 1]) * c.inv_sig : 0;
+            for (int p = 0; p < 2; p++) {
+                real e = 1;
+                for (int j = 0; j < (p ? NG : NF); j++)
+                    e += (real)(p ? lg[j] : lf[j]) * powl(x, p ? bx<D, false>(j) : bx<D, true>(j)) *
+                         powl(y, p ? by<D, false>(j) : by<D, true>(j));
+                const real exact = expl(-e), d = fabsl((p ? g : f) - exact);
+                err[who] += d;
+                worst[who] = std::max(worst[who], (double)(d / exact));
+                if (who == 0) sum += exact;
+            }
+        };
+        for (int l = 0; l < lat.n; l++) {
+            const bool child = l == 1;
+            const double hs = child ? 0.5 * c.inv_sig : c.inv_sig;
+            const double ox = child ? 2.0 * lat.fx + 0.5 : lat.fx, oy = child ? 2.0 * lat.fy + 0.5 : lat.fy;
+            auto point = [&](int k, int j, double f, double g) {
+                const real v[2] = {child ? lat.xn - 0.25L + 0.5L * k : (real)(lat.xn + k),
+                                   child ? lat.yn - 0.25L + 0.5L * j : (real)(lat.yn + j)};
+                take(0, v, f, g);
+            };
+            auto row_end = [](int) {};
+            auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
+            int jlo, jhi;
+            lat.rows(tab, child, jlo, jhi);
+            if (st.R <= kSweepR<D>)
+                lattice_sweep<D, false>(lf, lg, true, true, -ox * hs, -oy * hs, hs, 1.0, 1.0, jlo, jhi, ext, point,
+                                        row_end);
+            else
+                lattice_sweep<D, true>(lf, lg, true, true, -ox * hs, -oy * hs, hs, 1.0, 1.0, jlo, jhi, ext, point,
+                                       row_end);
+        }
+        auto row = [&](int cy, int xa, int xb) {
+            double cf[4], cg[3];
+            row_coeffs<D>(lf, lg, D == 2 ? ((double)cy - c.u[D - 1]) * c.inv_sig : 0.0, cf, cg);
+            auto point = [&](int k, double, double f, double g) {
+                const real v[2] = {(real)(xa + k), (real)cy};
+                take(1, v, f, g);
+            };
+            row_eval(cf, cg, true, true, ((double)xa - c.u[0]) * c.inv_sig, c.inv_sig, xb - xa + 1, point);
+        };
+        auto leaf = [&](const double* cp, double) {
+            const double x = (cp[0] - c.u[0]) * c.inv_sig, y = D == 2 ? (cp[D - 1] - c.u[D - 1]) * c.inv_sig : 0.0;
+            double cf[4], cg[3];
+            row_coeffs<D>(lf, lg, y, cf, cg);
+            const real v[2] = {cp[0], D == 2 ? cp[D - 1] : 0.0};
+            take(1, v, std::exp(-(((cf[3] * x + cf[2]) * x + cf[1]) * x + cf[0])),
+                 std::exp(-((cg[2] * x + cg[1]) * x + cg[0])));
+        };
+        st.for_each_row(row, leaf);
+    }
+    for (int k = 0; k < 2; k++) {
+        out[2 * k] = (double)(err[k] / sum);
+        out[2 * k + 1] = worst[k];
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -221,6 +314,13 @@ void check_take_back(double RT, double noise, int edge, int trials, unsigned see
         population<false>(k, start, mass, 0, tc, xm);
         out[2] += made != k.M;
     }
+}
+
+void check_populations(int D, double RT, int trials, unsigned seed, double* out) {
+    if (D == 1)
+        populations<1>(RT, trials, seed, out);
+    else
+        populations<2>(RT, trials, seed, out);
 }
 
 }

@@ -55,3 +55,12 @@ def test_phonon_take_back(lib, RT, edge):
     cells, left, kept, at_edge = call(lib.check_take_back, RT, 3e-7, edge, 1500 if edge else 300, 6, n_out=4)
     assert cells > 50 and kept > 30 and (not edge or at_edge > 50)
     assert left <= 40 * 2.0 ** -53
+
+
+# The lattice form's populations are no further off, weighted by the population, than the general stencil's,
+# which starts every row from exponentials of its own: within a fifth and two roundings (2^-52).
+@pytest.mark.parametrize("RT", [0.2, 0.35, 0.6, 1.5, 4.2, 8.0, 9.4, 10.2, 13.0, 16.0, 25.0, 32.0])
+@pytest.mark.parametrize("D", [1, 2])
+def test_lattice_form_populations(lib, D, RT):
+    mean, _, mean_rows, _ = call(lib.check_populations, D, RT, 30 if D == 2 else 200, 7, n_out=4)
+    assert 0 < mean <= 1.2 * mean_rows + 2.0 ** -52

@@ -198,8 +198,9 @@ __global__ void __launch_bounds__(128) noalloc_cell_kernel(Model m, Topo t, cons
         for (int j = 0; j < NG; j++) conG[j] = c.cg[j];
         RowTable<D> tab;
         tab.build(c, st, s_rows[D == 2 ? threadIdx.x : 0]);
+        Absorbed none;  // no walls here
         fp64_cell<D>(m, g, nullptr, Mout, stats, CellPlace{cell, lo, n, ix, iy}, bc, tc, conF, conG, c, st, tab, lf, lg,
-                     false);
+                     false, none);
     }
     counters_flush(bc, tc, stats);
 }

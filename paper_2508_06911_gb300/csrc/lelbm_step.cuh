@@ -694,6 +694,14 @@ __device__ __forceinline__ void scatter_cell(const Model& m, const Geometry& g, 
     ls.disp_max2 = fmax(ls.disp_max2, dmax2);
 }
 
+// What the no-slip walls took of a cell that scatter64 streamed, and the multipliers of its images, which the
+// caller launches (launch_images).
+struct Absorbed {
+    bool any = false;
+    double mass[4];  // as scatter_cell's absorbed
+    double lf[10], lg[6];
+};
+
 // Children of a row that scatter64 holds for ChildRow: two for each of at most four split points (the
 // paper's refinement radius); a row with more (refine_rad set larger) deposits them one by one.
 constexpr int kChildMax = 8;
@@ -703,7 +711,7 @@ template <int D, bool FRESH = false>
 __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                           const CellPlace& at, const CellState<D>& c, const Stencil<D>& st,
                                           const RowTable<D>& tab, const CellLattice<D>& lat, const double* lf,
-                                          const double* lg, LocalStats& ls, const double* conF, const double* conG) {
+                                          const double* lg, LocalStats& ls, Absorbed& due) {
     constexpr int NM = Dim<D>::NM;
     const bool has_g = m.K > 0.0;
     const double mfs = c.rho, mgs = c.rho * m.K * c.RT;  // rho dV f', rho K RT dV g'
@@ -785,13 +793,35 @@ __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, con
                          row_end);
     }
     if constexpr (D == 2) {
-        if (absorbed[0] != 0.0 || absorbed[1] != 0.0 || absorbed[2] != 0.0 || absorbed[3] != 0.0)
-            noslip_images(m, g, type, Mout, at.cell, at.ix, at.iy, c, st, lf, lg, conF, conG, mfs, mgs, absorbed);
+        if (absorbed[0] != 0.0 || absorbed[1] != 0.0 || absorbed[2] != 0.0 || absorbed[3] != 0.0) {
+            due.any = true;
+#pragma unroll
+            for (int k = 0; k < 4; k++) due.mass[k] = absorbed[k];
+#pragma unroll
+            for (int j = 0; j < Dim<D>::NF; j++) due.lf[j] = lf[j];
+#pragma unroll
+            for (int j = 0; j < Dim<D>::NG; j++) due.lg[j] = lg[j];
+        }
     }
     if (q > ls.q_max) ls.q_max = q;
     ls.points += q;
     ls.walls += walls;
     ls.disp_max2 = fmax(ls.disp_max2, 0.0625 * (double)far4);
+}
+
+// The images of the no-slip walls for the cells of a warp; whole warps call it.  Launched from scatter64, where
+// the lanes leave loops of different lengths, the images (two passes over the velocity set, every path
+// traced) ran lane after lane: 300 x 150 cylinder with a no-slip wall 11.5 ms a step, gathered here 6.6.
+__device__ __forceinline__ void launch_images(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
+                                              long long cell, const CellState<2>& c, const Stencil<2>& st,
+                                              const double* conF, const double* conG, const Absorbed& due) {
+    __syncwarp();
+    if (due.any) {
+        const CellPlace at = cell_place<2>(g, cell);
+        noslip_images(m, g, type, Mout, cell, at.ix, at.iy, c, st, due.lf, due.lg, conF, conG, c.rho,
+                      c.rho * m.K * c.RT, due.mass);
+    }
+    __syncwarp();
 }
 
 // Per-block counters in shared memory, flushed to DevStats once per block.
@@ -1090,7 +1120,7 @@ __device__ __forceinline__ bool fp64_lattice_cell(const Model& m, const Geometry
                                                   const CellPlace& at, BlockCounters& bc, unsigned int& pf,
                                                   unsigned int& pg, LocalStats& ls, const double* conF,
                                                   const double* conG, const CellState<D>& c, const Stencil<D>& st,
-                                                  const RowTable<D>& tab, double* lf, double* lg) {
+                                                  const RowTable<D>& tab, double* lf, double* lg, Absorbed& due) {
     CellLattice<D> lat;
     lat.init(c, tab);
     int sf, sg;
@@ -1101,7 +1131,7 @@ __device__ __forceinline__ bool fp64_lattice_cell(const Model& m, const Geometry
         keep_for_gather<D>(m, g, at.cell, c, st, lf, lg);
         count_set<D>(tab, lat, ls);
     } else {
-        scatter64<D, FRESH>(m, g, type, Mout, at, c, st, tab, lat, lf, lg, ls, conF, conG);
+        scatter64<D, FRESH>(m, g, type, Mout, at, c, st, tab, lat, lf, lg, ls, due);
     }
     return true;
 }
@@ -1113,14 +1143,15 @@ static __device__ __noinline__ bool fp64_hot_cell(const Model& m, const Geometry
                                                   const CellPlace at, BlockCounters* bc, TailCounts* t,
                                                   const double* conF, const double* conG, const CellState<D> c,
                                                   const Stencil<D> st, const RowTable<D> tab_in, double* lf_io,
-                                                  double* lg_io) {
+                                                  double* lg_io, Absorbed* due) {
     const RowTable<D> tab = tab_in;
     double lf[Dim<D>::NF], lg[Dim<D>::NG];
 #pragma unroll
     for (int j = 0; j < Dim<D>::NF; j++) lf[j] = lf_io[j];
 #pragma unroll
     for (int j = 0; j < Dim<D>::NG; j++) lg[j] = lg_io[j];
-    return fp64_lattice_cell<D, true>(m, g, type, Mout, at, *bc, t->pf, t->pg, t->ls, conF, conG, c, st, tab, lf, lg);
+    return fp64_lattice_cell<D, true>(m, g, type, Mout, at, *bc, t->pf, t->pg, t->ls, conF, conG, c, st, tab, lf, lg,
+                                      *due);
 }
 
 // The FP64 path's cell after the collision: EPR from the multipliers lf, lg, and moment streaming, in
@@ -1131,15 +1162,15 @@ __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, con
                                           DevStats* stats, const CellPlace& at, BlockCounters& bc,
                                           ThreadCounters& tc, double* conF, double* conG, const CellState<D>& c,
                                           const Stencil<D>& st, const RowTable<D>& tab, double* lf, double* lg,
-                                          bool learned) {
+                                          bool learned, Absorbed& due) {
     if (tab.ok && st.R <= 250 && abs(tab.xc) < (1 << 21) && abs(tab.yc) < (1 << 21)) {
         bool done;
         if (st.R <= kSweepR<D>) {
             done = fp64_lattice_cell<D, false>(m, g, type, Mout, at, bc, tc.pf, tc.pg, tc.ls, conF, conG, c, st, tab, lf,
-                                               lg);
+                                               lg, due);
         } else {
             TailCounts t{0, 0, 0, {0, 0.0, 0, 0}};
-            done = fp64_hot_cell<D>(m, g, type, Mout, at, &bc, &t, conF, conG, c, st, tab, lf, lg);
+            done = fp64_hot_cell<D>(m, g, type, Mout, at, &bc, &t, conF, conG, c, st, tab, lf, lg, &due);
             add_tail(tc, t);
         }
         if (done) return;
@@ -1356,7 +1387,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
                                             const double* __restrict__ Min, double* Mout,
                                             DevStats* stats, long long cell, BlockCounters& bc, ThreadCounters& tc,
                                             Con<PREC>* conF, Con<PREC>* conG, const CellState<D>& c, const Stencil<D>& st,
-                                            const float* dl, char2* rowbuf) {
+                                            const float* dl, char2* rowbuf, Absorbed& due) {
     static_assert(PREC != PREC_MIXED, "the mixed path steps cells in phases (mixed_block)");
     constexpr int NF = Dim<D>::NF, NG = Dim<D>::NG;
     tc.cells++;
@@ -1481,7 +1512,8 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
         const TailCounts t = fp64_tail_cold<D>(m, g, type, Mout, stats, cell, &bc, conF, conG, c, st);
         add_tail(tc, t);
     } else {
-        fp64_cell<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), bc, tc, conF, conG, c, st, tab, lf, lg, learned);
+        fp64_cell<D>(m, g, type, Mout, stats, cell_place<D>(g, cell), bc, tc, conF, conG, c, st, tab, lf, lg, learned,
+                     due);
     }
 }
 
@@ -1766,7 +1798,13 @@ __global__ void __launch_bounds__(NT, min_blocks<D, PREC>()) cell_update_kernel(
             Stencil<D> st;
             bool ok = false;
             if (active) ok = prepare_cell<D, PREC>(m, g, Min, stats, cell, bc, c, st);
-            if (ok) finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr, rowbuf);
+            Absorbed due;
+            if (ok)
+                finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr, rowbuf,
+                                     due);
+            if constexpr (D == 2 && PREC == PREC_FP64) {
+                if (g.noslip) launch_images(m, g, type, Mout, cell, c, st, conF, conG, due);
+            }
         }
     }
     counters_flush(bc, tc, stats);
@@ -1893,9 +1931,10 @@ __global__ void __launch_bounds__(128, batch_min_blocks<PREC, WIDE>()) batch_per
                     warp_mlp<D>(s_mlp, xin, ok, dl);
                     if (ok) tc.mlp_cells++;
                 }
+                Absorbed none;
                 if (ok)
                     finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st,
-                                         use_mlp ? dl : nullptr, nullptr);
+                                         use_mlp ? dl : nullptr, nullptr, none);
             }
             counters_to_block(bc, tc);  // keeps the 32-bit tallies of a long launch small
             __syncthreads();

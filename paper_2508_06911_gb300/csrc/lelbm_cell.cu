@@ -15,6 +15,9 @@ void CellVariant<D, PREC>::launch(const Model& m, const Geometry& g, const uint8
                                    double* Mout, DevStats* st, unsigned long long* work, int blocks, int threads,
                                    size_t smem, cudaStream_t s) {
     auto kern = cell_update_kernel<D, PREC, cell_threads<PREC>()>;
+    if constexpr (D == 2 && PREC == PREC_FP32) {
+        if (g.wall_dist) kern = cell_update_kernel<D, PREC, cell_threads<PREC>(), true>;
+    }
     if constexpr (D == 2 && PREC == PREC_MIXED) {
         if (threads > cell_threads<PREC>()) kern = cell_update_kernel<D, PREC, kWideThreads>;
     }

@@ -322,7 +322,81 @@ __device__ __forceinline__ void scatter_table32(const Model& m, const Geometry& 
     ls.disp_max2 = fmax(ls.disp_max2, (double)dmax);
 }
 
-// Moment streaming of the FP32 path for any cell: near a wall, or without a row table.
+// Moment streaming of the FP32 path for a cell with a row table and a wall in reach: every population is
+// traced on its own.  The warps near a wall are the last to finish, so the time of a step follows theirs:
+// all points go through one loop body with one call of the trace, where a site for each kind of point
+// had lanes that differ in rows and split points run one after the other, and the Newton solve is shared with
+// the warp's other cells.  600 x 300 cylinder 1.67 -> 1.20 ms a step (1.33 before the streaming of other cells was
+// split off), 1024 x 512 2.24 -> 1.83, 2048 x 1024 4.97 -> 4.37.
+__device__ __forceinline__ void scatter_near32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout, long long cell,
+                         const CellState<2>& c, const RowTable<2>& tab, const float* lf, const float* lg,
+                         LocalStats& ls) {
+    constexpr int NM = Dim<2>::NM;
+    const bool has_g = m.K > 0.0;
+    const float mfs = (float)c.rho;                              // rho dV f'
+    const float mgs = has_g ? (float)(c.rho * m.K * c.RT) : 0.f;  // rho K RT dV g'
+    const CellPlace at = cell_place<2>(g, cell);
+    Acc32 em{0.f, 0.f}, ee{0.f, 0.f}, ep[2];
+#pragma unroll
+    for (int a = 0; a < 2; a++) ep[a] = Acc32{0.f, 0.f};
+    unsigned int q = 0;
+    long long walls = 0;
+    int dmax = 0;
+#pragma unroll 1
+    for (int lat = 0; lat < 2; lat++) {
+        const int r_first = lat ? tab.band_first : 0, r_end = lat ? r_first + tab.band_n : tab.nrows;
+#pragma unroll 1
+        for (int r = r_first; r < r_end; r++) {
+            int rx0, rx1, ra, rb;
+            tab.row_ext(r, rx0, rx1, ra, rb);
+            const int cy = tab.y_first + r;
+            const bool split = ra <= rb;
+            if (!lat && rx0 <= rx1) {
+                const int ex = max(abs(rx0), abs(rx1));
+                dmax = max(dmax, ex * ex + cy * cy);
+            }
+#pragma unroll 1
+            for (int seg = 0; seg < (split ? 2 : (lat ? 0 : 1)); seg++) {
+                const int xa = lat ? ra : (seg == 0 ? rx0 : rb + 1);
+                const int xb = lat ? rb : (seg == 0 && split ? ra - 1 : rx1);
+                if (xa > xb) continue;
+                const float w = lat ? 0.25f : 1.f, h = lat ? 0.5f : 1.f;
+                const float oy = lat ? (seg == 0 ? -0.25f : 0.25f) : 0.f;
+                float cf[4], cg[3];
+                row_coeffs32<2>(lf, lg, tab.ty(cy, oy), cf, cg);
+                const int np = lat ? 2 * (xb - xa + 1) : xb - xa + 1;
+                const float cx0 = lat ? (float)xa - 0.25f : (float)xa, cyf = (float)cy + oy;  // exact
+                q += (unsigned int)np;
+                const float x0 = lat ? tab.tx(xa, -0.25f) : tab.tx(xa), sh = h * tab.s32;
+                float kf = 0.f;
+#pragma unroll 1
+                for (int k = 0; k < np; k++, kf += 1.f) {
+                    const float x = fmaf(kf, sh, x0);
+                    const float f = w * __expf(-fmaf(fmaf(fmaf(cf[3], x, cf[2]), x, cf[1]), x, cf[0]));
+                    const float gp = has_g ? w * __expf(-fmaf(fmaf(cg[2], x, cg[1]), x, cg[0])) : 0.f;
+                    const float cp[2] = {fmaf(kf, h, cx0), cyf};
+                    float v[NM];
+                    fractions32<2>(cp, mfs * f, mgs * gp, v);
+                    em.add(v[0]);
+                    ep[0].add(v[1]);
+                    ep[1].add(v[2]);
+                    ee.add(v[iM2<2>(0, 0)]);
+                    ee.add(v[iM2<2>(1, 1)]);
+                    ee.add(v[iG0<2>()]);
+                    const double cpd[2] = {(double)cp[0], (double)cp[1]};
+                    walls += stream_traced32(g, type, Mout, at.ix, at.iy, cpd, v) ? 1 : 0;
+                }
+            }
+        }
+    }
+    keep_shortfall32<2>(m, g, type, Mout, cell, c, em, ep, ee);
+    if (q > ls.q_max) ls.q_max = q;
+    ls.points += q;
+    ls.walls += walls;
+    ls.disp_max2 = fmax(ls.disp_max2, (double)dmax);
+}
+
+// Moment streaming of the FP32 path for a cell without a row table.
 template <int D>
 __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                                long long cell, const CellState<D>& c, const Stencil<D>& st,
@@ -1294,7 +1368,7 @@ __device__ __forceinline__ void keep_solution32(const Model& m, const Geometry& 
     }
 }
 
-// The FP32 path's cells near a wall or without a row table, out of line.  Returns false when the
+// The FP32 path's cells without a row table, out of line.  Returns false when the
 // FP32 solve failed (nothing is deposited).
 template <int D>
 static __device__ __noinline__ bool fp32_cell_general(const Model& m, const Geometry& g, const uint8_t* type,
@@ -1381,8 +1455,9 @@ __device__ __forceinline__ bool prepare_cell(const Model& m, const Geometry& g, 
     return true;
 }
 
-// dl: the learned correction of the Maxwellian start (fluons then phonons), or null.
-template <int D, int PREC>
+// dl: the learned correction of the Maxwellian start (fluons then phonons), or null.  WALLS: the grid has
+// solid cells (FP32 path, 2D; the other paths ask at run time).
+template <int D, int PREC, bool WALLS = false>
 __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, const uint8_t* type,
                                             const double* __restrict__ Min, double* Mout,
                                             DevStats* stats, long long cell, BlockCounters& bc, ThreadCounters& tc,
@@ -1483,12 +1558,7 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
         tab.build(c, st, rowbuf);
     if constexpr (PREC == PREC_FP32) {
         // FP32 Newton and FP32 streaming; the plain FP64 EPR is the fallback
-        bool near_wall = false;  // as in scatter_cell32
-        if constexpr (D == 2) {
-            if (g.wall_dist)
-                near_wall = (double)g.wall_dist[cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5;
-        }
-        if (tab.ok && !near_wall) {
+        if (tab.ok) {
             bool ok32;
 #pragma unroll 1
             for (;;) {
@@ -1500,6 +1570,13 @@ __device__ __forceinline__ void finish_cell(const Model& m, const Geometry& g, c
             }
             if (ok32) {
                 keep_solution32<D>(m, g, cell, bc, c, lf32, lg32, sf, sg);
+                if constexpr (WALLS) {
+                    // a wall in reach, as in scatter_cell
+                    if ((double)g.wall_dist[cell] <= fmax(fabs(c.u[0]), fabs(c.u[1])) + (double)st.R + 1.5) {
+                        scatter_near32(m, g, type, Mout, cell, c, tab, lf32, lg32, tc.ls);
+                        return;
+                    }
+                }
                 scatter_table32<D>(m, g, type, Mout, cell, c, tab, lf32, lg32, tc.ls);
                 return;
             }
@@ -1746,7 +1823,9 @@ constexpr int kMixedGroups = 2;
 template <int D, int PREC>
 constexpr int min_blocks() { return PREC == PREC_FP32 ? 4 : (PREC == PREC_MIXED ? 1 : 1); }
 
-template <int D, int PREC, int NT>
+// WALLS: a kernel of its own for the FP32 path beside solid cells, so that scatter_near32 costs other grids
+// nothing (with both in one kernel a 128^2 step at RT 16 took 0.97 ms, 0.92 without).
+template <int D, int PREC, int NT, bool WALLS = false>
 __global__ void __launch_bounds__(NT, min_blocks<D, PREC>()) cell_update_kernel(const __grid_constant__ Model m, const __grid_constant__ Geometry g,
                                                           const uint8_t* __restrict__ type,
                                                           const double* __restrict__ Min, double* Mout,
@@ -1800,8 +1879,8 @@ __global__ void __launch_bounds__(NT, min_blocks<D, PREC>()) cell_update_kernel(
             if (active) ok = prepare_cell<D, PREC>(m, g, Min, stats, cell, bc, c, st);
             Absorbed due;
             if (ok)
-                finish_cell<D, PREC>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr, rowbuf,
-                                     due);
+                finish_cell<D, PREC, WALLS>(m, g, type, Min, Mout, stats, cell, bc, tc, conF, conG, c, st, nullptr,
+                                            rowbuf, due);
             if constexpr (D == 2 && PREC == PREC_FP64) {
                 if (g.noslip) launch_images(m, g, type, Mout, cell, c, st, conF, conG, due);
             }

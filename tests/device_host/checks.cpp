@@ -68,6 +68,28 @@ struct Cell {
         solve_fg64<2>(c, tab, lat, conF, conG, true, lf, lg, m, sf, sg, pf, pg);
         return sf >= 0 && sg >= 0;
     }
+    // puts the drawn cell into Min as moments, with the drawn non-equilibrium phonon constraints, and takes it
+    // through the collision; false as draw
+    bool collide_at(std::vector<double>& Min, long long cell) {
+        double Me[11];
+        eq_moments<2>(m.K, c.rho, c.u, c.RT, Me);
+        Me[9] += c.rho * m.K * c.RT * c.sig * conG[1];
+        Me[10] += c.rho * m.K * c.RT * c.sig * conG[2];
+        for (int i = 0; i < 11; i++) Min[(size_t)i * kGrid * kGrid + cell] = Me[i];
+        collide<2>(Me, m, c);
+        if (!c.ok) return false;
+        st.init(c, m);
+        tab.build(c, st, rows);
+        if (!tab.ok) return false;
+        lat.init(c, tab);
+        for (int j = 0; j < 10; j++) conF[j] = c.cf[j];
+        for (int j = 0; j < 6; j++) conG[j] = c.cg[j];
+        maxwell_start_fg<2, 10, 6>(c.RT, lf, lg);
+        int sf, sg;
+        unsigned pf = 0, pg = 0;
+        solve_fg64<2>(c, tab, lat, conF, conG, true, lf, lg, m, sf, sg, pf, pg);
+        return sf >= 0 && sg >= 0;
+    }
     DFStream stream(double mass, int pop_cap) {
         DFStream ds{};
         ds.g = &g;
@@ -274,12 +296,13 @@ void check_take_back(double RT, double noise, int edge, int trials, unsigned see
     std::mt19937_64 rng(seed);
     std::normal_distribution<double> N01;
     Cell k;
+    const long long cell = (kGrid / 2) * kGrid + kGrid / 2;
+    std::vector<double> Min(11 * kGrid * kGrid);  // the moments that the collision takes the cell from
     for (int i = 0; i < 4; i++) out[i] = 0.0;
     for (int t = 0; t < trials; t++) {
-        if (!k.draw(rng, RT, 0.1, 1.0)) continue;
-        float lg32[6];
+        if (!k.draw(rng, RT, 0.1, 1.0) || !k.collide_at(Min, cell)) continue;
         double start[6], lam[6];
-        for (int j = 0; j < 6; j++) start[j] = lam[j] = lg32[j] = (float)(k.lg[j] + noise * N01(rng));
+        for (int j = 0; j < 6; j++) start[j] = lam[j] = (double)(float)(k.lg[j] + noise * N01(rng));
         double xm = k.st.R + 2.0;
         ThreadCounters tc{};
         if (edge) {
@@ -301,7 +324,7 @@ void check_take_back(double RT, double noise, int edge, int trials, unsigned see
         out[0] += 1.0;
         const std::vector<double> made = k.M;
         DFStream ds = k.stream(1.0, kDfPopCap);
-        df_take_back<2>(k.m, k.c, k.tab, lg32, k.conG, k.etab.data(), xm, ds, tc);
+        df_take_back<2>(k.m, k.g, Min.data(), cell, k.tab, start, k.etab.data(), xm, ds, tc);
         for (int i = 8; i < 11; i++) {
             double top = 0.0, left = 0.0;
             for (int j = 0; j < kGrid * kGrid; j++) {

@@ -1229,15 +1229,16 @@ static __device__ __noinline__ bool fp64_hot_cell(const Model& m, const Geometry
 }
 
 // The FP64 path's cell after the collision: EPR from the multipliers lf, lg, and moment streaming, in
-// lattice form where the cell has a row table whose offsets and velocities are exact in FP32
-// (|k|^3 and quarter cells below 2^24).
+// lattice form where the cell has a row table whose offsets are exact in FP32 (|k|^3 below 2^24) and whose
+// displacements fit the 32-bit tally of scatter64 and count_set ((4 |c|)^2 below 2^31 in two dimensions: |u| up
+// to 4096 cells a step and 250 more; quarter cells are exact in FP32 far beyond).
 template <int D>
 __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                           DevStats* stats, const CellPlace& at, BlockCounters& bc,
                                           ThreadCounters& tc, double* conF, double* conG, const CellState<D>& c,
                                           const Stencil<D>& st, const RowTable<D>& tab, double* lf, double* lg,
                                           bool learned, Absorbed& due) {
-    if (tab.ok && st.R <= 250 && abs(tab.xc) < (1 << 21) && abs(tab.yc) < (1 << 21)) {
+    if (tab.ok && st.R <= 250 && abs(tab.xc) < 4096 && abs(tab.yc) < 4096) {
         bool done;
         if (st.R <= kSweepR<D>) {
             done = fp64_lattice_cell<D, false>(m, g, type, Mout, at, bc, tc.pf, tc.pg, tc.ls, conF, conG, c, st, tab, lf,

@@ -530,12 +530,10 @@ extern "C" int lelbm_create(lelbm_t* out, const lelbm_params* p) {
             rc = LELBM_E_NOMEM;
     }
     if (!rc && p->precision == LELBM_MIXED) {
-        // scratch for the threads that can be resident (one 512-thread block an SM); without it the
-        // mixed path evaluates its populations twice
+        // scratch for the threads that can be resident; without it the mixed path evaluates its populations twice
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-        constexpr long long nt = kWideThreads;
-        const long long threads = std::min<long long>(sms * nt, h->ncell + nt);
+        const long long threads = df_pop_threads(D, h->ncell, h->geo.n_inst, sms);
         if (cudaMalloc((void**)&h->d_df_pop, sizeof(float2) * kDfPopCap * (size_t)threads) == cudaSuccess) {
             h->model.df_pop = h->d_df_pop;
             h->model.df_pop_threads = (int)threads;
@@ -826,12 +824,13 @@ extern "C" int lelbm_set_steps(lelbm_t h, const int* steps) {
     return LELBM_OK;
 }
 
+// Blocks of a persistent launch: those that can be resident, and no more than there are tubes.
 static int tuned_blocks(lelbm* h, const lelbm_tuning& t) {
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
     const int mx = batch_persistent_max_blocks_per_sm(h->p.precision, t.threads);
     const int per = (t.blocks_per_sm <= 0 || t.blocks_per_sm > mx) ? mx : t.blocks_per_sm;
-    return sms * per;
+    return std::min(sms * per, std::max(1, h->geo.n_inst));
 }
 
 // Enqueue one persistent launch (work-counter reset + kernel) on the handle's stream.

@@ -42,6 +42,17 @@ constexpr int kWideTubes = 760;  // five an SM
 constexpr int kDfPopCap = 512;
 constexpr int kDfPopR = 12;  // larger sets (2D) are not kept
 
+// Threads that can be resident in a mixed launch of a handle, for the scratch of the kept populations, which a
+// thread indexes by its place in the launch.  The cell update deals ncell cells out in blocks of at most
+// cell_threads (kWideThreads from kWideCells on), one an SM; the persistent batch has at most four blocks of 128
+// threads an SM, each with a tube of its own however short it is.
+inline long long df_pop_threads(int D, long long ncell, int n_inst, int sms) {
+    const long long block = D == 2 && ncell < kWideCells ? cell_threads<PREC_MIXED>() : kWideThreads;
+    const long long cells = ncell + block;
+    const long long used = D == 1 ? (cells > 128LL * n_inst ? cells : 128LL * n_inst) : cells;
+    return used < sms * block ? used : sms * block;
+}
+
 // Physical and numerical constants of one handle (Sec. II, App. C, App. D).
 struct Model {
     double K;           // internal degrees of freedom

@@ -346,4 +346,6 @@ void check_populations(int D, double RT, int trials, unsigned seed, double* out)
         populations<2>(RT, trials, seed, out);
 }
 
+long long check_pop_threads(int D, long long ncell, int n_inst, int sms) { return df_pop_threads(D, ncell, n_inst, sms); }
+
 }

@@ -64,3 +64,25 @@ def test_phonon_take_back(lib, RT, edge):
 def test_lattice_form_populations(lib, D, RT):
     mean, _, mean_rows, _ = call(lib.check_populations, D, RT, 30 if D == 2 else 200, 7, n_out=4)
     assert 0 < mean <= 1.2 * mean_rows + 2.0 ** -52
+
+
+# The scratch of the kept populations has a column for every thread of a mixed launch: a persistent batch of
+# tubes however short (four blocks of 128 threads an SM, no more than tubes) and a cell update of one block an SM.
+@pytest.mark.parametrize("n_inst,per_tube", [(1, 400), (7, 30), (700, 12), (760, 12), (4096, 12), (4096, 3000)])
+def test_scratch_of_kept_populations_1d(lib, n_inst, per_tube, sms=152):
+    f = lib.check_pop_threads
+    f.restype = ctypes.c_longlong
+    ncell = n_inst * per_tube
+    got = f(1, ctypes.c_longlong(ncell), n_inst, sms)
+    batch = min(n_inst, 4 * sms) * 128
+    cells = min(ncell + 384, sms * 384)
+    assert max(batch, min(cells, ncell)) <= got <= sms * 512
+
+
+@pytest.mark.parametrize("ncell", [1, 1000, 60000, 399999, 400000, 1 << 24])
+def test_scratch_of_kept_populations_2d(lib, ncell, sms=152):
+    f = lib.check_pop_threads
+    f.restype = ctypes.c_longlong
+    block = 384 if ncell < 400000 else 512
+    got = f(2, ctypes.c_longlong(ncell), 1, sms)
+    assert min(ncell + block - 1, sms * block) <= got <= sms * block

@@ -1146,9 +1146,15 @@ template <int D>
 static __device__ __noinline__ TailCounts fp64_general_cold(const Model& m, const Geometry& g, const uint8_t* type,
                                                             double* Mout, DevStats* stats, const CellPlace at,
                                                             BlockCounters* bc, double* conF, double* conG,
-                                                            const CellState<D> c, const Stencil<D> st, double* lf,
-                                                            double* lg, bool learned) {
+                                                            const CellState<D> c, const Stencil<D> st,
+                                                            const double* lf_start, const double* lg_start,
+                                                            bool learned) {
     TailCounts t{0, 0, 0, {0, 0.0, 0, 0}};
+    double lf[Dim<D>::NF], lg[Dim<D>::NG];  // copies: through the caller's pointers they would stay in memory
+#pragma unroll
+    for (int j = 0; j < Dim<D>::NF; j++) lf[j] = lf_start[j];
+#pragma unroll
+    for (int j = 0; j < Dim<D>::NG; j++) lg[j] = lg_start[j];
     fp64_tail<D>(m, g, type, Mout, stats, at, *bc, t.pf, t.pg, t.retry, t.ls, conF, conG, c, st, lf, lg, learned);
     return t;
 }

@@ -31,7 +31,7 @@ namespace lbm {
 // ---------------------------------------------------------------------------
 // exp(x) in FP64 with integer instructions: Tang's table-driven method (ACM TOMS 15, 1989) in 64-bit
 // fixed point.  x log2(e) = n + j / 512 + rho, 2^(j/512) from a table, 2^rho from five Taylor terms.
-// Every step carries at least 59 bits, so the result is rounded once (0.6 ulp at most).  About 70
+// Every step carries at least 59 bits, so the result is rounded once (0.62 ulp at most).  About 70
 // integer instructions, some 20 issue cycles of an SM, where the library's exp takes about 17 FP64
 // instructions, 16 cycles each.
 // ---------------------------------------------------------------------------

@@ -348,4 +348,39 @@ void check_populations(int D, double RT, int trials, unsigned seed, double* out)
 
 long long check_pop_threads(int D, long long ncell, int n_inst, int sms) { return df_pop_threads(D, ncell, n_inst, sms); }
 
+// The FP64 arithmetic in integer instructions and short forms, on n random arguments: out = largest error of
+// exp_int in ulps over |x| < 128, of recip64 and of quotient in ulps, then how many of the other results were wrong:
+// narrow (truncation; zero below 2^-126, infinity from 2^128), widen (exact), quarter (exact).
+void check_arithmetic(int n, unsigned seed, double* out) {
+    std::mt19937_64 rng(seed);
+    std::uniform_real_distribution<double> U(-1.0, 1.0);
+    for (int i = 0; i < 6; i++) out[i] = 0.0;
+    auto ulps = [](double got, real exact) {
+        int e;
+        std::frexp((double)exact, &e);
+        return (double)(fabsl(got - exact) / ldexpl(1.0L, e - 53));
+    };
+    const double edge[] = {0.0, -0.0, 1e-300, -1e-300, 1e-17, 0.6931471805599453, -0.6931471805599453, 127.999, -127.999,
+                           0x1p-60, -0x1p-52, 64.0, -64.0};
+    const int n_edge = (int)(sizeof edge / sizeof edge[0]);
+    for (int i = 0; i < n; i++) {
+        const double x = i < n_edge ? edge[i] : (i % 3 ? 128.0 * U(rng) : std::ldexp(U(rng), i % 60 - 56));
+        out[0] = std::max(out[0], ulps(exp_int(x), expl((real)x)));
+        const double b = std::ldexp(1.0 + std::fabs(U(rng)), (int)(rng() % 190) - 95);
+        const double a = std::ldexp(U(rng), (int)(rng() % 40) - 20);
+        const double y = recip64(b);
+        out[1] = std::max(out[1], ulps(y, 1.0L / (real)b));
+        out[2] = std::max(out[2], ulps(quotient(a, b, y), (real)a / (real)b));
+        const double v = std::ldexp(1.0 + std::fabs(U(rng)), (int)(rng() % 300) - 150);
+        const float f = narrow(v);
+        const float want = v < 0x1p-126 ? 0.f : (v >= 0x1p128 ? INFINITY : std::nextafterf((float)v, 0.f));
+        out[3] += v >= 0x1p-126 && v < 0x1p128 ? !((double)f <= v && (f == (float)v || f == want)) : f != want;
+        out[4] += std::isfinite(f) && (widen(f) != (double)f || widen(-f) != -(double)f);
+        const double w = i % 2 ? -v : v;
+        out[5] += quarter(w) != 0.25 * w || quarter(std::ldexp(w, -900)) != 0.25 * std::ldexp(w, -900);
+    }
+    out[4] += widen(0x1p-130f) != 0.0;
+    out[5] += quarter(0.0) != 0.0 || !std::isinf(quarter(INFINITY));
+}
+
 }

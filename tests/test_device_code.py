@@ -86,3 +86,12 @@ def test_scratch_of_kept_populations_2d(lib, ncell, sms=152):
     block = 384 if ncell < 400000 else 512
     got = f(2, ctypes.c_longlong(ncell), 1, sms)
     assert min(ncell + block - 1, sms * block) <= got <= sms * block
+
+
+# The exponential by integer instructions carries at least 59 bits and rounds once: half an ulp, a sixth for the
+# terms left out and cut off.  A reciprocal within one ulp, a quotient too; conversions and quarters exact.
+def test_integer_and_short_arithmetic(lib):
+    e, recip, quot, bad_narrow, bad_widen, bad_quarter = call(lib.check_arithmetic, 400000, 8, n_out=6)
+    assert e <= 2.0 / 3.0
+    assert recip <= 1.0 and quot <= 1.0
+    assert bad_narrow == bad_widen == bad_quarter == 0

@@ -636,10 +636,10 @@ static __device__ __noinline__ void noslip_images(const Model& m, const Geometry
                     double eg = 1.0;
 #pragma unroll
                     for (int j = 0; j < 6; j++) eg += li_g[j] * T[j];
-                    gp = dC * exp(-eg);
+                    gp = dC * exp_int(-eg);
                 }
                 const double cm[2] = {-cp[0], -cp[1]};
-                stream_traced(g, type, Mout, ix, iy, cm, mfs * (dC * exp(-ef)), mgs * gp,
+                stream_traced(g, type, Mout, ix, iy, cm, mfs * (dC * exp_int(-ef)), mgs * gp,
                               pass == 0 ? kStreamImageSum : kStreamImagePut, pass == 0 ? kept : unused, sf, sg, n);
             };
             si.for_each(image);
@@ -885,7 +885,8 @@ __device__ __forceinline__ void scatter64(const Model& m, const Geometry& g, con
 
 // The images of the no-slip walls for the cells of a warp; whole warps call it.  Launched from scatter64, where
 // the lanes leave loops of different lengths, the images (two passes over the velocity set, every path
-// traced) ran lane after lane: 300 x 150 cylinder with a no-slip wall 11.5 ms a step, gathered here 6.6.
+// traced) ran lane after lane: 300 x 150 cylinder with a no-slip wall 11.5 ms a step, gathered here 6.1 (with the
+// images' exponentials as integer code, 6.7 without).
 __device__ __forceinline__ void launch_images(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                               long long cell, const CellState<2>& c, const Stencil<2>& st,
                                               const double* conF, const double* conG, const Absorbed& due) {

@@ -1,9 +1,11 @@
 // Double-float finish of the EPR Newton (Eq. IID7-IID11) for the mixed path
 // (LELBM_MIXED) on the FP32 pipe.  GB300 runs FP64 at 1/64 of the FP32 rate, so the
 // part of the solve that needs more than FP32 precision -- the residual that the
-// 1e-12 tolerance of Sec. II.D judges, and the populations that moment streaming
-// (Eq. IIE3) deposits -- is evaluated in double-float arithmetic: a value is the
-// unevaluated sum h + l of two FP32 numbers (Dekker 1971), about 48 significant bits.
+// 1e-12 tolerance of Sec. II.D judges, and the populations that the correction evaluates --
+// is double-float arithmetic: a value is the unevaluated sum h + l of two FP32 numbers
+// (Dekker 1971), about 48 significant bits.  Moment streaming (Eq. IIE3) deposits those
+// populations with a small FP32 change (df_restream), or evaluates them again, and
+// multiplies out and adds their moments in FP64.
 //
 // Per population and stencil point the work is FP32 and integer only:
 //   - the exponent -(1 + lambda . T(t)) / ln 2 is a polynomial in the lattice offsets
@@ -711,7 +713,7 @@ __device__ __forceinline__ float df_update_size(const float* MJ, const double* r
 // such a judge would not serve, always gets the DF_STREAM pass.
 // What bounds a DF_STREAM pass is FP32 instructions (79 a point for the exponential and the sums, and 250
 // a row to set them up); this pass takes 15 and 25, and a load.  1024^2 mixed step at RT 0.6: 4.28 -> 3.87 ms,
-// at RT 0.35 8.07 -> 7.15 ms, four-quadrant flow 9.58 -> 7.85 ms; 4096 tubes, two steps, 33.0 -> 18.7 ms.
+// at RT 0.35 8.07 -> 7.15 ms, four-quadrant flow 9.58 -> 7.85 ms; 4096 tubes, two steps, 20.9 -> 15.0 ms.
 constexpr float kRestreamMax = 3e-6f, kRestreamErr = 3.f / 16777216.f;
 constexpr double kRestreamTol = 1e-12;
 

@@ -8,6 +8,8 @@
 //     both directions: a row costs about a dozen products where seven exponentials stood, and the
 //     error growth (~n^3/6 ulp over n steps) starts at the centre.
 //   - The children of split points are a lattice of spacing 1/2 of their own, swept the same way.
+//   - Hot cells (R_ac above kSweepR) start every row from its own exponentials instead, seven to ten
+//     of them to 25 points and more, since ratios compounded over so many rows lose too much.
 //   - A Newton pass sums only the residual's moments (degree <= 3 and <= 2) in FP64, as power sums
 //     of the integer offsets (exact weights, made by integer operations) moved to thermal units
 //     once per pass.  The Jacobian and the solve of an update are FP32, from the same populations:

@@ -558,9 +558,6 @@ __device__ __forceinline__ void scatter_cell32(const Model& m, const Geometry& g
     ls.disp_max2 = fmax(ls.disp_max2, (double)dmax);
 }
 
-// Moment streaming, Eq. (IIE3): T_N(c_i) rho f'_i and T_N(c_i) rho K RT g'_i added at
-// x + c_i.  Level-0 points land on one cell; refined points are shared between the
-// cells they overlap (cloud-in-cell).
 // Image populations of the no-slip walls (Sec. III.B, Eq. IIIB10-IIIB15) for a cell whose
 // streaming gave no-slip boundary n (1 at rest, 2 moving at u_w) the mass absorbed[2(n-1)]
 // (f) and the phonon energy absorbed[2(n-1)+1] (g).  The images of boundary n are the EPR
@@ -651,6 +648,9 @@ static __device__ __noinline__ void noslip_images(const Model& m, const Geometry
     }
 }
 
+// Moment streaming, Eq. (IIE3): T_N(c_i) rho f'_i and T_N(c_i) rho K RT g'_i added at
+// x + c_i.  Level-0 points land on one cell; refined points are shared between the
+// cells they overlap (cloud-in-cell).
 template <int D>
 __device__ __forceinline__ void scatter_cell(const Model& m, const Geometry& g, const uint8_t* type, double* Mout,
                                              const CellPlace& at, const CellState<D>& c, const Stencil<D>& st,
@@ -905,7 +905,6 @@ struct BlockCounters {
     unsigned long long cells, feq, fmx, q, dmax, pf, pg, pm, p32, redo, retry, walls, mlpc, pdf, pdfc;
 };
 
-// Per-thread tallies.
 // Per-thread tallies (32-bit: a thread adds them to its block's counters at least once per
 // time step, see counters_to_block).
 struct ThreadCounters {
@@ -923,8 +922,6 @@ __device__ __forceinline__ void counters_init(BlockCounters& bc) {
             bc.walls = bc.mlpc = bc.pdf = bc.pdfc = 0;
 }
 
-// Adds the thread tallies to the block counters, then (after a barrier) the block
-// counters to the device counters.  Every thread of the block must call it.
 // Sum and maximum of the lanes' values.
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     if (!__any_sync(0xffffffffu, v != 0)) return 0;
@@ -971,6 +968,8 @@ static __device__ __noinline__ void counters_to_block(BlockCounters& bc, ThreadC
     tc = ThreadCounters{0, 0, 0, 0, 0, 0, {0, 0.0, 0, 0}, 0, 0, 0};
 }
 
+// Adds the thread tallies to the block counters, then (after a barrier) the block
+// counters to the device counters.  Every thread of the block must call it.
 __device__ __forceinline__ void counters_flush(BlockCounters& bc, ThreadCounters& tc, DevStats* stats) {
     counters_to_block(bc, tc);
     __syncthreads();
@@ -1286,10 +1285,11 @@ static __device__ __noinline__ TailCounts fp64_tail_cold(const Model& m, const G
 // ---------------------------------------------------------------------------
 // The mixed path's finish (LELBM_MIXED): FP32 Newton to the FP32 noise floor, then per
 // population one double-float correction (residual in double-float, Jacobian in FP32 at
-// the same multipliers) and a double-float streaming pass that re-checks the residual of
-// exactly the populations it deposits against the FP64 path's tolerance (Sec. II.D).  A
-// miss takes the deposit back and corrects again; a second miss leaves the cell to the
-// FP64 EPR.
+// the same multipliers) and a streaming pass that re-checks the residual of exactly the
+// populations it deposits against the FP64 path's tolerance (Sec. II.D): from the kept
+// populations of the correction and an FP32 change where that is small (df_restream), else
+// evaluated again in double-float.  A miss takes the deposit back and corrects again; a
+// second miss leaves the cell to the FP64 EPR.
 // ---------------------------------------------------------------------------
 // Corrects and streams one population.  Returns the number of double-float Newton updates
 // (>= 1) once its deposit passed the check, -1 when nothing of it is deposited and the
@@ -1650,14 +1650,6 @@ static __device__ __noinline__ bool fp32_phase(const RowTable<D>& tab_in, const 
     return ok;
 }
 
-// The mixed path's cell update in block-synchronous phases.  The 128 cells a block claims go
-// together through (1) the collision, stencil set-up, warm start and row table, (2) the
-// FP32 Newton, (3) the phonons' and (4) the fluons' double-float correction and streaming,
-// with a block barrier between phases: the warps of a block then run the same code at the
-// same time, which keeps the instruction working set of an SM to a few phases.  Every
-// thread of the block calls this, active or not.
-// INLINE_MLP: the warm-start network runs here, warp-wide (the persistent 1D batch); the
-// cell-update kernel instead reads the corrections mlp_start_kernel wrote (m.mlp_start).
 // Barrier of the threads that step a chunk of cells together: the whole block
 // (nthreads = blockDim.x), or one group of nthreads threads (hardware barrier 1 + group).
 __device__ __forceinline__ void group_sync(int group, int nthreads) {
@@ -1667,6 +1659,14 @@ __device__ __forceinline__ void group_sync(int group, int nthreads) {
         asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(nthreads) : "memory");
 }
 
+// The mixed path's cell update in synchronous phases.  The cells that a group of threads claims (a
+// cell a thread) go together through (1) the collision, stencil set-up, warm start and row table, (2) the
+// FP32 Newton, (3) the phonons' and (4) the fluons' double-float correction and streaming,
+// with a barrier of the group between phases: its warps then run the same code at the
+// same time, which keeps the instruction working set of an SM to a few phases.  Every
+// thread of the group calls this, active or not.
+// INLINE_MLP: the warm-start network runs here, warp-wide (the persistent 1D batch); the
+// cell-update kernel instead reads the corrections mlp_start_kernel wrote (m.mlp_start).
 template <int D, bool INLINE_MLP>
 __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, const uint8_t* type,
                                             const double* __restrict__ Min, double* Mout, DevStats* stats,
@@ -1828,13 +1828,6 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
     }
 }
 
-// One time step of the whole padded grid: warps claim chunks of 32 consecutive cells
-// from a global counter (the cost of a cell varies with its temperature, q ~
-// (n sqrt RT)^D, so a static split leaves SMs idle at the end).
-// Blocks per SM the compiler must fit (registers): the FP32 variants, whose FP64 fallback
-// is out of line and whose per-thread tallies live in shared memory, are light enough in
-// their hot path for four 128-thread blocks (128 registers); the rest keep the full
-// register file.
 // Groups of the mixed path's block that claim and step their cells independently, each
 // with its own phase barriers: fewer warps wait at a barrier for the slowest one, while at
 // most two phases share an SM's instruction caches.  Two groups of six warps measured 4.8 %
@@ -1843,9 +1836,16 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
 // A block of a small grid is one group.
 constexpr int kMixedGroups = 2;
 
+// Blocks per SM the compiler must fit (registers): the FP32 variants, whose FP64 fallback
+// is out of line and whose per-thread tallies live in shared memory, are light enough in
+// their hot path for four 128-thread blocks (128 registers); the rest keep the full
+// register file.
 template <int D, int PREC>
 constexpr int min_blocks() { return PREC == PREC_FP32 ? 4 : (PREC == PREC_MIXED ? 1 : 1); }
 
+// One time step of the whole padded grid: warps claim chunks of 32 consecutive cells (on the mixed
+// path groups of warps, a cell a thread) from a global counter: the cost of a cell varies with its
+// temperature, q ~ (n sqrt RT)^D, so a static split leaves SMs idle at the end.
 // WALLS: a kernel of its own for the FP32 path beside solid cells, so that scatter_near32 costs other grids
 // nothing (with both in one kernel a 128^2 step at RT 16 took 0.97 ms, 0.92 without).
 template <int D, int PREC, int NT, bool WALLS = false>

@@ -1353,11 +1353,8 @@ __device__ __forceinline__ void solve_fg(const CellState<D>& c, const Stencil<D>
 }
 
 // ---------------------------------------------------------------------------
-// Mixed precision: the Newton passes over the velocity set run in FP32 (FP32 is
-// about 60x the FP64 rate on GB300); the small Cholesky solves stay FP64.  The
-// FP32 iterate is then corrected by one full FP64 Newton pass, and the
-// streaming pass checks the FP64 residual of exactly the populations it
-// deposits against the same tolerance as the FP64 path.
+// The FP32 Newton of the FP32 and mixed paths: passes over the velocity set and solves in FP32 (about
+// 60x the FP64 rate on GB300).  The mixed path corrects its result in double-float (lelbm_df.cuh).
 // ---------------------------------------------------------------------------
 // Coefficients of the FP32 exponent polynomials on the row y (as row_coeffs).
 template <int D>

@@ -1294,8 +1294,10 @@ static __device__ __noinline__ TailCounts fp64_tail_cold(const Model& m, const G
 // second miss leaves the cell to the FP64 EPR.
 // ---------------------------------------------------------------------------
 // Corrects and streams one population.  Returns the number of double-float Newton updates
-// (>= 1) once its deposit passed the check, -1 when nothing of it is deposited and the
-// FP64 EPR must solve the cell.
+// (1 or 2) once its deposit passed the check, plus kFromKept if the deposit was made from kept
+// populations; -1 when nothing of it is deposited and the FP64 EPR must solve the cell.
+constexpr int kFromKept = 4;
+
 template <int D, bool FLUON>
 __device__ __forceinline__ int df_population(const Model& m, const CellState<D>& c, const RowTable<D>& tab,
                                              double* lam, const double* con, const float2* etab, double xm,
@@ -1332,7 +1334,8 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
             else if (!df_pass<D, FLUON, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lam, con, etab, xm, r, rmax,
                                                    nullptr, ds, tc.ls, tc.pdf, ds.beta))
                 return -1;
-            if (undo == 0 && rmax + (again ? widen(kRestreamErr * change) : 0.0) <= m.tol) return it + 1;
+            if (undo == 0 && rmax + (again ? widen(kRestreamErr * change) : 0.0) <= m.tol)
+                return it + 1 + (again ? kFromKept : 0);
             // the deposited populations miss the tolerance: take them back
             ds.mh = -ds.mh;
             ds.ml = -ds.ml;
@@ -1342,28 +1345,36 @@ __device__ __forceinline__ int df_population(const Model& m, const CellState<D>&
     return -1;
 }
 
-// Takes back the phonon deposit that df_population made from the multipliers lg_start (the FP64 EPR then
-// streams the cell): the same passes from the same start with the mass negated, so that every addition
-// comes again with the other sign, whichever of the passes made it.  Out of line: it is rare; the
-// collision is recomputed from the cell's moments in Min and lg_start waits in the cell's scratch slots, so
-// that nothing stays live for it (with the cell and lg_start handed over a 4096^2 step took 98.3 ms, 96.9 so).
+// Takes back a phonon deposit that df_population made from kept populations, with `updates` updates from the
+// multipliers lg_start: the last correction pass and the streaming from what it keeps come again with the mass
+// negated, so that every addition comes with the other sign.  Out of line: it is rare; the collision is
+// recomputed from the cell's moments in Min and lg_start waits in the cell's scratch slots, so that
+// nothing stays live for it (with the cell and lg_start handed over a 4096^2 step took 98.3 ms, 96.9 so).
 template <int D>
 static __device__ __noinline__ void df_take_back(const Model& m, const Geometry& g, const double* __restrict__ Min,
                                                  long long cell, const RowTable<D> tab, const double* lg_start,
-                                                 const float2* etab, double xm, const DFStream& ds_in,
+                                                 int updates, const float2* etab, double xm, const DFStream& ds_in,
                                                  ThreadCounters& tc) {
-    double M[Dim<D>::NM], lg[Dim<D>::NG];
+    using Q = DFPop<D, false>;
+    double M[Dim<D>::NM], lg[Q::N], r[Q::N], rmax;
 #pragma unroll
     for (int i = 0; i < Dim<D>::NM; i++) M[i] = Min[i * g.ncell + cell];
     CellState<D> c;
     collide<D>(M, m, c);
 #pragma unroll
-    for (int j = 0; j < Dim<D>::NG; j++) lg[j] = lg_start[j];
+    for (int j = 0; j < Q::N; j++) lg[j] = lg_start[j];
     DFStream ds = ds_in;
     df_split(-(c.rho * m.K * c.RT), ds.mh, ds.ml);
-    const unsigned int redo = tc.redo;
-    df_population<D, false>(m, c, tab, lg, c.cg, etab, xm, ds, tc);
-    tc.redo = redo;  // misses are counted once
+    float dl[Q::N];
+    for (int it = 0; it < updates; it++) {
+        float MJ[Q::NJ];
+        df_pass<D, false, DF_CORR>(c.u[0], c.u[D - 1], c.inv_sig, tab, lg, c.cg, etab, xm, r, rmax, MJ, ds, tc.ls,
+                                   tc.pdfc, ds.beta);
+#pragma unroll
+        for (int j = 0; j < Q::N; j++) dl[j] = 0.f;
+        if (rmax > m.tol) df_update<D, false>(MJ, r, lg, dl);
+    }
+    df_restream<D, false>(tab, dl, r, rmax, ds, tc.ls, tc.pdf);
 }
 
 // The multipliers of a converged FP32 solve minus Eq. (IID13), for the next step, and its counts.
@@ -1806,12 +1817,21 @@ __device__ __forceinline__ void mixed_block(const Model& m, const Geometry& g, c
         uf = df_population<D, true>(m, c, tab, lf, conF, etab, xm, ds, tc);
         if (uf < 0) {
             alive = false;
-            if (has_g) df_take_back<D>(m, g, Min, cell, tab, conG, etab, xm, ds, tc);
+            if (has_g) {  // take the phonon deposit back: the FP64 EPR streams both
+                if (ug & kFromKept) {
+                    df_take_back<D>(m, g, Min, cell, tab, conG, ug & (kFromKept - 1), etab, xm, ds, tc);
+                } else {  // the pass that made it, at the same multipliers (its residual is not used)
+                    double r[NG], rmax;
+                    df_split(-(c.rho * m.K * c.RT), ds.mh, ds.ml);
+                    df_pass<D, false, DF_STREAM>(c.u[0], c.u[D - 1], c.inv_sig, tab, lg, conG, etab, xm, r, rmax,
+                                                 nullptr, ds, tc.ls, tc.pdf, ds.beta);
+                }
+            }
         }
     }
     if (alive) {
-        atomicAdd(&bc.hist[uf], 1ull);
-        if (has_g) atomicAdd(&bc.hist[ug], 1ull);
+        atomicAdd(&bc.hist[uf & (kFromKept - 1)], 1ull);
+        if (has_g) atomicAdd(&bc.hist[ug & (kFromKept - 1)], 1ull);
         if (m.lam_store) {  // the converged multipliers minus Eq. (IID13), as FP32 corrections
             const float l0 = (float)maxwell_l0<D>(c.RT);
 #pragma unroll

@@ -135,12 +135,15 @@ struct Cell {
 };
 
 template <bool FLUON>
-int population(Cell& k, const double* start, double mass, int pop_cap, ThreadCounters& tc, double xm = 0.0) {
+int population(Cell& k, const double* start, double mass, int pop_cap, ThreadCounters& tc, double xm = 0.0,
+               double* solution = nullptr) {
     double lam[10];
     for (int j = 0; j < DFPop<2, FLUON>::N; j++) lam[j] = start[j];
     DFStream ds = k.stream(mass, pop_cap);
-    return df_population<2, FLUON>(k.m, k.c, k.tab, lam, FLUON ? k.conF : k.conG, k.etab.data(),
+    const int u = df_population<2, FLUON>(k.m, k.c, k.tab, lam, FLUON ? k.conF : k.conG, k.etab.data(),
                                    xm > 0.0 ? xm : k.st.R + 2.0, ds, tc);
+    for (int j = 0; solution && j < DFPop<2, FLUON>::N; j++) solution[j] = lam[j];
+    return u;
 }
 
 template <bool FLUON>
@@ -320,11 +323,19 @@ void check_take_back(double RT, double noise, int edge, int trials, unsigned see
         }
         const double mass = k.c.rho * k.m.K * k.c.RT;
         std::fill(k.M.begin(), k.M.end(), 0.0);
-        if (population<false>(k, start, mass, kDfPopCap, tc, xm) < 0) continue;
+        const int u = population<false>(k, start, mass, kDfPopCap, tc, xm, lam);
+        if (u < 0) continue;
         out[0] += 1.0;
         const std::vector<double> made = k.M;
         DFStream ds = k.stream(1.0, kDfPopCap);
-        df_take_back<2>(k.m, k.g, Min.data(), cell, k.tab, start, k.etab.data(), xm, ds, tc);
+        if (u & kFromKept) {
+            df_take_back<2>(k.m, k.g, Min.data(), cell, k.tab, start, u & (kFromKept - 1), k.etab.data(), xm, ds, tc);
+        } else {  // as mixed_block
+            double r[6], rmax;
+            df_split(-mass, ds.mh, ds.ml);
+            df_pass<2, false, DF_STREAM>(k.c.u[0], k.c.u[1], k.c.inv_sig, k.tab, lam, k.conG, k.etab.data(), xm, r, rmax,
+                                         nullptr, ds, tc.ls, tc.pdf, k.beta);
+        }
         for (int i = 8; i < 11; i++) {
             double top = 0.0, left = 0.0;
             for (int j = 0; j < kGrid * kGrid; j++) {

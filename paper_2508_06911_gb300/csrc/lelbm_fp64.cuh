@@ -116,10 +116,12 @@ __device__ __forceinline__ void lattice_poly(const double* lam, double x0, doubl
 template <int D, bool FLUON>
 struct SweepFactors {
     double e0, r, l, r2, r3, l3;            // population, ratios to k = +1 and -1, second and third ratios
+    double el, l2;                          // 1D, apart: population at k = -1 and second ratio there (l from there)
     double u, ud, u2, u2d, u3, u3d;         // ratios of e0 to the rows j = +1 and -1, second, third
     double m11, i11, m12, i12, m21, i21;    // exp(-+p_11), exp(-+p_12), exp(-+p_21)
 
-    __device__ __forceinline__ void init(const double* p, double wgt) {
+    // apart (1D): the left side starts from exponentials of its own, at k = -1
+    __device__ __forceinline__ void init(const double* p, double wgt, bool apart) {
         using Q = DFPop<D, FLUON>;
         constexpr int NE = FLUON ? (D == 1 ? 6 : 17) : (D == 1 ? 4 : 9);
         double a[NE];
@@ -127,7 +129,7 @@ struct SweepFactors {
         const double p30 = FLUON ? p[FLUON ? Q::ix(3, 0) : 0] : 0.0;
         a[0] = p[0];
         a[1] = p10 + p20 + p30;
-        a[2] = p20 - p10 - p30;
+        a[2] = D == 1 && apart ? 3.0 * p20 - p10 - 7.0 * p30 : p20 - p10 - p30;
         a[3] = 2.0 * p20 + 6.0 * p30;
         if constexpr (FLUON) {
             a[4] = 6.0 * p30;
@@ -162,6 +164,10 @@ struct SweepFactors {
         if constexpr (FLUON) {
             r3 = a[4];
             l3 = a[5];
+        }
+        if (D == 1 && apart) {
+            el = wgt * exp_int(p10 - p20 + p30 - p[0]);
+            if constexpr (FLUON) l2 = exp_int(12.0 * p30 - 2.0 * p20);
         }
         if constexpr (D == 2) {
             constexpr int o = FLUON ? 6 : 4;
@@ -230,14 +236,18 @@ struct SweepRows {
 // compounded rounding of tall sets; up to R_ac = 7 (RT = 3.5 at n = 4) one anchor serves all.
 constexpr int kAnchorRows = 8;
 
-// Acoustic radius up to which the sweeps compound along y too.  The mean error of a population (weighted by
-// it, against 64 bits; the general stencil, whose rows each start afresh, in brackets): 2D, RT 0.6 1.6e-16
+// Acoustic radius up to which 2D sweeps compound along y too.  The mean error of a population (weighted by
+// it, against 64 bits; the general stencil, whose rows each start afresh, in brackets): RT 0.6 1.6e-16
 // (1.3e-15), RT 9.4 1.3e-15 (1.5e-15), but with sweeps RT 10 1.3e-15 (1.0e-15), RT 16 2.2e-15 (6.6e-16)
 // and RT 32 5.0e-15 (1.0e-15).  Beyond, rows that start afresh in the lattice form: RT 10 4.9e-16, RT 16
-// 6.2e-16, RT 32 1.0e-15.  1D: RT 8 2.7e-16 (6.2e-15), RT 9.4 3.6e-16 and afresh 2.7e-16 (3.3e-16).  Time of a
-// step: 128^2 at RT 16 4.8 -> 5.5 ms (13.1 on the general stencil), 64^2 at RT 32 8.2 -> 7.7 ms (17.6).
-template <int D>
-constexpr int kSweepR = D == 1 ? 11 : 12;
+// 6.2e-16, RT 32 1.0e-15.  Time of a step: 128^2 at RT 16 4.8 -> 5.5 ms (13.1 on the general stencil),
+// 64^2 at RT 32 8.2 -> 7.7 ms (17.6).
+constexpr int kSweepR = 12;
+
+// In 1D the left side of a row longer than this starts from exponentials of its own: RT 16 4.4e-16 (4.8e-16),
+// RT 150 9.4e-15 (9.4e-15), where from the centre's it lost a third more.  On every row they would cost
+// a 400-cell tube 6 % (the chain of a cell is what its step waits for).
+constexpr int kSweepLeft = 11;
 
 // The populations of one side of a row, from its point at thermal x outwards in steps of h (signed): with its
 // own exponentials, but for the last ratio, which is the same on every row.
@@ -301,6 +311,12 @@ __device__ __forceinline__ void lattice_sweep(const double* lf, const double* lg
         }
         return;
     }
+    bool apart = false;
+    if constexpr (D == 1) {
+        int i0, i1, h0, h1;
+        ext(0, i0, i1, h0, h1);
+        apart = i0 < -kSweepLeft;
+    }
     int ja = 0;
     while (ja - kAnchorRows > jlo) ja -= 2 * kAnchorRows + 1;
 #pragma unroll 1
@@ -310,12 +326,12 @@ __device__ __forceinline__ void lattice_sweep(const double* lf, const double* lg
         if (doF) {
             double p[DFPop<D, true>::NB];
             lattice_poly<D, true>(lf, x0, fma(widen((float)ja), h, y0), h, p);
-            ff.init(p, wf);
+            ff.init(p, wf, apart);
         }
         if (doG) {
             double p[DFPop<D, false>::NB];
             lattice_poly<D, false>(lg, x0, fma(widen((float)ja), h, y0), h, p);
-            fg.init(p, wg);
+            fg.init(p, wg, apart);
         }
         const double l3sq = doF ? ff.l3 * ff.l3 : 0.0;
 #pragma unroll 1
@@ -335,18 +351,18 @@ __device__ __forceinline__ void lattice_sweep(const double* lf, const double* lg
                     for (int left = 0; left < 2; left++) {
                         double e = 0.0, r = 0.0, r2 = 0.0, r3 = 0.0, eg = 0.0, rg = 0.0;
                         if (doF) {
-                            e = sf.E;
+                            e = apart && left ? ff.el : sf.E;
                             r = left ? sf.L : sf.R;
-                            r2 = left ? sf.R2 * l3sq : sf.R2;
+                            r2 = !left ? sf.R2 : (apart ? ff.l2 : sf.R2 * l3sq);
                             r3 = left ? ff.l3 : ff.r3;
                         }
                         if (doG) {
-                            eg = sg.E;
+                            eg = apart && left ? fg.el : sg.E;
                             rg = left ? sg.L : sg.R;
                         }
                         const int n = left ? -i0 : i1;
 #pragma unroll 1
-                        for (int i = 0; i <= n; i++) {
+                        for (int i = apart ? left : 0; i <= n; i++) {
                             const int k = left ? -i : i;
                             if (!(left && i == 0) && k >= i0 && k <= i1 && (k < h0 || k > h1)) point(k, j, e, eg);
                             if (doF) {

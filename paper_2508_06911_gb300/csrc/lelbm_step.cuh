@@ -1248,7 +1248,7 @@ __device__ __forceinline__ void fp64_cell(const Model& m, const Geometry& g, con
                                           bool learned, Absorbed& due) {
     if (tab.ok && st.R <= 250 && abs(tab.xc) < 4096 && abs(tab.yc) < 4096) {
         bool done;
-        if (st.R <= kSweepR<D>) {
+        if (D == 1 || st.R <= kSweepR) {
             done = fp64_lattice_cell<D, false>(m, g, type, Mout, at, bc, tc.pf, tc.pg, tc.ls, conF, conG, c, st, tab, lf,
                                                lg, due);
         } else {

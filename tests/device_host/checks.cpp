@@ -246,7 +246,7 @@ void populations(double RT, int trials, unsigned seed, double* out) {
             auto ext = [&](int j, int& i0, int& i1, int& h0, int& h1) { lat.ext(tab, child, j, i0, i1, h0, h1); };
             int jlo, jhi;
             lat.rows(tab, child, jlo, jhi);
-            if (st.R <= kSweepR<D>)
+            if (D == 1 || st.R <= kSweepR)
                 lattice_sweep<D, false>(lf, lg, true, true, -ox * hs, -oy * hs, hs, 1.0, 1.0, jlo, jhi, ext, point,
                                         row_end);
             else
